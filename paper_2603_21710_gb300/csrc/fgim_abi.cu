@@ -1609,7 +1609,7 @@ fgim_status fgim_autotune(const fgim_shard* shards, int32_t h, const fgim_params
         ck(cudaEventCreate(&e0));
         ck(cudaEventCreate(&e1));
         const int ht0 = ht_bits_for(L);
-        BeamShape best = {4, ht0};
+        BeamShape best = {beam_warps(P.d), ht0};
         float best_ms = -1.f;
         bool had = false;
         BeamShape before = best;
@@ -1622,10 +1622,10 @@ fgim_status fgim_autotune(const fgim_shard* shards, int32_t h, const fgim_params
             }
         }
         const int wpbs[3] = {1, 2, 4};
-        for (int wi = 0; wi < 3; ++wi)
+        for (int wi = P.d <= 128 ? 1 : 0; wi < 3; ++wi)   // resident blocks (beam_grid) gain nothing from one warp each
             for (int dh = -2; dh <= 1; ++dh) {
                 const BeamShape cand = {wpbs[wi], std::min(13, std::max(6, ht0 + dh))};
-                if ((size_t)warp_layout(P.d, L, cand.htbits, params->k, !bytes).bytes * cand.wpb > 227 * 1024) continue;
+                if ((size_t)warp_layout(P.d, L, cand.htbits, params->k, P.d > 128).bytes * cand.wpb > 227 * 1024) continue;
                 {
                     std::lock_guard<std::mutex> lk(g_tune_mu);
                     g_tuned[key] = cand;

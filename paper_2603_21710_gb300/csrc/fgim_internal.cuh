@@ -14,8 +14,8 @@
 // product gives 1 - sum, cosine 1 - sum * (inv_a * inv_b). Every step is a single
 // rounded operation whose operands are symmetric in a and b, so delta(a, b) equals
 // delta(b, a) bit for bit, and the same (id, distance) pair always yields the same key.
-// Warps compute it one row at a time (butterfly) or 32 rows at a time (transpose
-// reduction, which forms exactly the same sums).
+// Warps compute it one row at a time (butterfly) or several rows at a time, eight lanes per row or
+// the rows' partials exchanged together (the same sums, added in the same tree).
 #pragma once
 
 #include <cstdint>
@@ -205,41 +205,6 @@ __device__ __forceinline__ float warp_butterfly(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
-}
-
-// v[r] = this lane's partial of row r (r < 32). Returns the butterfly sum of row `lane`:
-// at offset o each lane keeps the half of its rows whose bit o matches its own lane bit
-// and adds its partner's partials of those rows, forming the butterfly's sums.
-__device__ __forceinline__ float warp_transpose_reduce(float (&v)[32], int lane) {
-#pragma unroll
-    for (int o = 16, n = 16; o > 0; o >>= 1, n >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int r = 0; r < 16; ++r) {
-            if (r < n) {
-                const float send = up ? v[r] : v[r + n];
-                const float keep = up ? v[r + n] : v[r];
-                const float recv = __shfl_xor_sync(0xffffffffu, send, o);
-                v[r] = __fadd_rn(keep, recv);
-            }
-        }
-    }
-    return v[0];
-}
-
-// P[l * 33 + r] = lane l's partial of row r. Returns the butterfly sum of row r, added in the
-// butterfly's tree (pairs of lanes 16 apart, then 8, 4, 2, 1; every pair sum is commutative).
-__device__ __forceinline__ float smem_tree_sum(const float* P, int r) {
-    float a[16];
-#pragma unroll
-    for (int l = 0; l < 16; ++l) a[l] = __fadd_rn(P[l * 33 + r], P[(l + 16) * 33 + r]);
-#pragma unroll
-    for (int l = 0; l < 8; ++l) a[l] = __fadd_rn(a[l], a[l + 8]);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) a[l] = __fadd_rn(a[l], a[l + 4]);
-#pragma unroll
-    for (int l = 0; l < 2; ++l) a[l] = __fadd_rn(a[l], a[l + 2]);
-    return __fadd_rn(a[0], a[1]);
 }
 
 // Non-canonical FP32 distance by one thread: sequential over the chunks with four

@@ -1,12 +1,11 @@
 // Alg. 1 (KNNSearch) on the GPU, shared by the cross query of Alg. 2 (k_cross.cu) and the
 // evaluation / reachability searches (k_search.cu).
 //
-// One warp runs one beam search. The pool C (<= L keys, sorted by (delta, id)) and its
-// "expanded" marks live in shared memory; each expansion reads the expanded vertex's
-// adjacency row (one id per lane), drops ids already evaluated, compacts the rest, loads
-// their rows coalesced (each warp load covers one row, eight rows in flight), forms the
-// canonical distances of up to 32 rows with one transpose reduction, and merges them
-// into the pool with warp_merge.
+// One warp runs one beam search. The pool C (<= L keys, sorted by (delta, id)) lives in registers
+// with a copy in shared memory; each expansion reads the expanded vertex's adjacency row (one id
+// per lane), drops ids already evaluated, compacts the rest, loads their rows coalesced (eight
+// lanes per row up to 128 coordinates), forms the canonical distances of up to 32 rows and merges
+// those that beat the pool's worst entry into the pool all at once.
 //
 // Evaluated ids are remembered in a small direct-mapped table that may forget an id
 // when another id lands on its slot (never the reverse). A forgotten id is evaluated
@@ -28,11 +27,43 @@
 
 namespace fgim {
 
-__device__ __forceinline__ int ht_slot(int v, int bits) { return (int)(((uint32_t)v * 2654435761u) >> (32 - bits)); }
+// The table of evaluated ids: 2^htbits slots of 16 bits. A local id is multiplied by an odd constant
+// modulo 2^b (b = the bits of a local id, at least htbits), which is a bijection; the product's top
+// htbits bits are the slot and the rest is the tag kept there, so a slot names one id exactly. Ids whose
+// tag needs more than 16 bits (graphs above 2^(htbits + 16) vertices) are not remembered, which is
+// always allowed.
+constexpr uint16_t kNoTag = 0xffffu;
+struct VisitedHash {
+    uint32_t mask;    // 2^b - 1
+    uint32_t tmask;   // the tag's bits
+    int sh;           // b - htbits
+    __device__ __forceinline__ VisitedHash(int nt, int htbits) {
+        const int b = max(nt > 1 ? 32 - __clz(nt - 1) : 1, htbits);
+        mask = b >= 32 ? 0xffffffffu : (1u << b) - 1u;
+        sh = b - htbits;
+        tmask = (1u << sh) - 1u;
+    }
+    // true when v is in the table (it is after the call, if its tag fits)
+    __device__ __forceinline__ bool seen(uint16_t* ht, int v) const {
+        const uint32_t x = ((uint32_t)v * 2654435761u) & mask;
+        const uint32_t tag = x & tmask;
+        uint16_t* p = ht + (x >> sh);
+        if (tag >= kNoTag) return false;
+        if (*p == (uint16_t)tag) return true;
+        *p = (uint16_t)tag;
+        return false;
+    }
+    __device__ __forceinline__ void add(uint16_t* ht, int v) const { seen(ht, v); }
+};
 
-struct WarpCounters {
-    long long ndc = 0;
-    long long hops = 0;
+__device__ __forceinline__ void ht_clear(uint16_t* ht, int htbits, int lane) {
+    uint4* p = reinterpret_cast<uint4*>(ht);
+    for (int i = lane; i < (1 << htbits) / 8; i += 32) p[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+}
+
+struct WarpCounters {   // the same in every lane
+    unsigned long long ndc = 0;
+    unsigned long long hops = 0;
 };
 
 __device__ __forceinline__ float4 u8x4_to_float4(uint32_t w) {
@@ -51,69 +82,89 @@ __device__ __forceinline__ float4 row_chunk(const uint8_t* row, int c) {
     return u8x4_to_float4(*reinterpret_cast<const uint32_t*>(row + 4 * c));
 }
 
-// lane_part over a row of either storage (the same additions as lane_part)
-template <int METRIC, typename RT>
-__device__ __forceinline__ float lane_part_rows(const float* q, const RT* row, int nc4, int lane) {
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-    for (int c = lane; c < nc4; c += 32) {
-        const float4 x = reinterpret_cast<const float4*>(q)[c];
-        const float4 y = row_chunk(row, c);
-        if (METRIC == FGIM_L2SQ) {
-            const float e0 = __fsub_rn(x.x, y.x), e1 = __fsub_rn(x.y, y.y);
-            const float e2 = __fsub_rn(x.z, y.z), e3 = __fsub_rn(x.w, y.w);
-            s0 = fmaf(e0, e0, s0);
-            s1 = fmaf(e1, e1, s1);
-            s2 = fmaf(e2, e2, s2);
-            s3 = fmaf(e3, e3, s3);
-        } else {
-            s0 = fmaf(x.x, y.x, s0);
-            s1 = fmaf(x.y, y.y, s1);
-            s2 = fmaf(x.z, y.z, s2);
-            s3 = fmaf(x.w, y.w, s3);
-        }
-    }
-    return __fadd_rn(__fadd_rn(s0, s1), __fadd_rn(s2, s3));
-}
-
-// The query as bytes for byte rows: this lane's 16 bytes (chunk lane % lanes-per-row) and
-// the sum of the squared coordinates.
-struct QBytes {
+// The query as the warp's lanes hold it. Byte rows: this lane's 16 bytes (chunk lane %
+// lanes-per-row) and the sum of the squared coordinates. FP32 rows up to 128 coordinates: the
+// lane's float4 chunks p, p + 8, p + 16, p + 24 (p = lane % 8; zero past the row). Wider rows: the
+// whole query in shared memory.
+struct Query {
     uint4 w;
     uint32_t q2;
+    float4 c[4];
+    const float* q;
 };
 
-__device__ __forceinline__ uint32_t pack4(const float* v) {
-    return __float2uint_rn(v[0]) | (__float2uint_rn(v[1]) << 8) | (__float2uint_rn(v[2]) << 16) |
-           (__float2uint_rn(v[3]) << 24);
+__device__ __forceinline__ uint32_t pack4(const float4 v) {
+    return __float2uint_rn(v.x) | (__float2uint_rn(v.y) << 8) | (__float2uint_rn(v.z) << 16) |
+           (__float2uint_rn(v.w) << 24);
 }
 
-__device__ __forceinline__ QBytes query_bytes(const float* q, int d, int lane) {
-    QBytes b;
-    const int lpr = byte_lanes(d);
-    const int part = lane & (lpr - 1);
-    b.w = make_uint4(0u, 0u, 0u, 0u);
-    if (part < (d >> 4)) {
-        const float* c = q + 16 * part;
-        b.w = make_uint4(pack4(c), pack4(c + 4), pack4(c + 8), pack4(c + 12));
+// src: the query's FP32 row in global memory; qs: d floats of this warp's shared memory (wide rows)
+template <bool SMALLD, typename RT>
+__device__ __forceinline__ Query load_query(const float* __restrict__ src, float* qs, int d, int lane) {
+    Query Q;
+    const float4* s4 = reinterpret_cast<const float4*>(src);
+    if constexpr (sizeof(RT) == 1) {
+        const int lsh = byte_lanes_log2(d);
+        const int part = lane & ((1 << lsh) - 1);
+        Q.w = make_uint4(0u, 0u, 0u, 0u);
+        if (part < (d >> 4)) {
+            const float4* c = s4 + 4 * part;
+            Q.w = make_uint4(pack4(c[0]), pack4(c[1]), pack4(c[2]), pack4(c[3]));
+        }
+        uint32_t s = __dp4a(Q.w.x, Q.w.x, 0u);
+        s = __dp4a(Q.w.y, Q.w.y, s);
+        s = __dp4a(Q.w.z, Q.w.z, s);
+        s = __dp4a(Q.w.w, Q.w.w, s);
+        Q.q2 = row_group_sum(s, lsh);   // integers: exact in any order
+    } else if constexpr (SMALLD) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int c = (lane & 7) + 8 * i;
+            Q.c[i] = c < (d >> 2) ? s4[c] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    } else {
+        float4* q4 = reinterpret_cast<float4*>(qs);
+        for (int c = lane; c < (d >> 2); c += 32) q4[c] = s4[c];
+        Q.q = qs;
+        __syncwarp();
     }
-    uint32_t s = 0;
-    for (int c = lane; c < d; c += 32) s += __float2uint_rn(q[c]) * __float2uint_rn(q[c]);
-    b.q2 = __reduce_add_sync(kFull, s);
-    return b;
+    return Q;
 }
 
-// Canonical distances between the query (q in shared memory; qreg = this lane's chunk when
-// d <= 128) and the U <= 32 rows base[rid[r]]; lane r receives row r's distance.
-// FP32 rows load coalesced (one warp load per row, eight rows in flight); every lane stores
-// its partials in P (32 x 33 floats of this warp's shared memory) and lane r re-adds row r
-// in tree order.
+// The sums of four partials per lane over the eight lanes of a row (offsets 4, 2, 1, the last
+// three levels of the butterfly), all four together: each exchange step halves the values a lane
+// keeps, so lane p of row group s ends with the total of partial p / 2. Lane r then takes the total of
+// row r when r is in [r0, r0 + 16): partial (r - r0) / 4, group r % 4 (r0 a multiple of 16). The additions
+// are the butterfly's (each is commutative), so FP32 totals are the canonical ones.
+template <typename T, typename ADD>
+__device__ __forceinline__ T take_row_totals(const T (&v)[4], int r0, T mine, int lane, ADD add) {
+    const bool b2 = (lane & 4) != 0, b1 = (lane & 2) != 0;
+    const T h0 = add(b2 ? v[2] : v[0], __shfl_xor_sync(kFull, b2 ? v[0] : v[2], 4));
+    const T h1 = add(b2 ? v[3] : v[1], __shfl_xor_sync(kFull, b2 ? v[1] : v[3], 4));
+    T x = add(b1 ? h1 : h0, __shfl_xor_sync(kFull, b1 ? h0 : h1, 2));
+    x = add(x, __shfl_xor_sync(kFull, x, 1));
+    const T got = __shfl_sync(kFull, x, 8 * (lane & 3) + 2 * ((lane >> 2) & 3));
+    return (lane & 16) == r0 ? got : mine;
+}
+
+// Canonical distance sums between the query and the U <= 32 rows base[rid[r]]; lane r receives row r's.
+// FP32 rows up to 128 coordinates: eight lanes per row, four rows per warp load, eight loads in
+// flight. Lane p adds the partials of chunks p, p + 16 and p + 8, p + 24 (the butterfly's offsets 16
+// and 8) by itself and the eight lanes' sums go through its last three levels four rows at a time. (One
+// row per warp load with the 32 x 32 partials re-added through 4 KB of shared memory, the earlier form,
+// took a third more instructions per row and halved the warps that fit on an SM.)
+// Wider rows: eight rows at a time, one lane per chunk, two chunks of every row (16 loads) in
+// flight; the eight rows' partials go through the butterfly together. The kernels are compiled for fewer
+// resident warps here (16 per SM in the cross query, 12 in k_search): the gather is bound by L2 and DRAM
+// latency, and loads in flight count for more than warps. Measured (d = 768 BF16, 120k): cross query
+// 13.9 ms with 8 loads and 20 warps, 12.5 ms so; k_search 1.51 and 0.89 ms.
 // Byte rows (d <= 128, d % 16 == 0): every partial sum of the canonical FP32 value is then an
 // integer below 128 * 255^2 < 2^24, so it is exact and the canonical value is the exact
 // integer result. Lanes take 16 bytes each (32 / lanes-per-row rows per warp load) and form
 // |q|^2 + |x|^2 - 2 q.x with four-way byte dot products, summed over the row's lanes.
 template <int METRIC, bool SMALLD, typename RT>
-__device__ __forceinline__ float rows_delta(const RT* __restrict__ base, const int32_t* rid, int U, const float* q,
-                                            float4 qreg, const QBytes& qb, int d, int lane, float* P) {
+__device__ __forceinline__ float rows_delta(const RT* __restrict__ base, const int32_t* rid, int U, const Query& Q,
+                                            int d, int lane) {
     const int nc4 = d >> 2;
     if constexpr (sizeof(RT) == 1) {
         const int lpr = byte_lanes(d);
@@ -134,10 +185,10 @@ __device__ __forceinline__ float rows_delta(const RT* __restrict__ base, const i
             uint32_t sv[4];
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
-                uint32_t sq = __dp4a(qb.w.x, w[t].x, 0u);
-                sq = __dp4a(qb.w.y, w[t].y, sq);
-                sq = __dp4a(qb.w.z, w[t].z, sq);
-                sq = __dp4a(qb.w.w, w[t].w, sq);
+                uint32_t sq = __dp4a(Q.w.x, w[t].x, 0u);
+                sq = __dp4a(Q.w.y, w[t].y, sq);
+                sq = __dp4a(Q.w.z, w[t].z, sq);
+                sq = __dp4a(Q.w.w, w[t].w, sq);
                 if (METRIC == FGIM_L2SQ) {
                     uint32_t sx = __dp4a(w[t].x, w[t].x, 0u);
                     sx = __dp4a(w[t].y, w[t].y, sx);
@@ -148,23 +199,8 @@ __device__ __forceinline__ float rows_delta(const RT* __restrict__ base, const i
                     sv[t] = sq;
                 }
             }
-            if (lsh == 3) {
-                // eight lanes per row: the four loads' partials are summed over the eight lanes
-                // together (each exchange step halves the values a lane keeps), so lane part p of
-                // row group s ends with the total of load p / 2, row 4 (p / 2) + s of the batch;
-                // unsigned additions in any order give the same (exact) totals
-                const int p = lane & 7;
-                const bool b2 = (p & 4) != 0, b1 = (p & 2) != 0;
-                const uint32_t keep0 = b2 ? sv[2] : sv[0], keep1 = b2 ? sv[3] : sv[1];
-                const uint32_t send0 = b2 ? sv[0] : sv[2], send1 = b2 ? sv[1] : sv[3];
-                const uint32_t h0 = keep0 + __shfl_xor_sync(kFull, send0, 4);
-                const uint32_t h1 = keep1 + __shfl_xor_sync(kFull, send1, 4);
-                uint32_t x = (b1 ? h1 : h0) + __shfl_xor_sync(kFull, b1 ? h0 : h1, 2);
-                x += __shfl_xor_sync(kFull, x, 1);
-                // lane r of the batch (rows 4 t0 .. 4 t0 + 15) takes row r: load r / 4 - t0, group r % 4
-                const int tn = (lane >> 2) - t0;
-                const uint32_t got = __shfl_sync(kFull, x, 8 * (lane & 3) + 2 * (tn & 3));
-                if (tn >= 0 && tn < 4) mine = got;
+            if (lsh == 3) {   // eight lanes per row: t0 is 0 or 4, the batch holds rows 4 t0 .. 4 t0 + 15
+                mine = take_row_totals(sv, 4 * t0, mine, lane, [](uint32_t a, uint32_t b) { return a + b; });
             } else {
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
@@ -176,156 +212,177 @@ __device__ __forceinline__ float rows_delta(const RT* __restrict__ base, const i
                 }
             }
         }
-        if (METRIC == FGIM_L2SQ) mine += qb.q2;
+        if (METRIC == FGIM_L2SQ) mine += Q.q2;
         return lane < U ? (float)mine : 0.f;
-    } else {
-        if (SMALLD) {
-            const bool has = lane < nc4;
-            for (int b = 0; b < U; b += 8) {
-                float4 y[8];
+    } else if constexpr (SMALLD) {
+        const int part = lane & 7, sub = lane >> 3;
+        float mine = 0.f;
+        for (int r0 = 0; r0 < U; r0 += 16) {
+            float sv[4];
 #pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    const int r = b + t;
-                    y[t] = (r < U && has) ? row_chunk(base + (long long)rid[r] * d, lane)
-                                          : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
+            for (int hf = 0; hf < 2; ++hf) {
+                float4 y[2][4];
 #pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    const int r = b + t;
-                    if (r < U) P[lane * 33 + r] = has ? chunk_part<METRIC>(qreg, y[t]) : 0.f;
-                }
-            }
-        } else {
-            // wide rows: eight rows at a time, chunk by chunk (eight loads in flight per lane);
-            // each row keeps the four accumulators and the chunk order of lane_part_rows
-            for (int b = 0; b < U; b += 8) {
-                const RT* rowp[8];
+                for (int t = 0; t < 2; ++t) {
+                    const int r = r0 + 8 * hf + 4 * t + sub;
+                    const bool ok = r < U;
+                    const RT* row = base + (long long)(ok ? rid[r] : 0) * d;
 #pragma unroll
-                for (int t = 0; t < 8; ++t) rowp[t] = base + (long long)rid[b + t < U ? b + t : b] * d;
-                float acc[8][4];
-#pragma unroll
-                for (int t = 0; t < 8; ++t) acc[t][0] = acc[t][1] = acc[t][2] = acc[t][3] = 0.f;
-                for (int c = lane; c < nc4; c += 32) {
-                    const float4 x = reinterpret_cast<const float4*>(q)[c];
-                    float4 y[8];
-#pragma unroll
-                    for (int t = 0; t < 8; ++t)
-                        y[t] = b + t < U ? row_chunk(rowp[t], c) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                    for (int t = 0; t < 8; ++t) {
-                        if (METRIC == FGIM_L2SQ) {
-                            const float e0 = __fsub_rn(x.x, y[t].x), e1 = __fsub_rn(x.y, y[t].y);
-                            const float e2 = __fsub_rn(x.z, y[t].z), e3 = __fsub_rn(x.w, y[t].w);
-                            acc[t][0] = fmaf(e0, e0, acc[t][0]);
-                            acc[t][1] = fmaf(e1, e1, acc[t][1]);
-                            acc[t][2] = fmaf(e2, e2, acc[t][2]);
-                            acc[t][3] = fmaf(e3, e3, acc[t][3]);
-                        } else {
-                            acc[t][0] = fmaf(x.x, y[t].x, acc[t][0]);
-                            acc[t][1] = fmaf(x.y, y[t].y, acc[t][1]);
-                            acc[t][2] = fmaf(x.z, y[t].z, acc[t][2]);
-                            acc[t][3] = fmaf(x.w, y[t].w, acc[t][3]);
-                        }
+                    for (int i = 0; i < 4; ++i) {
+                        y[t][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (ok && part + 8 * i < nc4) y[t][i] = row_chunk(row, part + 8 * i);
                     }
                 }
 #pragma unroll
-                for (int t = 0; t < 8; ++t)
-                    if (b + t < U)
-                        P[lane * 33 + b + t] = __fadd_rn(__fadd_rn(acc[t][0], acc[t][1]), __fadd_rn(acc[t][2], acc[t][3]));
+                for (int t = 0; t < 2; ++t) {
+                    float pt[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) pt[i] = chunk_part<METRIC>(Q.c[i], y[t][i]);
+                    sv[2 * hf + t] = __fadd_rn(__fadd_rn(pt[0], pt[2]), __fadd_rn(pt[1], pt[3]));
+                }
             }
+            mine = take_row_totals(sv, r0, mine, lane, [](float a, float b) { return __fadd_rn(a, b); });
         }
-        __syncwarp();
-        const float s = lane < U ? smem_tree_sum(P, lane) : 0.f;
-        __syncwarp();
-        return s;
+        return mine;
+    } else {
+        // each row keeps four accumulators per lane, in the chunk order of lane_part
+        float mine = 0.f;
+        for (int b = 0; b < U; b += 8) {
+            const RT* rowp[8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) rowp[t] = base + (long long)rid[b + t < U ? b + t : b] * d;
+            float acc[8][4];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) acc[t][0] = acc[t][1] = acc[t][2] = acc[t][3] = 0.f;
+#pragma unroll 2
+            for (int c = lane; c < nc4; c += 32) {
+                const float4 x = reinterpret_cast<const float4*>(Q.q)[c];
+                float4 y[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t)
+                    y[t] = b + t < U ? row_chunk(rowp[t], c) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    if (METRIC == FGIM_L2SQ) {
+                        const float e0 = __fsub_rn(x.x, y[t].x), e1 = __fsub_rn(x.y, y[t].y);
+                        const float e2 = __fsub_rn(x.z, y[t].z), e3 = __fsub_rn(x.w, y[t].w);
+                        acc[t][0] = fmaf(e0, e0, acc[t][0]);
+                        acc[t][1] = fmaf(e1, e1, acc[t][1]);
+                        acc[t][2] = fmaf(e2, e2, acc[t][2]);
+                        acc[t][3] = fmaf(e3, e3, acc[t][3]);
+                    } else {
+                        acc[t][0] = fmaf(x.x, y[t].x, acc[t][0]);
+                        acc[t][1] = fmaf(x.y, y[t].y, acc[t][1]);
+                        acc[t][2] = fmaf(x.z, y[t].z, acc[t][2]);
+                        acc[t][3] = fmaf(x.w, y[t].w, acc[t][3]);
+                    }
+                }
+            }
+            // the butterfly over the eight rows together: offsets 16, 8 and 4 halve the rows a lane
+            // keeps (row lane / 4 is left), offsets 2 and 1 finish it
+            float v[8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t)
+                v[t] = __fadd_rn(__fadd_rn(acc[t][0], acc[t][1]), __fadd_rn(acc[t][2], acc[t][3]));
+#pragma unroll
+            for (int o = 16, n = 4; o >= 4; o >>= 1, n >>= 1) {
+                const bool up = (lane & o) != 0;
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    if (t < n)
+                        v[t] = __fadd_rn(up ? v[t + n] : v[t], __shfl_xor_sync(kFull, up ? v[t] : v[t + n], o));
+            }
+            v[0] = __fadd_rn(v[0], __shfl_xor_sync(kFull, v[0], 2));
+            v[0] = __fadd_rn(v[0], __shfl_xor_sync(kFull, v[0], 1));
+            const float got = __shfl_sync(kFull, v[0], 4 * (lane & 7));
+            if ((lane & 24) == b) mine = got;
+        }
+        return mine;
     }
 }
 
 // Alg. 1 over one graph whose rows are Xt[v] / adj[v * M] for local ids v < nt. Keys carry
-// global ids (local + id_off). The pool C (<= L <= 32 * MAXS keys, sorted by (delta, id))
-// lives in registers: entry e = 32 s + lane is pk[s] of that lane, its "expanded" mark bit s
-// of expd. Candidates that cannot beat the worst entry of a full pool are never inserted.
-// MAXS = 1 (L <= 32) inserts a batch at once: each candidate's rank among the pool (a
-// binary search of the shared-memory copy, which holds the pool in slots 0 .. n - 1 and empty
-// keys after) and among the other candidates, each pool entry's shift, one scatter through
-// shared memory (pool, pflag). Larger pools insert one candidate at a time (one ballot for its
-// rank, one shift).
-// Returns the pool size and leaves the pool in pool[0 .. size).
+// global ids (local + id_off). The pool C (<= L <= 32 * MAXS entries, sorted by (delta, id)) lives in
+// registers: entry e = 32 s + lane is pk[s] of that lane; pool[] in shared memory holds a copy. An
+// entry's low word is id << 1 | expanded (ids are below 2^31), so entries of different ids order by
+// (delta, id) whatever their marks, and the empty key (all ones) reads as expanded. Slots past the
+// pool's size, and past L, hold the empty key, so pool[L - 1] is the key a candidate has to beat.
+// The candidates of an expansion that beat it enter together: each finds its rank among the pool
+// entries by a binary search of the copy, its rank among the other candidates and every pool
+// entry's shift come from one loop over them, and one scatter through shared memory writes the
+// merged pool. (Inserting them one by one, a ballot and a shift of all slots each, took half of the
+// kernel's instructions at L = 48.)
+// Returns the pool size and leaves the keys (delta, id) in pool[0 .. size).
 // scratch: 32 ints of shared memory for the compacted neighbour ids.
 constexpr int kPoolSlots = 4;
-
-template <int MAXS>
-__device__ __forceinline__ uint64_t pick_slot(const uint64_t (&pk)[MAXS], int s) {
-    uint64_t v = pk[0];
-#pragma unroll
-    for (int t = 1; t < MAXS; ++t)
-        if (s == t) v = pk[t];
-    return v;
-}
+__host__ __device__ inline int pool_entries(int L) { return L <= 32 ? 32 : L <= 64 ? 64 : 128; }
 
 template <int METRIC, bool SMALLD, typename RT, int MAXS>
-__device__ int beam_search(const RT* __restrict__ Xt, const float* __restrict__ invt, const int32_t* __restrict__ adj,
-                           int M, long long nt, int ep, long long id_off, const float* q, float4 qreg,
-                           const QBytes& qb, float qinv, int d, int L, uint64_t* pool, uint8_t* pflag, int32_t* ht,
-                           int htbits, int32_t* scratch, float* P, WarpCounters& ctr, int* status,
+__device__ __forceinline__ int beam_search(const RT* __restrict__ Xt, const float* __restrict__ invt, const int32_t* __restrict__ adj,
+                           int M, int nt, int ep, int id_off, const Query& Q, float qinv, int d, int L, uint64_t* pool,
+                           uint16_t* ht, int htbits, int32_t* scratch, WarpCounters& ctr, int* status,
                            bool dedupe = true) {
     const int lane = lane_id();
     const unsigned lt = (1u << lane) - 1u;
-    const int H = 1 << htbits;
-    const int S = MAXS == 1 ? 1 : (L + 31) >> 5;
-    for (int s = lane; s < H; s += 32) ht[s] = -1;
-    if (lane == 0) scratch[0] = ep;
-    if (MAXS == 1) pool[lane] = kEmptyKey;   // slots past the pool size stay empty
-    __syncwarp();
-    if (ep < 0 || ep >= nt || L < 1 || S > MAXS || (MAXS == 1 && L > 32)) {
+    if (ep < 0 || ep >= nt || L < 1 || L > 32 * MAXS) {
         if (lane == 0) atomicOr(status, kErrBounds);
         return 0;
     }
+    const VisitedHash H(nt, htbits);
+    ht_clear(ht, htbits, lane);
+    if (lane == 0) scratch[0] = ep;
     uint64_t pk[MAXS];
 #pragma unroll
-    for (int s = 0; s < MAXS; ++s) pk[s] = kEmptyKey;
-    unsigned expd = 0u;
-    int n;
-    uint64_t worst = kEmptyKey;   // pool entry L - 1 once the pool is full
+    for (int s = 0; s < MAXS; ++s) {
+        pk[s] = kEmptyKey;
+        pool[32 * s + lane] = kEmptyKey;
+    }
+    __syncwarp();
     {
-        const float dd = rows_delta<METRIC, SMALLD, RT>(Xt, scratch, 1, q, qreg, qb, d, lane, P);
-        uint64_t key = kEmptyKey;
+        const float dd = rows_delta<METRIC, SMALLD, RT>(Xt, scratch, 1, Q, d, lane);
         if (lane == 0) {
             const float inv = (METRIC == FGIM_COSINE) ? __fmul_rn(qinv, invt[ep]) : 1.f;
-            key = mkkey(delta_finish<METRIC>(dd, inv), (int32_t)(ep + id_off));
-            ht[ht_slot(ep, htbits)] = ep;
-            ctr.ndc++;
-            pk[0] = key;
-            pool[0] = key;
+            pk[0] = mkkey(delta_finish<METRIC>(dd, inv), (int32_t)((uint32_t)(ep + id_off) << 1));
+            pool[0] = pk[0];
+            H.add(ht, ep);
         }
-        n = 1;
-        if (L == 1) worst = shfl64(key, 0);
         __syncwarp();
     }
     // every vertex is expanded at most once, so nt + 1 iterations always suffice; status[1],
     // when positive, is a smaller expansion budget (a test hook for the timeout path)
     bool done = false;
     const int hop_budget = status[1];
-    const long long budget = hop_budget > 0 ? (long long)hop_budget : nt + 1;
-    for (long long it = 0; it <= nt; ++it) {
-        int first = -1;
+    const unsigned budget = hop_budget > 0 ? (unsigned)hop_budget : (unsigned)nt + 1u;
+    unsigned it = 0, ndc = 1;
+    for (; it <= (unsigned)nt; ++it) {
+        // the first entry not yet expanded
+        int slot = -1;
+        unsigned open = 0u;
 #pragma unroll
         for (int s = 0; s < MAXS; ++s) {
-            if (s < S && first < 0) {
-                const unsigned m = __ballot_sync(kFull, 32 * s + lane < n && !((expd >> s) & 1u));
-                if (m) first = 32 * s + __ffs(m) - 1;
+            if (slot < 0) {
+                open = __ballot_sync(kFull, ((uint32_t)pk[s] & 1u) == 0u);
+                if (open) slot = s;
             }
         }
-        if (first < 0) {
+        if (slot < 0) {
             done = true;
             break;
         }
         if (it >= budget) break;
-        const uint64_t fk = shfl64(pick_slot<MAXS>(pk, first >> 5), first & 31);
-        if (lane == (first & 31)) expd |= 1u << (first >> 5);
-        if (lane == 0) ctr.hops++;
-        const long long u = (long long)key_id(fk) - id_off;
-        const int32_t* row = adj + u * M;
+        const int src = __ffs(open) - 1;
+        uint32_t lo = (uint32_t)pk[0];
+#pragma unroll
+        for (int s = 1; s < MAXS; ++s)
+            if (slot == s) lo = (uint32_t)pk[s];
+        const int u = (int)(__shfl_sync(kFull, lo, src) >> 1) - id_off;
+        if (lane == src) {
+#pragma unroll
+            for (int s = 0; s < MAXS; ++s)
+                if (slot == s) pk[s] |= 1ull;
+            reinterpret_cast<uint32_t*>(pool)[2 * (32 * slot + lane)] = lo | 1u;   // the copy's mark
+        }
+        const int32_t* row = adj + (long long)u * M;
         for (int c0 = 0; c0 < M; c0 += 32) {
             int v = (c0 + lane < M) ? row[c0 + lane] : -1;
             if (v >= nt) {
@@ -338,174 +395,148 @@ __device__ int beam_search(const RT* __restrict__ Xt, const float* __restrict__ 
                 const unsigned same = __match_any_sync(kFull, v);
                 if ((same & lt) != 0u) v = -1;
             }
-            if (v >= 0) {
-                const int s = ht_slot(v, htbits);
-                if (ht[s] == v) v = -1;
-                else ht[s] = v;
-            }
+            if (v >= 0 && H.seen(ht, v)) v = -1;
             const unsigned m = __ballot_sync(kFull, v >= 0);
+            if (m == 0u) continue;
             const int U = __popc(m);
-            if (U == 0) continue;
             if (v >= 0) scratch[__popc(m & lt)] = v;
             __syncwarp();
-            const float dd = rows_delta<METRIC, SMALLD, RT>(Xt, scratch, U, q, qreg, qb, d, lane, P);
+            const float dd = rows_delta<METRIC, SMALLD, RT>(Xt, scratch, U, Q, d, lane);
             uint64_t cand = kEmptyKey;
             if (lane < U) {
                 const int32_t w = scratch[lane];
                 const float inv = (METRIC == FGIM_COSINE) ? __fmul_rn(qinv, invt[w]) : 1.f;
-                cand = mkkey(delta_finish<METRIC>(dd, inv), (int32_t)(w + id_off));
-                ctr.ndc++;
+                cand = mkkey(delta_finish<METRIC>(dd, inv), (int32_t)((uint32_t)(w + id_off) << 1));
             }
+            ndc += (unsigned)U;
+            bool valid = cand < pool[L - 1];
+            __syncwarp();   // scratch has been read, pool[L - 1] too
+            if (__ballot_sync(kFull, valid) == 0u) continue;
+            // rank of the candidate among the pool's entries: halving steps over its 32, 64 or 128
+            // slots (a valid candidate ranks below the last one: it beats entry L - 1). An entry
+            // equal but for the mark means it is pooled already (the lossy table let it in).
+            int pos = 0;
+#pragma unroll
+            for (int st = 16 * MAXS; st > 0; st >>= 1)
+                if (pool[pos + st - 1] < cand) pos += st;
+            if (valid && (pool[pos] | 1ull) == (cand | 1ull)) valid = false;
+            unsigned vm = __ballot_sync(kFull, valid);
+            if (vm == 0u) continue;
+            // the candidates are distinct: rank among them, and each pool entry's shift
+            int crank = pos, shift[MAXS];
+#pragma unroll
+            for (int s = 0; s < MAXS; ++s) shift[s] = 0;
+            do {
+                const uint64_t cj = shfl64(cand, __ffs(vm) - 1);
+                vm &= vm - 1;
+                crank += cj < cand ? 1 : 0;
+#pragma unroll
+                for (int s = 0; s < MAXS; ++s) shift[s] += cj < pk[s] ? 1 : 0;
+            } while (vm);
+            // merged order: pool entry e goes to e + shift, a candidate to its rank among both
             __syncwarp();
-            bool valid = cand < worst;
-            if constexpr (MAXS == 1) {
-                if (__ballot_sync(kFull, valid) == 0u) continue;
-                // rank of the candidate among the pool entries (pool[e] is the empty key for
-                // e >= n): five halving steps over the 32 slots. A valid candidate ranks below
-                // slot 31 (it beats the worst entry of a full pool, or the pool has empty slots).
-                // An equal entry means it is pooled already (the lossy visited table let it in).
-                int pos = 0;
 #pragma unroll
-                for (int st = 16; st > 0; st >>= 1)
-                    if (pool[pos + st - 1] < cand) pos += st;
-                if (valid && pool[pos] == cand) valid = false;
-                unsigned vm = __ballot_sync(kFull, valid);
-                if (vm == 0u) continue;
-                const int added = __popc(vm);
-                // the candidates are distinct: rank among them, and each pool entry's shift
-                int crank = 0, shift = 0;
-                while (vm) {
-                    const int j = __ffs(vm) - 1;
-                    vm &= vm - 1;
-                    const uint64_t cj = shfl64(cand, j);
-                    crank += cj < cand ? 1 : 0;
-                    shift += cj < pk[0] ? 1 : 0;
-                }
-                // merged order: pool entry e goes to e + shift, a candidate to pos + crank
-                const bool in_pool = lane < n;
-                const int pe = lane + shift, pc = pos + crank;
-                __syncwarp();
-                if (in_pool && pe < L) {
-                    pool[pe] = pk[0];
-                    pflag[pe] = (uint8_t)(expd & 1u);
-                }
-                if (valid && pc < L) {
-                    pool[pc] = cand;
-                    pflag[pc] = 0;
-                }
-                __syncwarp();
-                n = n + added < L ? n + added : L;
-                pk[0] = pool[lane];
-                expd = lane < n ? (unsigned)pflag[lane] : 0u;
-                __syncwarp();
-                if (n == L) worst = shfl64(pk[0], L - 1);
-            } else {
-                unsigned vm;
-                while ((vm = __ballot_sync(kFull, valid)) != 0u) {
-                    const int src = __ffs(vm) - 1;
-                    const uint64_t c = shfl64(cand, src);
-                    if (lane == src) valid = false;
-                    bool eq = false;
-                    int pos = 0;
-#pragma unroll
-                    for (int s = 0; s < MAXS; ++s) {
-                        if (s < S) {
-                            eq |= pk[s] == c;
-                            pos += __popc(__ballot_sync(kFull, pk[s] < c));
-                        }
-                    }
-                    if (__any_sync(kFull, eq)) continue;   // already in the pool (same id, same key)
-                    // entries pos .. n - 1 move up by one; the slots are updated from the last
-                    // one down so every slot reads its predecessor's old entries
-#pragma unroll
-                    for (int s = MAXS - 1; s >= 0; --s) {
-                        if (s < S) {
-                            const uint64_t up = shfl64(pk[s], (lane + 31) & 31);
-                            const unsigned eup = __shfl_sync(kFull, (expd >> s) & 1u, (lane + 31) & 31);
-                            uint64_t prev = up;
-                            unsigned eprev = eup;
-                            if (s > 0) {
-                                const uint64_t w31 = shfl64(pk[s > 0 ? s - 1 : 0], 31);
-                                const unsigned e31 = __shfl_sync(kFull, (expd >> (s > 0 ? s - 1 : 0)) & 1u, 31);
-                                if (lane == 0) {
-                                    prev = w31;
-                                    eprev = e31;
-                                }
-                            }
-                            const int e = 32 * s + lane;
-                            if (e > pos && !(s == 0 && lane == 0)) {
-                                pk[s] = prev;
-                                expd = (expd & ~(1u << s)) | (eprev << s);
-                            } else if (e == pos) {
-                                pk[s] = c;
-                                expd &= ~(1u << s);
-                            }
-                            if (e >= L) {
-                                pk[s] = kEmptyKey;
-                                expd &= ~(1u << s);
-                            }
-                        }
-                    }
-                    n = n < L ? n + 1 : L;
-                    if (n == L) worst = shfl64(pick_slot<MAXS>(pk, (L - 1) >> 5), (L - 1) & 31);
-                    valid = valid && cand < worst;
-                }
+            for (int s = 0; s < MAXS; ++s) {
+                const int e = 32 * s + lane + shift[s];
+                if (shift[s] != 0 && pk[s] != kEmptyKey && e < L) pool[e] = pk[s];
             }
+            if (valid && crank < L) pool[crank] = cand;
+            __syncwarp();
+#pragma unroll
+            for (int s = 0; s < MAXS; ++s) pk[s] = pool[32 * s + lane];
         }
     }
     if (!done && lane == 0) atomicOr(status, kErrTimeout);
+    ctr.ndc += ndc;
+    ctr.hops += it;
+    int n = 0;
+    __syncwarp();
 #pragma unroll
-    for (int s = 0; s < MAXS; ++s)
-        if (s < S && 32 * s + lane < n) pool[32 * s + lane] = pk[s];
+    for (int s = 0; s < MAXS; ++s) {
+        n += __popc(__ballot_sync(kFull, pk[s] != kEmptyKey));
+        if (pk[s] != kEmptyKey) pool[32 * s + lane] = (pk[s] & 0xffffffff00000000ull) | ((uint32_t)pk[s] >> 1);
+    }
     __syncwarp();
     return n;
 }
 
-__device__ __forceinline__ void warp_add_counters(WarpCounters& c, unsigned long long* out) {
-    long long a = c.ndc, b = c.hops;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(kFull, a, o);
-        b += __shfl_xor_sync(kFull, b, o);
-    }
+__device__ __forceinline__ void warp_add_counters(const WarpCounters& c, unsigned long long* out) {
     if (lane_id() == 0 && out) {
-        atomicAdd(out + 0, (unsigned long long)a);
-        atomicAdd(out + 1, (unsigned long long)b);
+        atomicAdd(out + 0, (unsigned long long)c.ndc);
+        atomicAdd(out + 1, (unsigned long long)c.hops);
     }
+}
+
+// The items (queries, rows) of a beam-search launch: a warp starts with its own and takes further ones
+// from *next, which counts the items handed out so, until it passes the last.
+__device__ __forceinline__ long long first_item() {
+    return (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+}
+template <bool MORE>   // false: one item per warp
+__device__ __forceinline__ long long next_item(unsigned long long* next) {
+    if (!MORE || !next) return 0x7fffffffffffffffLL;
+    unsigned long long v = 0;
+    if (lane_id() == 0) v = atomicAdd(next, 1ull);
+    __syncwarp();
+    return (long long)shfl64(v, 0) + (long long)gridDim.x * (blockDim.x >> 5);
 }
 
 // shared-memory layout of one warp; all offsets multiples of 16 bytes
 struct WarpLayout {
-    int q, pool, pflag, ht, res, scratch, part, bytes;
+    int q, pool, ht, res, scratch, bytes;
 };
 
 __host__ __device__ inline int align16(int x) { return (x + 15) & ~15; }
 
-// part (the 32 x 33 partial matrix) is needed by FP32 rows only
-__host__ __device__ inline WarpLayout warp_layout(int d, int L, int htbits, int kres, bool part = true) {
+// qrow: the query is kept in shared memory (rows wider than 128 coordinates)
+__host__ __device__ inline WarpLayout warp_layout(int d, int L, int htbits, int kres, bool qrow) {
     WarpLayout w;
     int o = 0;
     w.q = o;
-    o += align16(d * 4);
-    // the pool holds at least 32 slots: a one-slot register pool searches all 32 for a rank
-    const int ps = L < 32 ? 32 : L;
+    if (qrow) o += align16(d * 4);
     w.pool = o;
-    o += align16(ps * 8);
-    w.pflag = o;
-    o += align16(ps);
+    o += pool_entries(L) * 8;
     w.ht = o;
-    o += align16((1 << htbits) * 4);
+    o += (1 << htbits) * 2;
     w.res = o;
     o += align16(kres * 8);
     w.scratch = o;
     o += 32 * 4;
-    w.part = o;
-    if (part) o += 32 * 33 * 4;
     w.bytes = o;
     return w;
 }
 
 // ---------------------------------------------------------------------------- host
+// Warps per block when the autotuner has no choice for the workload. Rows of up to 128 coordinates: the
+// launch keeps as many blocks as fit and every warp takes its items from a counter, so that no warp
+// waits for the longest search of its block and the shape of a block does not matter (cross query of
+// the 1M Sift-like merge 56.7 ms with one block of four warps per four rows, 54.6 ms with blocks of one
+// warp, 52.5 ms so with one, two or four). Wider rows: one warp per block and per item; the loop over
+// items costs registers that the loads in flight need there (120k, d = 768 BF16: 12.5 ms, 14.9 ms as
+// resident blocks).
+static inline int beam_warps(int d) { return d <= 128 ? 4 : 1; }
+
+// Grid of a beam-search kernel over nq items of rows of d coordinates, and the counter its warps take
+// their items from: *next (counters[8], zeroed here) hands out the items after the first of every warp;
+// nullptr: one item per warp (few items, wide rows).
+template <typename K>
+cudaError_t beam_grid(K kernel, int d, int wpb, size_t smem, long long nq, unsigned long long* counters, unsigned* blocks,
+                      unsigned long long** next, cudaStream_t s) {
+    const long long need = (nq + wpb - 1) / wpb;
+    *blocks = (unsigned)need;
+    *next = nullptr;
+    if (d > 128) return cudaSuccess;
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess || need <= sms * 4LL) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, wpb * 32, smem)) != cudaSuccess) return e;
+    if (per_sm < 1 || need <= (long long)per_sm * sms) return e;
+    *blocks = (unsigned)(per_sm * sms);
+    *next = counters + 8;
+    return cudaMemsetAsync(*next, 0, sizeof(**next), s);
+}
+
 static inline int ht_bits_for(int L) {
     int want = 32 * L;
     int b = 9;
@@ -525,21 +556,36 @@ static inline int ht_bits_for(int L) {
         }                                                                                        \
     } while (0)
 // BF16 rows (d > 128 only: small rows gain little)
-#define FGIM_DISPATCH_ALL_WIDE(M, L, MACRO, RT)                                                     \
-    do {                                                                                          \
-        const int ms_ = (L) <= 32 ? 1 : kPoolSlots;                                               \
-        if ((M) == FGIM_L2SQ) {                                                                   \
-            if (ms_ == 1) MACRO(FGIM_L2SQ, false, RT, 1); else MACRO(FGIM_L2SQ, false, RT, kPoolSlots); \
-        } else if ((M) == FGIM_IP) {                                                              \
-            if (ms_ == 1) MACRO(FGIM_IP, false, RT, 1); else MACRO(FGIM_IP, false, RT, kPoolSlots); \
-        } else {                                                                                  \
-            if (ms_ == 1) MACRO(FGIM_COSINE, false, RT, 1); else MACRO(FGIM_COSINE, false, RT, kPoolSlots); \
-        }                                                                                         \
+#define FGIM_DISPATCH_WIDE_MS(M, MACRO, RT, MS)                                                   \
+    do {                                                                                         \
+        if ((M) == FGIM_L2SQ) MACRO(FGIM_L2SQ, false, RT, MS);                                   \
+        else if ((M) == FGIM_IP) MACRO(FGIM_IP, false, RT, MS);                                  \
+        else MACRO(FGIM_COSINE, false, RT, MS);                                                  \
     } while (0)
-// register pool of one slot (L <= 32) or of kPoolSlots slots
+#define FGIM_DISPATCH_ALL_WIDE(M, L, MACRO, RT)                                                  \
+    do {                                                                                         \
+        if ((L) <= 32) FGIM_DISPATCH_WIDE_MS(M, MACRO, RT, 1);                                   \
+        else if ((L) <= 64) FGIM_DISPATCH_WIDE_MS(M, MACRO, RT, 2);                              \
+        else FGIM_DISPATCH_WIDE_MS(M, MACRO, RT, kPoolSlots);                                    \
+    } while (0)
+// byte rows (d <= 128 only)
+#define FGIM_DISPATCH_BYTES_MS(M, MACRO, MS)                                                     \
+    do {                                                                                         \
+        if ((M) == FGIM_L2SQ) MACRO(FGIM_L2SQ, true, uint8_t, MS);                               \
+        else if ((M) == FGIM_IP) MACRO(FGIM_IP, true, uint8_t, MS);                              \
+        else MACRO(FGIM_COSINE, true, uint8_t, MS);                                              \
+    } while (0)
+#define FGIM_DISPATCH_ALL_BYTES(M, L, MACRO)                                                     \
+    do {                                                                                         \
+        if ((L) <= 32) FGIM_DISPATCH_BYTES_MS(M, MACRO, 1);                                      \
+        else if ((L) <= 64) FGIM_DISPATCH_BYTES_MS(M, MACRO, 2);                                 \
+        else FGIM_DISPATCH_BYTES_MS(M, MACRO, kPoolSlots);                                       \
+    } while (0)
+// register pool of one slot (L <= 32), two (L <= 64) or kPoolSlots slots
 #define FGIM_DISPATCH_ALL(M, D, L, MACRO, RT)                                                     \
     do {                                                                                         \
         if ((L) <= 32) FGIM_DISPATCH_METRIC_D(M, D, MACRO, RT, 1);                               \
+        else if ((L) <= 64) FGIM_DISPATCH_METRIC_D(M, D, MACRO, RT, 2);                          \
         else FGIM_DISPATCH_METRIC_D(M, D, MACRO, RT, kPoolSlots);                                \
     } while (0)
 

@@ -74,20 +74,12 @@ __global__ void __launch_bounds__(128) k_layer_knn(const float* __restrict__ Xl,
     const unsigned lt = (1u << lane) - 1u;
     const long long u = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
     if (u >= n) return;
-    const size_t per_warp = (size_t)align16(d * 4) + align16(kk * 8) + 32 * 4 + (sizeof(RT) == 1 ? 0 : 32 * 33 * 4);
+    const int qb = SMALLD ? 0 : align16(d * 4);   // wide rows keep the query in shared memory
+    const size_t per_warp = (size_t)qb + align16(kk * 8) + 32 * 4;
     unsigned char* base = smem + per_warp * warp;
-    float* q = reinterpret_cast<float*>(base);
-    uint64_t* list = reinterpret_cast<uint64_t*>(base + align16(d * 4));
-    int32_t* scratch = reinterpret_cast<int32_t*>(base + align16(d * 4) + align16(kk * 8));
-    float* P = reinterpret_cast<float*>(base + align16(d * 4) + align16(kk * 8) + 32 * 4);
-    const float4* src = reinterpret_cast<const float4*>(Xl + u * d);
-    for (int c = lane; c < (d >> 2); c += 32) reinterpret_cast<float4*>(q)[c] = src[c];
-    __syncwarp();
-    const float4 qreg = (SMALLD && lane < (d >> 2)) ? reinterpret_cast<const float4*>(q)[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
-    QBytes qb;
-    qb.w = make_uint4(0u, 0u, 0u, 0u);
-    qb.q2 = 0u;
-    if (sizeof(RT) == 1) qb = query_bytes(q, d, lane);
+    uint64_t* list = reinterpret_cast<uint64_t*>(base + qb);
+    int32_t* scratch = reinterpret_cast<int32_t*>(base + qb + align16(kk * 8));
+    const Query Q = load_query<SMALLD, RT>(Xl + u * d, reinterpret_cast<float*>(base), d, lane);
     const float qinv = METRIC == FGIM_COSINE ? inv[u] : 1.f;
     int nl = 0;
     for (long long c0 = 0; c0 < u; c0 += 32) {
@@ -97,7 +89,7 @@ __global__ void __launch_bounds__(128) k_layer_knn(const float* __restrict__ Xl,
         const int U = __popc(m);
         if (ok) scratch[__popc(m & lt)] = (int32_t)v;
         __syncwarp();
-        const float dd = rows_delta<METRIC, SMALLD, RT>(Xr, scratch, U, q, qreg, qb, d, lane, P);
+        const float dd = rows_delta<METRIC, SMALLD, RT>(Xr, scratch, U, Q, d, lane);
         uint64_t key = kEmptyKey;
         if (lane < U) {
             const int32_t w = scratch[lane];
@@ -117,7 +109,7 @@ cudaError_t launch_layer_knn(const float* Xl, const uint8_t* X8l, const float* i
     if (n <= 0) return cudaSuccess;
     const bool bytes = X8l && byte_rows_ok(d);
     const int wpb = 4;
-    const size_t per_warp = (size_t)align16(d * 4) + align16(kk * 8) + 32 * 4 + (bytes ? 0 : 32 * 33 * 4);
+    const size_t per_warp = (size_t)(d > 128 ? align16(d * 4) : 0) + align16(kk * 8) + 32 * 4;
     const size_t smem = per_warp * wpb;
     const unsigned blocks = (unsigned)((n + wpb - 1) / wpb);
     cudaError_t e = cudaSuccess;
