@@ -673,7 +673,7 @@ static void prune(Ctx& c, const Problem& P, const fgim_params* p, const fgim_knn
     rule.kind = p->prune_rule;
     rule.alpha2 = (float)((double)p->alpha * (double)p->alpha);   // alpha^2 and 3 tau rounded once to FP32
     rule.tau3 = (float)(3.0 * (double)p->tau);
-    ck(launch_prune(P.X, P.X8, P.inv, P.N, P.d, P.metric, *g, T, p->R, rule, e_ids, e_dist, e_cnt, c.status, c.s));
+    ck(launch_prune(P.X, P.X8, P.Xh, P.inv, P.N, P.d, P.metric, *g, T, p->R, rule, e_ids, e_dist, e_cnt, c.status, c.s));
 }
 
 static void reverse_insert(Ctx& c, long long N, int R, const int32_t* e_ids, const float* e_dist, const int32_t* e_cnt,
@@ -1266,7 +1266,7 @@ static void build_layer_graph(Ctx& c, const float* X, int dim, int metric, const
     float* e_dist = c.alloc<float>(nl * M);
     int32_t* e_cnt = c.alloc<int32_t>(nl);
     const PruneRule rng = {FGIM_PRUNE_ALPHA_RNG, 1.f, 0.f};   // HNSW's heuristic: alpha = 1, no indegree clause
-    ck(launch_prune(L.X, L.X8, L.inv, nl, dim, metric, g1, T, M, rng, e_ids, e_dist, e_cnt, c.status, c.s));
+    ck(launch_prune(L.X, L.X8, L.Xh, L.inv, nl, dim, metric, g1, T, M, rng, e_ids, e_dist, e_cnt, c.status, c.s));
     const int wide = FGIM_MAX_K;   // own and reverse edges together (their 128 nearest if more)
     int32_t* w_ids = c.alloc<int32_t>(nl * wide);
     float* w_dist = c.alloc<float>(nl * wide);
@@ -1286,7 +1286,7 @@ static void build_layer_graph(Ctx& c, const float* X, int dim, int metric, const
     g2.n = nl;
     g2.k = wide;
     float* f_dist = c.alloc<float>(nl * M);
-    ck(launch_prune(L.X, L.X8, L.inv, nl, dim, metric, g2, T, M, rng, adj, f_dist, deg, c.status, c.s));
+    ck(launch_prune(L.X, L.X8, L.Xh, L.inv, nl, dim, metric, g2, T, M, rng, adj, f_dist, deg, c.status, c.s));
 }
 
 fgim_status fgim_hnsw_layer(const void* vectors, int64_t n, int32_t dim, int32_t dtype, int32_t metric,
@@ -1400,7 +1400,7 @@ fgim_status fgim_build_pg(const void* vectors, int64_t n, int32_t dim, int32_t d
             g1.dist = res_d;
             g1.n = b;
             g1.k = ef;
-            ck(launch_prune(P.X, P.X8, P.inv, n, dim, metric, g1, zeros, M, heur, e_ids, e_dist, e_cnt, c.status, c.s));
+            ck(launch_prune(P.X, P.X8, P.Xh, P.inv, n, dim, metric, g1, zeros, M, heur, e_ids, e_dist, e_cnt, c.status, c.s));
             // 2. the batch's lists go in, their entries are reverse edges of their targets
             ck(cudaMemsetAsync(cin, 0, sizeof(int32_t) * n, c.s));
             ck(cudaMemsetAsync(fill, 0, sizeof(int32_t) * n, c.s));
@@ -1422,7 +1422,7 @@ fgim_status fgim_build_pg(const void* vectors, int64_t n, int32_t dim, int32_t d
                 g2.dist = ov_dist;
                 g2.n = nov;
                 g2.k = M + (int)b;
-                ck(launch_prune(P.X, P.X8, P.inv, n, dim, metric, g2, zeros, M, heur, o_ids, o_dist, o_cnt, c.status,
+                ck(launch_prune(P.X, P.X8, P.Xh, P.inv, n, dim, metric, g2, zeros, M, heur, o_ids, o_dist, o_cnt, c.status,
                                 c.s));
                 ck(launch_pg_write_back(ov_tgt, nov, M, o_ids, o_dist, o_cnt, adj, nd, deg, c.s));
             }

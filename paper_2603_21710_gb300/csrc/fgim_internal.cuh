@@ -207,40 +207,6 @@ __device__ __forceinline__ float warp_butterfly(float v) {
     return v;
 }
 
-// Non-canonical FP32 distance by one thread: sequential over the chunks with four
-// accumulators. Used only as a filter; decisions near its value are re-taken with the
-// canonical distance (the two differ by less than fp32_pair_margin of the sum of |terms|).
-template <int METRIC>
-__device__ __forceinline__ float seq_sum(const float4* __restrict__ a, const float4* __restrict__ b, int nc4) {
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll 4
-    for (int c = 0; c < nc4; ++c) {
-        const float4 x = a[c];
-        const float4 y = b[c];
-        if (METRIC == FGIM_L2SQ) {
-            const float e0 = x.x - y.x, e1 = x.y - y.y, e2 = x.z - y.z, e3 = x.w - y.w;
-            s0 = fmaf(e0, e0, s0);
-            s1 = fmaf(e1, e1, s1);
-            s2 = fmaf(e2, e2, s2);
-            s3 = fmaf(e3, e3, s3);
-        } else {
-            s0 = fmaf(x.x, y.x, s0);
-            s1 = fmaf(x.y, y.y, s1);
-            s2 = fmaf(x.z, y.z, s2);
-            s3 = fmaf(x.w, y.w, s3);
-        }
-    }
-    return (s0 + s1) + (s2 + s3);
-}
-
-// canonical distance of one row pair by one warp (all lanes get it)
-template <int METRIC>
-__device__ __forceinline__ float warp_delta(const float* a, const float* b, int d, float inv_ab, int lane) {
-    const float p = lane_part<METRIC>(reinterpret_cast<const float4*>(a), reinterpret_cast<const float4*>(b), d >> 2,
-                                      lane);
-    return delta_finish<METRIC>(warp_butterfly(p), inv_ab);
-}
-
 // rounding margin between two FP32 evaluations of the same distance that both follow
 // sums of at most d/4 + 8 terms per chain: the worst-case relative error of either is
 // below (d/4 + 8) * 2^-24 of the sum of |terms| (Higham, Accuracy and Stability of

@@ -124,11 +124,13 @@ cudaError_t launch_repair_rounds(fgim_knng& g, int32_t* T, const int32_t* zeros,
 cudaError_t launch_zero_flags(const int32_t* T, long long N, int32_t* flag, cudaStream_t s);
 cudaError_t launch_nonzero_flags(const uint8_t* v, long long N, int32_t* flag, cudaStream_t s);
 
-// ---- k_prune.cu
-// Alg. 5 neighbour selection of the g.n lists of g (ids in 0 .. N - 1, rows of X) with `rule`
-cudaError_t launch_prune(const float* X, const uint8_t* X8, const float* inv_norm, long long N, int d, int metric,
-                         const fgim_knng& g, const int32_t* T, int R, PruneRule rule, int32_t* e_ids, float* e_dist,
+// ---- k_select.cu
+// Alg. 5 neighbour selection of the g.n lists of g (ids in 0 .. N - 1, rows of X; X8 and Xh: the same
+// rows as bytes and as BF16, or nullptr) with `rule`
+cudaError_t launch_prune(const float* X, const uint8_t* X8, const uint16_t* Xh, const float* inv_norm, long long N,
+                         int d, int metric, const fgim_knng& g, const int32_t* T, int R, PruneRule rule, int32_t* e_ids, float* e_dist,
                          int32_t* e_cnt, int* status, cudaStream_t s);
+// ---- k_prune.cu
 struct ReverseBuffers {
     int32_t* cnt;
     long long* off;

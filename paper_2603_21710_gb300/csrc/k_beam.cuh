@@ -162,7 +162,11 @@ __device__ __forceinline__ T take_row_totals(const T (&v)[4], int r0, T mine, in
 // integer below 128 * 255^2 < 2^24, so it is exact and the canonical value is the exact
 // integer result. Lanes take 16 bytes each (32 / lanes-per-row rows per warp load) and form
 // |q|^2 + |x|^2 - 2 q.x with four-way byte dot products, summed over the row's lanes.
-template <int METRIC, bool SMALLD, typename RT>
+// SKIP (FP32 rows up to 128 coordinates): the chunks past the row's end are left out by a branch (the same for
+// every lane) instead of adding zeros. Faster where many warps share an SM (cross query at d = 96:
+// 16.8 -> 15.0 ms, d = 32: 0.46 -> 0.42 ms), slower where few searches wait for each other's chain
+// (k_search of 10,000 queries 0.90 -> 0.99 ms), so k_search leaves it off.
+template <int METRIC, bool SMALLD, typename RT, bool SKIP = true>
 __device__ __forceinline__ float rows_delta(const RT* __restrict__ base, const int32_t* rid, int U, const Query& Q,
                                             int d, int lane) {
     const int nc4 = d >> 2;
@@ -235,9 +239,10 @@ __device__ __forceinline__ float rows_delta(const RT* __restrict__ base, const i
                 }
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
-                    float pt[4];
+                    float pt[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) pt[i] = chunk_part<METRIC>(Q.c[i], y[t][i]);
+                    for (int i = 0; i < 4; ++i)
+                        if (!SKIP || 8 * i < nc4) pt[i] = chunk_part<METRIC>(Q.c[i], y[t][i]);
                     sv[2 * hf + t] = __fadd_rn(__fadd_rn(pt[0], pt[2]), __fadd_rn(pt[1], pt[3]));
                 }
             }
@@ -317,7 +322,7 @@ __device__ __forceinline__ float rows_delta(const RT* __restrict__ base, const i
 constexpr int kPoolSlots = 4;
 __host__ __device__ inline int pool_entries(int L) { return L <= 32 ? 32 : L <= 64 ? 64 : 128; }
 
-template <int METRIC, bool SMALLD, typename RT, int MAXS>
+template <int METRIC, bool SMALLD, typename RT, int MAXS, bool SKIP>
 __device__ __forceinline__ int beam_search(const RT* __restrict__ Xt, const float* __restrict__ invt, const int32_t* __restrict__ adj,
                            int M, int nt, int ep, int id_off, const Query& Q, float qinv, int d, int L, uint64_t* pool,
                            uint16_t* ht, int htbits, int32_t* scratch, WarpCounters& ctr, int* status,
@@ -339,7 +344,7 @@ __device__ __forceinline__ int beam_search(const RT* __restrict__ Xt, const floa
     }
     __syncwarp();
     {
-        const float dd = rows_delta<METRIC, SMALLD, RT>(Xt, scratch, 1, Q, d, lane);
+        const float dd = rows_delta<METRIC, SMALLD, RT, SKIP>(Xt, scratch, 1, Q, d, lane);
         if (lane == 0) {
             const float inv = (METRIC == FGIM_COSINE) ? __fmul_rn(qinv, invt[ep]) : 1.f;
             pk[0] = mkkey(delta_finish<METRIC>(dd, inv), (int32_t)((uint32_t)(ep + id_off) << 1));
@@ -401,7 +406,7 @@ __device__ __forceinline__ int beam_search(const RT* __restrict__ Xt, const floa
             const int U = __popc(m);
             if (v >= 0) scratch[__popc(m & lt)] = v;
             __syncwarp();
-            const float dd = rows_delta<METRIC, SMALLD, RT>(Xt, scratch, U, Q, d, lane);
+            const float dd = rows_delta<METRIC, SMALLD, RT, SKIP>(Xt, scratch, U, Q, d, lane);
             uint64_t cand = kEmptyKey;
             if (lane < U) {
                 const int32_t w = scratch[lane];

@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(128, sizeof(RT) == 1 ? 8 : SMALLD ? 5 : 4) k_c
         for (int j = t.grp[i]; j < t.gend[i]; ++j) {
             if (j == i) continue;
             const int nj = (int)(t.off[j + 1] - t.off[j]);
-            const int np = beam_search<METRIC, SMALLD, RT, MAXS>(Xr + t.off[j] * d,
+            const int np = beam_search<METRIC, SMALLD, RT, MAXS, true>(Xr + t.off[j] * d,
                                                                  inv_norm ? inv_norm + t.off[j] : nullptr, t.adj[j], t.M[j],
                                                                  nj, t.entry[j], (int)t.off[j], Q, qinv, d, Lq, pool, ht,
                                                                  htbits, scratch, ctr, status, dedupe);

@@ -1,14 +1,5 @@
-// Stage (c): k-NNG -> PG (Alg. 5) and the reachability fix.
-//
-// Neighbour selection runs one warp per vertex u. The candidate rows of u are staged in
-// shared memory (padded stride) when they fit; candidates are visited in ascending
-// (delta, id); for each one every kept w is tested in parallel (one lane per w) with the
-// selection rule (PruneRule: alpha-RNG delta(u, v) < alpha^2 * delta(w, v) keeps v, with alpha^2
-// rounded once to FP32 and the product in FP32; or MRNG; or tau-MNG). A lane's own sequential FP32 distance decides whenever the decision is further
-// from the boundary than the rounding margin between it and the canonical distance; the few
-// decisions inside the margin are re-taken with the canonical distance (whole warp), so the
-// outcome is exactly that of the canonical distance.
-// A vertex whose only in-edge is u (T(v) = 1) is kept unconditionally (Alg. 5).
+// Stage (c): the connectivity enhancement of Alg. 5 and the reachability fix (the neighbour
+// selection is in k_select.cu).
 //
 // Connectivity enhancement builds the reverse lists of the pruned snapshot E' by a
 // counting sort and merges them into E'(u), keeping the R smallest (delta, id).
@@ -26,405 +17,6 @@ namespace fgim {
 namespace cg = cooperative_groups;
 
 static inline long long cdivl(long long a, long long b) { return (a + b - 1) / b; }
-
-template <int METRIC, bool STAGE>
-__global__ void __launch_bounds__(64) k_prune(const float* __restrict__ X, const float* __restrict__ inv_norm,
-                                              long long N, long long nrows, int d, int k, const int32_t* __restrict__ ids,
-                                              const float* __restrict__ dist, const int32_t* __restrict__ T, int R,
-                                              PruneRule rule, int32_t* __restrict__ e_ids, float* __restrict__ e_dist,
-                                              int32_t* __restrict__ e_cnt, int* status) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int warp = threadIdx.x >> 5;
-    const int lane = lane_id();
-    const long long u = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
-    if (u >= nrows) return;
-    const int stride = d + 4;
-    const int nc4 = d >> 2;
-    const size_t per_warp = ((size_t)(STAGE ? k * stride * 4 : 0) + (size_t)k * 12 + 16 + 15) & ~(size_t)15;
-    unsigned char* base = smem + per_warp * warp;
-    float* rows = reinterpret_cast<float*>(base);
-    int32_t* cidv = reinterpret_cast<int32_t*>(base + (STAGE ? (size_t)k * stride * 4 : 0));
-    int32_t* kept = cidv + k;
-    float* nrm = reinterpret_cast<float*>(kept + k);
-    const float eps = fp32_pair_margin(d);
-
-    // valid prefix of list(u)
-    int nv = 0;
-    for (int s0 = 0; s0 < k; s0 += 32) {
-        const int s = s0 + lane;
-        int32_t id = s < k ? ids[u * k + s] : -1;
-        if (id >= N) {
-            atomicOr(status, kErrBounds);
-            id = -1;
-        }
-        if (s < k) cidv[s] = id;
-        nv += __popc(__ballot_sync(kFull, id >= 0));
-    }
-    __syncwarp();
-    if (STAGE) {
-        // coalesced: each warp pass copies one row
-        for (int r = 0; r < nv; ++r) {
-            const float4* src = reinterpret_cast<const float4*>(X + (long long)cidv[r] * d);
-            float4* dst = reinterpret_cast<float4*>(rows + r * stride);
-            for (int c = lane; c < nc4; c += 32) dst[c] = src[c];
-        }
-        __syncwarp();
-    }
-    auto rowp = [&](int idx) -> const float4* {
-        return STAGE ? reinterpret_cast<const float4*>(rows + idx * stride)
-                     : reinterpret_cast<const float4*>(X + (long long)cidv[idx] * d);
-    };
-    if (METRIC == FGIM_IP) {
-        // norms bound the rounding margin of the inner products
-        for (int r = lane; r < nv; r += 32) nrm[r] = sqrtf(seq_sum<FGIM_IP>(rowp(r), rowp(r), nc4)) * 1.0001f;
-        __syncwarp();
-    }
-    int nk = 0;
-    for (int t = 0; t < nv && nk < R; ++t) {
-        const int32_t v = cidv[t];
-        bool keep = T[v] == 1;
-        if (!keep) {
-            const float duv = dist[u * k + t];
-            const float4* rv = rowp(t);
-            bool occluded = false;
-            for (int s0 = 0; s0 < nk && !occluded; s0 += 32) {
-                const int s = s0 + lane;
-                bool occ = false, near = false;
-                float inv = 1.f;
-                if (s < nk) {
-                    const int wi = kept[s];
-                    const float sum = seq_sum<METRIC>(rowp(wi), rv, nc4);
-                    if (METRIC == FGIM_COSINE) inv = __fmul_rn(inv_norm[cidv[wi]], inv_norm[v]);
-                    const float dt = delta_finish<METRIC>(sum, inv);
-                    float md;   // bound on |filter distance - canonical distance|
-                    if (METRIC == FGIM_L2SQ) md = eps * sum * 1.01f;
-                    else if (METRIC == FGIM_IP) md = eps * nrm[wi] * nrm[t];
-                    else md = 2.f * eps;
-                    if (rule.kind == 0) {
-                        const float bound = rule.alpha2 * dt;
-                        // plus the rounding of the product
-                        const float m = rule.alpha2 * md + 2.f * 5.9604645e-8f * fabsf(bound);
-                        near = fabsf(duv - bound) <= m;
-                        occ = !near && !(duv < bound);
-                    } else {
-                        const bool can = rule.kind == 1 || dist[u * k + wi] < duv;
-                        const float thr = rule_thr(rule, duv);
-                        near = can && fabsf(dt - thr) <= md;
-                        occ = can && !near && dt < thr;
-                    }
-                }
-                if (__any_sync(kFull, occ)) {
-                    occluded = true;
-                    break;
-                }
-                // undecided: re-take each near decision with the canonical distance
-                unsigned nm = __ballot_sync(kFull, near);
-                while (nm && !occluded) {
-                    const int l = __ffs(nm) - 1;
-                    nm &= nm - 1;
-                    const int wi = kept[s0 + l];
-                    const float invl = (METRIC == FGIM_COSINE) ? __fmul_rn(inv_norm[cidv[wi]], inv_norm[v]) : 1.f;
-                    const float dc = delta_finish<METRIC>(
-                        warp_butterfly(lane_part<METRIC>(rowp(wi), rv, nc4, lane)), invl);
-                    if (rule_occludes(rule, duv, dist[u * k + wi], dc)) occluded = true;
-                }
-            }
-            keep = !occluded;
-        }
-        if (keep) {
-            if (lane == 0) kept[nk] = t;
-            ++nk;
-            __syncwarp();
-        }
-    }
-    for (int s = lane; s < R; s += 32) {
-        if (s < nk) {
-            e_ids[u * R + s] = cidv[kept[s]];
-            e_dist[u * R + s] = dist[u * k + kept[s]];
-        } else {
-            e_ids[u * R + s] = -1;
-            e_dist[u * R + s] = __int_as_float(0x7f800000);
-        }
-    }
-    if (lane == 0) e_cnt[u] = nk;
-}
-
-// Wide FP32 rows (d > 128): the warp forms every distance together in the canonical order
-// (lane chunks, butterfly), reading both rows coalesced from global memory, and tests the
-// kept neighbours of u one after another, stopping at the first that occludes v. Each
-// decision is taken on the canonical distance, which is what the filter-and-recheck form
-// decides as well, so the lists are the same; a rejected candidate usually costs a few
-// distances instead of one per kept neighbour.
-template <int METRIC>
-__global__ void __launch_bounds__(128) k_prune_wide(const float* __restrict__ X, const float* __restrict__ inv_norm,
-                                                    long long N, long long nrows, int d, int k, const int32_t* __restrict__ ids,
-                                                    const float* __restrict__ dist, const int32_t* __restrict__ T,
-                                                    int R, PruneRule rule, int32_t* __restrict__ e_ids,
-                                                    float* __restrict__ e_dist, int32_t* __restrict__ e_cnt,
-                                                    int* status) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int warp = threadIdx.x >> 5;
-    const int lane = lane_id();
-    const long long u = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
-    if (u >= nrows) return;
-    const int nc4 = d >> 2;
-    int32_t* cidv = reinterpret_cast<int32_t*>(smem) + (size_t)warp * 2 * k;
-    int32_t* kept = cidv + k;
-    int nv = 0;
-    for (int s0 = 0; s0 < k; s0 += 32) {
-        const int s = s0 + lane;
-        int32_t id = s < k ? ids[u * k + s] : -1;
-        if (id >= N) {
-            atomicOr(status, kErrBounds);
-            id = -1;
-        }
-        if (s < k) cidv[s] = id;
-        nv += __popc(__ballot_sync(kFull, id >= 0));
-    }
-    __syncwarp();
-    int nk = 0;
-    for (int t = 0; t < nv && nk < R; ++t) {
-        const int32_t v = cidv[t];
-        bool keep = T[v] == 1;
-        if (!keep) {
-            const float duv = dist[u * k + t];
-            const float4* rv = reinterpret_cast<const float4*>(X + (long long)v * d);
-            keep = true;
-            for (int s = 0; s < nk; ++s) {
-                const int32_t w = cidv[kept[s]];
-                const float sum = warp_butterfly(
-                    lane_part<METRIC>(reinterpret_cast<const float4*>(X + (long long)w * d), rv, nc4, lane));
-                const float inv = (METRIC == FGIM_COSINE) ? __fmul_rn(inv_norm[w], inv_norm[v]) : 1.f;
-                if (rule_occludes(rule, duv, dist[u * k + kept[s]], delta_finish<METRIC>(sum, inv))) {
-                    keep = false;
-                    break;
-                }
-            }
-        }
-        if (keep) {
-            if (lane == 0) kept[nk] = t;
-            ++nk;
-            __syncwarp();
-        }
-    }
-    for (int s = lane; s < R; s += 32) {
-        if (s < nk) {
-            e_ids[u * R + s] = cidv[kept[s]];
-            e_dist[u * R + s] = dist[u * k + kept[s]];
-        } else {
-            e_ids[u * R + s] = -1;
-            e_dist[u * R + s] = __int_as_float(0x7f800000);
-        }
-    }
-    if (lane == 0) e_cnt[u] = nk;
-}
-
-__host__ __device__ inline size_t prune_bytes_per_warp(int k, int d) {
-    return ((size_t)k * (d + 16) + (size_t)k * 16 + 15) & ~(size_t)15;
-}
-
-// Byte rows (every coordinate an integer in [0, 255], d <= 128, d % 16 == 0): the canonical
-// FP32 distance of two rows is then an exact integer (every partial sum is an integer below
-// 2^24), computed here directly: |a|^2 + |b|^2 - 2 a.b with four-way byte dot products. No
-// filter or re-check is needed. The candidate rows of u are staged as bytes (stride d + 16,
-// which spreads the lanes' rows over the banks), with their squared norms.
-template <int METRIC>
-__global__ void __launch_bounds__(128) k_prune_bytes(const uint8_t* __restrict__ X8, const float* __restrict__ inv_norm,
-                                                     long long N, long long nrows, int d, int k, const int32_t* __restrict__ ids,
-                                                     const float* __restrict__ dist, const int32_t* __restrict__ T,
-                                                     int R, PruneRule rule, int32_t* __restrict__ e_ids,
-                                                     float* __restrict__ e_dist, int32_t* __restrict__ e_cnt,
-                                                     int* status) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int warp = threadIdx.x >> 5;
-    const int lane = lane_id();
-    const long long u = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
-    if (u >= nrows) return;
-    const int stride = d + 16;
-    const size_t per_warp = prune_bytes_per_warp(k, d);
-    unsigned char* base = smem + per_warp * warp;
-    unsigned char* rows = base;
-    uint32_t* n2 = reinterpret_cast<uint32_t*>(base + (size_t)k * stride);
-    float* invs = reinterpret_cast<float*>(n2 + k);
-    int32_t* cidv = reinterpret_cast<int32_t*>(invs + k);
-    int32_t* kept = cidv + k;
-
-    // valid prefix of list(u), and its T and delta(u, .) held two per lane
-    int nv = 0;
-    for (int s0 = 0; s0 < k; s0 += 32) {
-        const int s = s0 + lane;
-        int32_t id = s < k ? ids[u * k + s] : -1;
-        if (id >= N) {
-            atomicOr(status, kErrBounds);
-            id = -1;
-        }
-        if (s < k) cidv[s] = id;
-        nv += __popc(__ballot_sync(kFull, id >= 0));
-    }
-    __syncwarp();
-    // stage the rows: 32 / lpr rows per warp load, lanes of a row take 16 bytes each
-    const int lpr = byte_lanes(d);
-    const int rpi = 32 >> byte_lanes_log2(d);
-    const int lsh = byte_lanes_log2(d);
-    const int sub = lane >> lsh, part = lane & (lpr - 1);
-    const bool has = part < (d >> 4);
-    for (int r0 = 0; r0 < nv; r0 += 4 * rpi) {
-        uint4 w[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int r = r0 + q * rpi + sub;
-            w[q] = make_uint4(0u, 0u, 0u, 0u);
-            if (r < nv && has) w[q] = *reinterpret_cast<const uint4*>(X8 + (long long)cidv[r] * d + 16 * part);
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int r = r0 + q * rpi + sub;
-            uint32_t sq = __dp4a(w[q].x, w[q].x, 0u);
-            sq = __dp4a(w[q].y, w[q].y, sq);
-            sq = __dp4a(w[q].z, w[q].z, sq);
-            sq = __dp4a(w[q].w, w[q].w, sq);
-            sq = row_group_sum(sq, lsh);
-            if (r < nv) {
-                if (has) *reinterpret_cast<uint4*>(rows + (size_t)r * stride + 16 * part) = w[q];
-                if (part == 0) n2[r] = sq;
-            }
-        }
-    }
-    if (METRIC == FGIM_COSINE)
-        for (int r = lane; r < nv; r += 32) invs[r] = inv_norm[cidv[r]];
-    // T(v) and delta(u, v) of the candidates, two per lane
-    int tA = 0, tB = 0;
-    float dA = 0.f, dB = 0.f;
-    if (lane < nv) {
-        tA = T[cidv[lane]];
-        dA = dist[u * k + lane];
-    }
-    if (lane + 32 < nv) {
-        tB = T[cidv[lane + 32]];
-        dB = dist[u * k + lane + 32];
-    }
-    __syncwarp();
-    const int c16n = d >> 4;
-    int nk = 0;
-    for (int t = 0; t < nv && nk < R; ++t) {
-        const int tv = __shfl_sync(kFull, t < 32 ? tA : tB, t & 31);
-        bool keep = tv == 1;
-        if (!keep) {
-            const float duv = __shfl_sync(kFull, t < 32 ? dA : dB, t & 31);
-            const unsigned char* rv = rows + (size_t)t * stride;
-            bool occ = false;
-            for (int s0 = 0; s0 < nk; s0 += 32) {
-                const int s = s0 + lane;
-                if (s < nk) {
-                    const int wi = kept[s];
-                    const unsigned char* rw = rows + (size_t)wi * stride;
-                    // four independent chains (integer sums: any order gives the same total)
-                    uint32_t d0 = 0u, d1 = 0u, d2 = 0u, d3 = 0u;
-                    for (int c = 0; c < c16n; ++c) {
-                        const uint4 a = *reinterpret_cast<const uint4*>(rw + 16 * c);
-                        const uint4 b = *reinterpret_cast<const uint4*>(rv + 16 * c);
-                        d0 = __dp4a(a.x, b.x, d0);
-                        d1 = __dp4a(a.y, b.y, d1);
-                        d2 = __dp4a(a.z, b.z, d2);
-                        d3 = __dp4a(a.w, b.w, d3);
-                    }
-                    const uint32_t dot = (d0 + d1) + (d2 + d3);
-                    float dc;
-                    if (METRIC == FGIM_L2SQ) dc = (float)(n2[wi] + n2[t] - 2u * dot);
-                    else if (METRIC == FGIM_IP) dc = delta_finish<FGIM_IP>((float)dot, 1.f);
-                    else dc = delta_finish<FGIM_COSINE>((float)dot, __fmul_rn(invs[wi], invs[t]));
-                    occ |= rule_occludes(rule, duv, dist[u * k + wi], dc);
-                }
-            }
-            keep = !__any_sync(kFull, occ);
-        }
-        if (keep) {
-            if (lane == 0) kept[nk] = t;
-            ++nk;
-            __syncwarp();
-        }
-    }
-    for (int s = lane; s < R; s += 32) {
-        if (s < nk) {
-            e_ids[u * R + s] = cidv[kept[s]];
-            e_dist[u * R + s] = dist[u * k + kept[s]];
-        } else {
-            e_ids[u * R + s] = -1;
-            e_dist[u * R + s] = __int_as_float(0x7f800000);
-        }
-    }
-    if (lane == 0) e_cnt[u] = nk;
-}
-
-cudaError_t launch_prune(const float* X, const uint8_t* X8, const float* inv_norm, long long N, int d, int metric,
-                         const fgim_knng& g, const int32_t* T, int R, PruneRule rule, int32_t* e_ids, float* e_dist,
-                         int32_t* e_cnt, int* status, cudaStream_t s) {
-    const long long nrows = g.n;   // lists to prune (ids range over 0 .. N - 1)
-    if (nrows <= 0) return cudaSuccess;
-    const int k = g.k;
-    if (X8 && byte_rows_ok(d) && k <= 64) {
-        const int wpb = 4;
-        const size_t smem = prune_bytes_per_warp(k, d) * wpb;
-        cudaError_t e = cudaSuccess;
-#define FGIM_LAUNCH_PB(MT)                                                                                        \
-    do {                                                                                                          \
-        e = cudaFuncSetAttribute(k_prune_bytes<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);     \
-        if (e != cudaSuccess) break;                                                                              \
-        LaunchScope ls("k_prune", s);                                                                             \
-        k_prune_bytes<MT><<<(unsigned)cdivl(nrows, wpb), wpb * 32, smem, s>>>(X8, inv_norm, N, nrows, d, k, g.ids, g.dist, T, \
-                                                                          R, rule, e_ids, e_dist, e_cnt, status);\
-        e = cudaGetLastError();                                                                                   \
-    } while (0)
-        if (metric == FGIM_L2SQ) FGIM_LAUNCH_PB(FGIM_L2SQ);
-        else if (metric == FGIM_IP) FGIM_LAUNCH_PB(FGIM_IP);
-        else FGIM_LAUNCH_PB(FGIM_COSINE);
-#undef FGIM_LAUNCH_PB
-        return e;
-    }
-    if (d > 128) {
-        const int wpb = 4;
-        const size_t smem = (size_t)wpb * 2 * k * sizeof(int32_t);
-        cudaError_t e = cudaSuccess;
-#define FGIM_LAUNCH_PW(MT)                                                                                        \
-    do {                                                                                                          \
-        LaunchScope ls("k_prune", s);                                                                             \
-        k_prune_wide<MT><<<(unsigned)cdivl(nrows, wpb), wpb * 32, smem, s>>>(X, inv_norm, N, nrows, d, k, g.ids, g.dist, T, R,  \
-                                                                         rule, e_ids, e_dist, e_cnt, status);   \
-        e = cudaGetLastError();                                                                                   \
-    } while (0)
-        if (metric == FGIM_L2SQ) FGIM_LAUNCH_PW(FGIM_L2SQ);
-        else if (metric == FGIM_IP) FGIM_LAUNCH_PW(FGIM_IP);
-        else FGIM_LAUNCH_PW(FGIM_COSINE);
-#undef FGIM_LAUNCH_PW
-        return e;
-    }
-    const int wpb = 2;
-    const size_t staged = ((size_t)k * (d + 4) * 4 + (size_t)k * 12 + 16 + 15) & ~(size_t)15;
-    const size_t unstaged = ((size_t)k * 12 + 16 + 15) & ~(size_t)15;
-    const bool stage = staged * wpb <= 160 * 1024;
-    const size_t smem = (stage ? staged : unstaged) * wpb;
-    cudaError_t e = cudaSuccess;
-#define FGIM_LAUNCH_P(MT, ST)                                                                                     \
-    do {                                                                                                          \
-        e = cudaFuncSetAttribute(k_prune<MT, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);       \
-        if (e != cudaSuccess) break;                                                                              \
-        LaunchScope ls("k_prune", s);                                                                             \
-        k_prune<MT, ST><<<(unsigned)cdivl(nrows, wpb), wpb * 32, smem, s>>>(X, inv_norm, N, nrows, d, k, g.ids, g.dist, T, R, \
-                                                                        rule, e_ids, e_dist, e_cnt, status);    \
-        e = cudaGetLastError();                                                                                   \
-    } while (0)
-    if (stage) {
-        if (metric == FGIM_L2SQ) FGIM_LAUNCH_P(FGIM_L2SQ, true);
-        else if (metric == FGIM_IP) FGIM_LAUNCH_P(FGIM_IP, true);
-        else FGIM_LAUNCH_P(FGIM_COSINE, true);
-    } else {
-        if (metric == FGIM_L2SQ) FGIM_LAUNCH_P(FGIM_L2SQ, false);
-        else if (metric == FGIM_IP) FGIM_LAUNCH_P(FGIM_IP, false);
-        else FGIM_LAUNCH_P(FGIM_COSINE, false);
-    }
-#undef FGIM_LAUNCH_P
-    return e;
-}
 
 // ---------------------------------------------------------------------------- reverse insertion
 __global__ void k_e_count(const int32_t* __restrict__ e_ids, long long total, int32_t* __restrict__ cnt) {

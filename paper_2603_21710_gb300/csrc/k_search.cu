@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(128, sizeof(RT) == 1 ? 8 : SMALLD ? 5 : 3) k_s
         if (METRIC == FGIM_COSINE) qinv = qids ? inv_norm[qids[qi]] : q_inv[qi];
         const Query qr = load_query<SMALLD, RT>(qsrc, reinterpret_cast<float*>(base + lay.q), d, lane);
         const int ent = qentry ? qentry[qi] : entry;   // per-query entries (the HNSW descent's result)
-        const int np = beam_search<METRIC, SMALLD, RT, MAXS>(Xr, inv_norm, graph, R, (int)n, ent, 0, qr, qinv, d, L, pool,
+        const int np = beam_search<METRIC, SMALLD, RT, MAXS, false>(Xr, inv_norm, graph, R, (int)n, ent, 0, qr, qinv, d, L, pool,
                                                              ht, htbits, scratch, ctr, status);
         for (int s = lane; s < topk; s += 32) {
             if (s < np) {
