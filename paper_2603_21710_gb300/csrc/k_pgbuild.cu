@@ -98,6 +98,8 @@ __global__ void k_pg_rev_fill(const int32_t* __restrict__ rows, long long b, int
     rev[off[v] + atomicAdd(fill + v, 1)] = mkkey(e_dist[i], rows[bi]);
 }
 
+constexpr int kMergeCap = 128;   // the longest list warp_merge can hold
+
 // Per target v (warp per target): its list and its new reverse edges in ascending (distance, id);
 // at most M of them stay as they are, more go to the overflow lists for the heuristic.
 __global__ void __launch_bounds__(128) k_pg_rev_merge(const int32_t* __restrict__ targets, long long nt,
@@ -115,13 +117,37 @@ __global__ void __launch_bounds__(128) k_pg_rev_merge(const int32_t* __restrict_
     const int32_t v = targets[ti];
     uint64_t* list = reinterpret_cast<uint64_t*>(smem) + (size_t)warp * W;
     const int c0 = cnt[v];
+    const long long b0 = off[v], m = off[v + 1] - off[v];
+    if (c0 + m > kMergeCap) {
+        // a hub: more keys than a merged list may hold (the keys are distinct and at most W, more than M):
+        // each key's place is the number of smaller ones, written straight to the overflow list
+        const int total = (int)(c0 + m);
+        for (int s = lane; s < total; s += 32)
+            list[s] = s < c0 ? mkkey(nd[(long long)v * M + s], nbr[(long long)v * M + s]) : rev[b0 + (s - c0)];
+        __syncwarp();
+        int slot = 0;
+        if (lane == 0) slot = atomicAdd(n_ov, 1);
+        slot = __shfl_sync(kFull, slot, 0);
+        for (int s = lane; s < total; s += 32) {
+            const uint64_t key = list[s];
+            int r = 0;
+            for (int q = 0; q < total; ++q) r += list[q] < key ? 1 : 0;
+            ov_ids[(long long)slot * W + r] = key_id(key);
+            ov_dist[(long long)slot * W + r] = key_dist(key);
+        }
+        for (int s = total + lane; s < W; s += 32) {
+            ov_ids[(long long)slot * W + s] = -1;
+            ov_dist[(long long)slot * W + s] = __int_as_float(0x7f800000);
+        }
+        if (lane == 0) ov_tgt[slot] = v;
+        return;
+    }
     int n = 0;
     for (int s0 = 0; s0 < c0; s0 += 32) {
         const uint64_t key = s0 + lane < c0 ? mkkey(nd[(long long)v * M + s0 + lane], nbr[(long long)v * M + s0 + lane])
                                             : kEmptyKey;
         n = warp_merge<false>(list, nullptr, n, W, key, 0);
     }
-    const long long b0 = off[v], m = off[v + 1] - off[v];
     for (long long s0 = 0; s0 < m; s0 += 32) {
         const uint64_t key = s0 + lane < m ? rev[b0 + s0 + lane] : kEmptyKey;
         n = warp_merge<false>(list, nullptr, n, W, key, 0);
