@@ -527,10 +527,10 @@ static void stage_a(Ctx& c, const Problem& P, const fgim_params* p, int h, fgim_
                           F ? F->phi : nullptr, F ? F->src : nullptr, F ? F->Nv : P.N, P.Xh));
 }
 
-static void refine_pass(Ctx& c, const Problem& P, const fgim_params* p, fgim_knng* g, fgim_stats* st) {
-    StageRange range("fgim stage b: Visit + Update (Alg. 3)");
+// The buffers of the refinement passes of a merge, and the join's operand (made by the first pass).
+// All passes use the same: each pass resets what it reads.
+static RefineBuffers refine_buffers(Ctx& c, const Problem& P, const fgim_params* p, int k) {
     const long long N = P.N;
-    const int k = g->k;
     const int rev_cap = resolve_rev_cap(p);
     RefineBuffers b;
     std::memset(&b, 0, sizeof(b));
@@ -587,21 +587,47 @@ static void refine_pass(Ctx& c, const Problem& P, const fgim_params* p, fgim_knn
         b.sparse_nn = o >= 0 ? o : kSparseNNDefault;
     }
     b.X8 = P.X8;
-    b.Xb = nullptr;
-    b.fp8 = false;
-    if (p->join_filter == FGIM_PREC_BF16 && P.d % 16 == 0) {
-        b.Xb = c.alloc<__nv_bfloat16>(N * P.d);
-        b.tcm = c.alloc<float4>(N);
-        ck(launch_prep_bf16(P.X, N, P.d, reinterpret_cast<__nv_bfloat16*>(b.Xb), b.tcm, c.s));
-    } else if (p->join_filter == FGIM_PREC_FP8E4M3 && P.d % 32 == 0) {
-        // E4M3 rows (one byte per coordinate) with one scale per vector, addressed like BF16 pairs
-        uint8_t* Xq = c.alloc<uint8_t>(N * P.d);
-        b.tcm = c.alloc<float4>(N);
-        ck(launch_prep_fp8(P.X, N, P.d, Xq, b.tcm, c.s));
-        b.Xb = reinterpret_cast<__nv_bfloat16*>(Xq);
-        b.fp8 = true;
-    }
+    return b;
+}
 
+// The copy of the vectors that the tensor-core tile of Update reads: E4M3 when asked for and fine
+// enough for these lists (decided on the lists of the first pass), else BF16 where that is exact, else FP16.
+static void join_operand(Ctx& c, const Problem& P, const fgim_knng* g, RefineBuffers& b) {
+    const long long N = P.N;
+    if (b.join_filter == FGIM_PREC_FP32 || b.Xb) return;
+    b.tcm = c.alloc<float4>(N);
+    if (b.join_filter == FGIM_PREC_FP8E4M3) {
+        b.dp = (P.d + 31) / 32 * 32;
+        uint8_t* Xq = c.alloc<uint8_t>(N * b.dp);
+        int* coarse = c.alloc<int>(1);
+        ck(launch_prep_fp8(P.X, N, P.d, b.dp, Xq, b.tcm, c.s));
+        ck(launch_fp8_coarse(*g, b.tcm, P.inv, P.metric, coarse, c.s));
+        if (2LL * c.read_i32(coarse) <= N) {
+            b.Xb = Xq;   // one byte per coordinate, addressed like 16-bit pairs
+            b.fp8 = true;
+            return;
+        }
+    }
+    b.dp = (P.d + 15) / 16 * 16;
+    b.Xb = c.alloc<uint16_t>(N * b.dp);
+    if (!P.X8 && !P.Xh) {
+        int* not_bf16 = c.alloc<int>(1);
+        ck(launch_prep_f16(P.X, N, P.d, b.dp, b.Xb, b.tcm, not_bf16, c.s));
+        if (c.read_i32(not_bf16) != 0) {
+            b.f16 = true;
+            return;
+        }
+    }
+    ck(launch_prep_bf16(P.X, N, P.d, b.dp, b.Xb, b.tcm, c.s));
+}
+
+static void refine_pass(Ctx& c, const Problem& P, const fgim_params* p, fgim_knng* g, fgim_stats* st,
+                        RefineBuffers& b) {
+    StageRange range("fgim stage b: Visit + Update (Alg. 3)");
+    const long long N = P.N;
+    const int rev_cap = resolve_rev_cap(p);
+    const long long cap = b.prop_cap;
+    join_operand(c, P, g, b);
     ck(refine_visit(*g, rev_cap, b, c.s));
     ck(cudaMemsetAsync(b.pending, 0, N, c.s));
     ck(cudaMemsetAsync(b.prop_count, 0, sizeof(unsigned long long), c.s));
@@ -849,7 +875,8 @@ fgim_status fgim_refine_pass(const fgim_shard* shards, int32_t h, const fgim_par
         need(knng->n == total_n(shards, h) && knng->k >= 1 && knng->k <= FGIM_MAX_K, FGIM_EINVAL, "knng shape mismatch");
         Ctx c((cudaStream_t)stream);
         Problem P = make_problem(c, shards, h, params);
-        refine_pass(c, P, params, knng, &t_stats);
+        RefineBuffers b = refine_buffers(c, P, params, knng->k);
+        refine_pass(c, P, params, knng, &t_stats, b);
         c.finish(&t_stats);
     });
     end_call();
@@ -954,8 +981,10 @@ static void merge_impl(Ctx& c, const fgim_shard* shards, int32_t h, const fgim_p
     stage_a(c, P0, params, h, &g, masked ? &F : nullptr);
     const Problem P = masked ? compact_problem(c, P0, F, params) : P0;
     int32_t* T = c.alloc<int32_t>(N);
+    RefineBuffers b;
+    if (params->iters > 0) b = refine_buffers(c, P, params, k);
     for (int it = 0; it < params->iters; ++it) {
-        refine_pass(c, P, params, &g, &t_stats);
+        refine_pass(c, P, params, &g, &t_stats, b);
         repair(c, P, &g, T, &t_stats);
     }
     if (params->iters == 0) ck(launch_indegree(g.ids, N, k, T, false, nullptr, c.s));
@@ -1069,8 +1098,10 @@ static void merge_union(Ctx& c, const fgim_shard* const* shards, const int32_t* 
     ck(launch_cross_query(P.t, P.X, P.X8, P.inv, N, P.metric, k, Lmax, &g, c.ctr + 0, c.status, c.s, nullptr, nullptr,
                           N, P.Xh));
     int32_t* T = c.alloc<int32_t>(N);
+    RefineBuffers b;
+    if (p->iters > 0) b = refine_buffers(c, P, p, k);
     for (int it = 0; it < p->iters; ++it) {
-        refine_pass(c, P, p, &g, &t_stats);
+        refine_pass(c, P, p, &g, &t_stats, b);
         repair(c, P, &g, T, &t_stats);
     }
     if (p->iters == 0) ck(launch_indegree(g.ids, N, k, T, false, nullptr, c.s));

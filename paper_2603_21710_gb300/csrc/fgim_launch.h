@@ -94,11 +94,13 @@ struct RefineBuffers {
     bool fp8;                   // Xb holds E4M3 rows with per-vector scales (tcm.w) instead of BF16 rows
     int32_t* blist;
     long long blist_cap;
-    // tensor-core filter inputs: BF16 copy of the vectors and per row (|x|^2, bound on |x|,
-    // bound on the BF16 conversion error |bf(x) - x|, unused)
+    // tensor-core filter inputs: BF16, FP16 (f16) or E4M3 (fp8) copy of the vectors, rows of dp >= dim
+    // values, and per row (|x|^2, bound on |x|, bound on the conversion error, value of one unit)
     int join_filter;
     void* Xb;
     float4* tcm;
+    int dp;
+    bool f16;
     // the vectors as bytes when every coordinate is an integer in [0, 255], else nullptr
     const uint8_t* X8;
 };
@@ -108,11 +110,17 @@ cudaError_t refine_join(const ShardTable& t, const float* X, const float* inv_no
                         RefineBuffers& b, const int32_t* vlist, long long nv, unsigned long long* pairs,
                         unsigned long long* cands, int* status, cudaStream_t s);
 cudaError_t refine_merge(const fgim_knng& g, RefineBuffers& b, long long nprop, cudaStream_t s);
-cudaError_t launch_prep_fp8(const float* X, long long N, int d, uint8_t* Xq, float4* tcm, cudaStream_t s);
+cudaError_t launch_prep_fp8(const float* X, long long N, int d, int dp, uint8_t* Xq, float4* tcm, cudaStream_t s);
+// the lists for which the E4M3 tile's error bound is too coarse to decide much
+cudaError_t launch_fp8_coarse(const fgim_knng& g, const float4* tcm, const float* inv_norm, int metric, int* count,
+                              cudaStream_t s);
 // *out = some adjacency row of the input graphs repeats an id within a 32-entry chunk (uses
 // status[2] as scratch; synchronizes the stream)
 cudaError_t adjacency_has_repeats(const ShardTable& t, long long N, int* status, cudaStream_t s, bool* out);
-cudaError_t launch_prep_bf16(const float* X, long long N, int d, __nv_bfloat16* Xb, float4* tcm, cudaStream_t s);
+cudaError_t launch_prep_bf16(const float* X, long long N, int d, int dp, void* Xb, float4* tcm, cudaStream_t s);
+// *not_bf16 = some coordinate is not a BF16 value
+cudaError_t launch_prep_f16(const float* X, long long N, int d, int dp, void* Xb, float4* tcm, int* not_bf16,
+                            cudaStream_t s);
 cudaError_t launch_indegree(const int32_t* ids, long long N, int k, int32_t* T, bool clear_replaced, uint8_t* flags,
                             cudaStream_t s);
 // rounds rho0 .. rho0 + rounds - 1 of the Alg. 4 repair; ff[rho0 - 1] holds the first pending

@@ -562,14 +562,18 @@ __global__ void __launch_bounds__(kJThreads, 2) k_join_staged(
     if (threadIdx.x == 0) atomicAdd(cands_count, (unsigned long long)nc);
 }
 
-// ---- tensor-core filter (BF16 tcgen05 Gram tile), exact FP32 re-rank
+// ---- tensor-core filter (16-bit tcgen05 Gram tile), exact FP32 re-rank
 //
-// Per vertex v the candidate rows (BF16 copies) are staged in shared memory (K-major,
+// Per vertex v the candidate rows (16-bit copies) are staged in shared memory (K-major,
 // 128-byte swizzle) and one 128 x N x d tcgen05.mma tile (FP32 accumulation in TMEM) gives
-// D_ij ~ x_i . x_j for every pair of C_n x C. The filter value is
+// D_ij ~ x_i . x_j for every pair of C_n x C. The copies are BF16 where that is exact (byte rows,
+// BF16-stored vectors) and otherwise FP16 of the row scaled by a power of two that brings its largest
+// coordinate near 2^14: 11 significant bits instead of 8 at the same bytes, so the bound below is eight
+// times tighter and that many fewer pairs are left for the re-rank (300k unit-norm rows of d = 96: of 146 M
+// pairs BF16 left 16.9 M, for 0.18 M proposals). The filter value is
 //   L2: n2_i + n2_j - 2 D_ij,  IP: 1 - D_ij,  cosine: 1 - D_ij * inv_i * inv_j,
 // and a pair direction survives when the value minus a bound on its error can still beat
-// the target's worst key. The bound (Cauchy-Schwarz on the BF16 conversion errors e = bf(x)
+// the target's worst key. The bound (Cauchy-Schwarz on the conversion errors e = copy(x)
 // - x, plus the FP32 accumulation and rounding terms of Higham's bound with g = (d + 16) u):
 //   |D - x_i.x_j| <= |e_i||x_j| + |x_i||e_j| + |e_i||e_j| + g (|x_i| + |e_i|)(|x_j| + |e_j|).
 // On integer-valued data the conversion is exact (e = 0) and the bound is tiny. Survivors are
@@ -581,17 +585,19 @@ constexpr int kTCPropBuf = 256;    // proposals buffered per CTA
 constexpr int kTCKChunk = 128;     // dimensions staged per K chunk of the Gram tile
 
 
-__global__ void k_prep_bf16(const float* __restrict__ X, long long N, int d, __nv_bfloat16* __restrict__ Xb,
+// rows of dp >= d entries (zeros past d); tcm = (|x|^2, bound on |x|, bound on |copy - x|, value of
+// one unit of the copy)
+__global__ void k_prep_bf16(const float* __restrict__ X, long long N, int d, int dp, __nv_bfloat16* __restrict__ Xb,
                             float4* __restrict__ tcm) {
     const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (row >= N) return;
     const float* x = X + row * d;
-    __nv_bfloat16* xb = Xb + row * d;
+    __nv_bfloat16* xb = Xb + row * dp;
     float s = 0.f, se = 0.f;
     bool inexact = false;
-    for (int c = lane; c < d; c += 32) {
-        const float v = x[c];
+    for (int c = lane; c < dp; c += 32) {
+        const float v = c < d ? x[c] : 0.f;
         const __nv_bfloat16 b = __float2bfloat16_rn(v);
         xb[c] = b;
         const float e = __bfloat162float(b) - v;
@@ -609,16 +615,60 @@ __global__ void k_prep_bf16(const float* __restrict__ X, long long N, int d, __n
         // |e| == 0 exactly when the BF16 row equals the FP32 row; squares of conversion errors
         // below 2^-75 can underflow, so an inexact row never reports less than 1e-18
         const float en = inexact ? fmaxf(sqrtf(se) * 1.0001f, 1e-18f) : 0.f;
-        tcm[row] = make_float4(s, sqrtf(s) * 1.0001f, en, 0.f);
+        tcm[row] = make_float4(s, sqrtf(s) * 1.0001f, en, 1.f);
     }
+}
+
+// FP16 rows scaled by 2^t (exact), t such that the largest coordinate's exponent becomes 14 (t within
+// +-60, so that the product of two unscaling factors stays finite; conversion saturates); *not_bf16 |= 1
+// unless every coordinate is a BF16 value
+__global__ void k_prep_f16(const float* __restrict__ X, long long N, int d, int dp, __half* __restrict__ Xb,
+                           float4* __restrict__ tcm, int* not_bf16) {
+    const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (row >= N) return;
+    const float* x = X + row * d;
+    float amax = 0.f;
+    for (int c = lane; c < d; c += 32) amax = fmaxf(amax, fabsf(x[c]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(kFull, amax, o));
+    const int ex = (int)(__float_as_uint(amax) >> 23) - 127;   // floor(log2 amax); zeros and denormals: -127
+    const int t = min(max(14 - ex, -60), 60);
+    const float up = __uint_as_float((uint32_t)(127 + t) << 23), down = __uint_as_float((uint32_t)(127 - t) << 23);
+    __half* xb = Xb + row * dp;
+    float s = 0.f, se = 0.f;
+    bool inexact = false;
+    uint32_t low = 0u;
+    for (int c = lane; c < dp; c += 32) {
+        const float v = c < d ? x[c] : 0.f;
+        low |= __float_as_uint(v) & 0xffffu;
+        const float w = v * up;
+        const __half h = __float2half_rn(fminf(fmaxf(w, -65504.f), 65504.f));
+        xb[c] = h;
+        const float e = fmaf(down, __half2float(h), -v);   // one rounding
+        inexact |= e != 0.f || w != w;
+        s = fmaf(v, v, s);
+        se = fmaf(e, e, se);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(kFull, s, o);
+        se += __shfl_xor_sync(kFull, se, o);
+    }
+    inexact = __any_sync(kFull, inexact);
+    if (lane == 0) {
+        const float en = inexact ? fmaxf(sqrtf(se) * 1.0001f, 1e-18f) : 0.f;
+        tcm[row] = make_float4(s, sqrtf(s) * 1.0001f, en, down);
+    }
+    if (__any_sync(kFull, low != 0u) && lane == 0 && *not_bf16 == 0) *not_bf16 = 1;
 }
 
 // FP8 E4M3 rows with one scale per vector: s = amax |x| / 448 (1 for an all-zero row),
 // q = saturating round-to-nearest E4M3 of x / s; the MMA forms sum q_a q_b and the filter takes
 // s_a s_b times it. tcm = (|x|^2, bound on |x|, bound on |x - s q|, s); the conversion error is
 // what the filter's bound is built from (every row counts as inexact).
-__global__ void k_prep_fp8(const float* __restrict__ X, long long N, int d, __nv_fp8_storage_t* __restrict__ Xq,
-                           float4* __restrict__ tcm) {
+__global__ void k_prep_fp8(const float* __restrict__ X, long long N, int d, int dp,
+                           __nv_fp8_storage_t* __restrict__ Xq, float4* __restrict__ tcm) {
     const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (row >= N) return;
@@ -628,10 +678,10 @@ __global__ void k_prep_fp8(const float* __restrict__ X, long long N, int d, __nv
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(kFull, amax, o));
     const float sc = amax > 0.f ? amax / 448.f : 1.f;
-    __nv_fp8_storage_t* xq = Xq + row * d;
+    __nv_fp8_storage_t* xq = Xq + row * dp;
     float s = 0.f, se = 0.f;
-    for (int c = lane; c < d; c += 32) {
-        const float v = x[c];
+    for (int c = lane; c < dp; c += 32) {
+        const float v = c < d ? x[c] : 0.f;
         const __nv_fp8_storage_t q = __nv_cvt_float_to_fp8(v / sc, __NV_SATFINITE, __NV_E4M3);
         xq[c] = q;
         const float dq = __half2float(__half(__nv_cvt_fp8_to_halfraw(q, __NV_E4M3)));
@@ -647,17 +697,54 @@ __global__ void k_prep_fp8(const float* __restrict__ X, long long N, int d, __nv
     if (lane == 0) tcm[row] = make_float4(s, sqrtf(s) * 1.0001f, fmaxf(sqrtf(se) * 1.001f, 1e-18f), sc);
 }
 
-cudaError_t launch_prep_fp8(const float* X, long long N, int d, uint8_t* Xq, float4* tcm, cudaStream_t s) {
+cudaError_t launch_prep_fp8(const float* X, long long N, int d, int dp, uint8_t* Xq, float4* tcm, cudaStream_t s) {
     if (N <= 0) return cudaSuccess;
     LaunchScope ls("k_prep_fp8", s);
-    k_prep_fp8<<<(unsigned)cdivll(N * 32, 256), 256, 0, s>>>(X, N, d, reinterpret_cast<__nv_fp8_storage_t*>(Xq), tcm);
+    k_prep_fp8<<<(unsigned)cdivll(N * 32, 256), 256, 0, s>>>(X, N, d, dp, reinterpret_cast<__nv_fp8_storage_t*>(Xq), tcm);
     return cudaGetLastError();
 }
 
-cudaError_t launch_prep_bf16(const float* X, long long N, int d, __nv_bfloat16* Xb, float4* tcm, cudaStream_t s) {
+cudaError_t launch_prep_bf16(const float* X, long long N, int d, int dp, void* Xb, float4* tcm, cudaStream_t s) {
     if (N <= 0) return cudaSuccess;
     LaunchScope ls("k_prep_bf16", s);
-    k_prep_bf16<<<(unsigned)cdivll(N * 32, 256), 256, 0, s>>>(X, N, d, Xb, tcm);
+    k_prep_bf16<<<(unsigned)cdivll(N * 32, 256), 256, 0, s>>>(X, N, d, dp, static_cast<__nv_bfloat16*>(Xb), tcm);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_prep_f16(const float* X, long long N, int d, int dp, void* Xb, float4* tcm, int* not_bf16,
+                            cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(not_bf16, 0, sizeof(int), s);
+    if (e != cudaSuccess || N <= 0) return e;
+    LaunchScope ls("k_prep_f16", s);
+    k_prep_f16<<<(unsigned)cdivll(N * 32, 256), 256, 0, s>>>(X, N, d, dp, static_cast<__half*>(Xb), tcm, not_bf16);
+    return cudaGetLastError();
+}
+
+// *count += the vertices whose E4M3 row's error bound for a pair of rows like it, twice |e| |x| in units of
+// the inner product, is more than 1/8 of the distance of its list's last entry: there the E4M3
+// tile decides next to nothing (36k rows of d = 960: it left 150 M of 162 M pairs to the re-rank)
+__global__ void k_fp8_coarse(const int32_t* __restrict__ ids, const float* __restrict__ dist, long long N, int k,
+                             const float4* __restrict__ tcm, const float* __restrict__ inv_norm, int metric,
+                             int* __restrict__ count) {
+    const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    bool coarse = false;
+    if (v < N && ids[v * k + k - 1] >= 0) {
+        const float4 m = tcm[v];
+        float b = 2.f * m.z * m.y;
+        if (metric == FGIM_L2SQ) b *= 2.f;
+        else if (metric == FGIM_COSINE) b *= inv_norm[v] * inv_norm[v];
+        coarse = b > 0.125f * fabsf(dist[v * k + k - 1]);
+    }
+    const unsigned m = __ballot_sync(kFull, coarse);
+    if ((threadIdx.x & 31) == 0 && m) atomicAdd(count, __popc(m));
+}
+
+cudaError_t launch_fp8_coarse(const fgim_knng& g, const float4* tcm, const float* inv_norm, int metric, int* count,
+                              cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int), s);
+    if (e != cudaSuccess || g.n <= 0) return e;
+    LaunchScope ls("k_fp8_coarse", s);
+    k_fp8_coarse<<<(unsigned)cdivll(g.n, 256), 256, 0, s>>>(g.ids, g.dist, g.n, g.k, tcm, inv_norm, metric, count);
     return cudaGetLastError();
 }
 
@@ -722,13 +809,13 @@ __host__ __device__ inline TCLayout tc_layout(int cm, int d) {
 }
 
 // One CTA per vertex v (vlist[blockIdx.x]); C_n = the first nn candidates, C = all nc.
-// FP8: the staged operand holds E4M3 rows with one scale per vector (k_prep_fp8) instead of BF16
-// rows; each Gram entry is then scaled by the two vectors' scales, the filter's bound takes their
-// conversion errors, and the re-rank always reads the FP32 rows.
+// Xb: the staged operand, rows of dp BF16 or FP16 values, or (FP8) of dp E4M3 ones; each row has a
+// factor (tcm.w, 1 for BF16), so each Gram entry is scaled by the two rows' factors, and the filter's bound
+// takes their conversion errors.
 template <int METRIC, bool BYTES, bool LARGE, bool FP8>
 __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
-    ShardTable t, const float* __restrict__ X, const __nv_bfloat16* __restrict__ Xb, const uint8_t* __restrict__ X8,
-    const float4* __restrict__ tcm, const float* __restrict__ inv_norm, int k, const int32_t* __restrict__ ids,
+    ShardTable t, const float* __restrict__ X, const __nv_bfloat16* __restrict__ Xb, int dp, bool f16,
+    const uint8_t* __restrict__ X8, const float4* __restrict__ tcm, const float* __restrict__ inv_norm, int k, const int32_t* __restrict__ ids,
     const uint64_t* __restrict__ wk, const int32_t* __restrict__ cand, const int32_t* __restrict__ nn_arr, const int32_t* __restrict__ no_arr, int cmax,
     int cm, uint32_t tmem_cols, const int32_t* __restrict__ vlist, int32_t* __restrict__ prop_tgt,
     uint64_t* __restrict__ prop_key, unsigned long long* prop_count, long long prop_cap, uint8_t* __restrict__ pending,
@@ -753,11 +840,11 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
         return;
     }
     const int d = t.dim;
-    const int du = FP8 ? d / 2 : d;   // row length in 2-byte staging units (an E4M3 pair per unit)
+    const int du = FP8 ? dp / 2 : dp;   // staged row in 2-byte units (a 16-bit value or an E4M3 pair; zeros past d)
     const TCLayout L = tc_layout(cm, du);
     unsigned char* op = smem + L.op;
-    float4* meta = reinterpret_cast<float4*>(smem + L.meta);   // n2, |x| bound, |e| bound, cosine 1/|x|
-    float4* colf = reinterpret_cast<float4*>(smem + L.colf);   // P, worst distance, shard (bits), -
+    float4* meta = reinterpret_cast<float4*>(smem + L.meta);   // n2, y, z (see the filter), cosine 1/|x|
+    float4* colf = reinterpret_cast<float4*>(smem + L.colf);   // P, worst distance, shard (bits), factor
     uint64_t* thr = reinterpret_cast<uint64_t*>(smem + L.thr);
     int32_t* cid = reinterpret_cast<int32_t*>(smem + L.cid);
     int2* hkv = reinterpret_cast<int2*>(smem + L.hkv);   // (candidate id or -1, its index)
@@ -780,10 +867,10 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
     const int npad = ((nc + 15) / 16) * 16;   // MMA N
     const int kcp_sh = (kcp & (kcp - 1)) == 0 ? __ffs(kcp) - 1 : -1;   // shift for / kcp when a power of two
     const int nch = (kc + kcp - 1) / kcp;   // K chunks
-    const float g = (float)(d + 16) * 5.9604645e-8f;
-    // squared L2 on exactly converted rows: lo = P_i + P_j - 2 D_ij with P = (1 - Cf) |x|^2
-    // lies below (value - bound) of the general test (see the filter)
-    const float Cf = 1.2f * (4.001f * g + 12.01f * 5.9604645e-8f);
+    constexpr float u32 = 5.9604645e-8f;   // 2^-24
+    const float g = (float)(d + 16) * u32;
+    // P = (1 - Cf) |x|^2 of the squared-L2 tests (see the filter)
+    const float Cf = BYTES ? 1.2f * (4.001f * g + 12.01f * u32) : 1.1f * (2.f * u32 + g) + 1.1f * g + 16.f * u32;
 
     if (tid < nc) cid[tid] = cA;
     if (tid + NT < nc) cid[tid + NT] = cB;
@@ -865,9 +952,14 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
         thr[i] = wkey;
         if (m.z != 0.f) atomicOr(misc + 2, 1);
         colf[i] = make_float4((1.f - Cf) * m.x, wkey == kEmptyKey ? __int_as_float(0x7f800000) : key_dist(wkey),
-                              __int_as_float(shard_of(t, c)), FP8 ? m.w : 0.f);   // w: the E4M3 scale
-        m.w = inv;
-        meta[i] = m;
+                              __int_as_float(shard_of(t, c)), METRIC == FGIM_COSINE ? m.w * inv : m.w);
+        float y = m.y, e = m.z;
+        if (METRIC == FGIM_COSINE) {
+            y *= inv;
+            e *= inv;
+        }
+        const float gz = METRIC == FGIM_L2SQ ? g + 4.1f * u32 : 2.01f * g;
+        meta[i] = make_float4(m.x, y, e + gz * (y + e), inv);
     };
     if (tid < nc) put_meta(tid, cA, wkA, mA, invA);
     if (tid + NT < nc) put_meta(tid + NT, cB, wkB, mB, invB);
@@ -931,10 +1023,9 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
-    // every row converted exactly to BF16 and the whole row fits one staged chunk: the re-rank
-    // may read the staged tile instead of the FP32 rows
-    const bool exact = !FP8 && misc[2] == 0 && nch == 1;
-    const bool exact_rows = !FP8 && misc[2] == 0;
+    // every row converted exactly to BF16 and the whole row fits one staged chunk: the re-rank may read
+    // the staged tile instead of the FP32 rows
+    const bool exact = !FP8 && !f16 && misc[2] == 0 && nch == 1;
     bool ok_mma = true;
     for (int ch = 0; ch < nch && ok_mma; ++ch) {
         if (ch > 0) {
@@ -948,12 +1039,13 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
             tc::fence_after_sync();
         }
         if (tid == 0) {
-            const uint32_t idesc = FP8 ? tc::idesc_e4m3(128, LARGE ? npad : 128) : tc::idesc_bf16(128, LARGE ? npad : 128);
+            const int n_cols = LARGE ? npad : 128;
+            const uint32_t idesc = FP8 ? tc::idesc_e4m3(128, n_cols) : f16 ? tc::idesc_f16(128, n_cols) : tc::idesc_bf16(128, n_cols);
             const uint32_t base = tc::smem_u32(op);
             for (int s = 0; s < L.dpad / 16; ++s) {   // 32 bytes of every row per MMA
                 const uint64_t desc = tc::smem_desc_sw128(base + (uint32_t)((s >> 2) * rows * 128 + (s & 3) * 32));
                 if (FP8) tc::mma_e4m3(tmem, desc, desc, idesc, (ch > 0 || s > 0) ? 1u : 0u);
-                else tc::mma_bf16(tmem, desc, desc, idesc, (ch > 0 || s > 0) ? 1u : 0u);
+                else tc::mma_f16(tmem, desc, desc, idesc, (ch > 0 || s > 0) ? 1u : 0u);
             }
             tc::commit_to(mbar);
         }
@@ -977,11 +1069,20 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
     bool rows_ready = !BYTES;
 
     // Filter. A pair survives when lo, a lower bound of its exact value, can still beat the
-    // worst key of a list it is not already in. General test: lo = value - bound with the
-    // bound of the file comment (cs term: e_i x_j + e_j (x_i + e_i) + g (x_i + e_i)(x_j + e_j)).
-    // Squared L2 on exactly converted rows (e = 0): with s2 = n2_i + n2_j, 2 x_i x_j <= 1.0002 s2
-    // and |D| <= (1 + g) x_i x_j, the general bound is at most 1.1 s2 (4.001 g + 12.01 u); Cf
-    // adds margin for the rounding of P_i + P_j - 2 D, so lo = P_i + P_j - 2 D is lower still.
+    // worst key of a list it is not already in. With T = D times both rows' factors (cosine: and inverse
+    // norms), x, e the bounds on a row's norm and conversion error (cosine: times its inverse norm), the error
+    // of T is at most cs = e_i x_j + (x_i + e_i) (e_j + g (x_j + e_j)) and |T| <= 1.01 (x_i + e_i)(x_j + e_j):
+    //   IP, cosine: value 1 - T, bound 1.1 (cs + g |1 - T|) + rounding <= 1.1 (e_i x_j + (x_i + e_i)
+    //     (e_j + 2.01 g (x_j + e_j)) + g) + 10 u, that is lo = K - T - A_i y_j - B_i z_j with y = x, A = 1.1 e,
+    //     B = 1.1 (x + e), z = e + 2.01 g (x + e);
+    //   squared L2: value s2 - 2 T with s2 = n2_i + n2_j, bound 1.1 (2 cs + g s2 + (2 u + g) |value| + 4 u
+    //     (s2 + 2 |T|)): lo = P_i + P_j - 2 (1 - c1) T - A_i y_j - B_i z_j with c1 = 1.1 (2 u + g), P = (1 - c1 -
+    //     1.1 g - 16 u) n2 (16 u: the 4 u term and the rounding of this expression), A = 2.2 e, B = 2.2 (x + e),
+    //     z = e + (g + 4.1 u)(x + e). (A negative value is within the bound of zero, where c1 times it is
+    //     covered by the factor 1.1.)
+    // Byte rows (squared L2, e = 0): with s2 = n2_i + n2_j, 2 x_i x_j <= 1.0002 s2 and |D| <= (1 + g) x_i x_j,
+    // the general bound is at most 1.1 s2 (4.001 g + 12.01 u); Cf adds margin for the rounding of
+    // P_i + P_j - 2 D, so lo = P_i + P_j - 2 D is lower still.
     //
     // Pairs are {i, j} with i < nn (new) and i < j < nc. Both MMA operands are the staged
     // tile, so D is symmetric and the lane of TMEM row r (candidate a) evaluates the pairs
@@ -992,37 +1093,26 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
     const int a = LARGE ? r : tc_cand(r);    // this lane's candidate
     const bool r_ok = a < nc;
     const float4 fr = r_ok ? colf[a] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float Pr = fr.x, tdr = fr.y, sr = fr.w;
+    const float Pr = fr.x, tdr = fr.y, wr = fr.w;
     const int shr = r_ok ? __float_as_int(fr.z) : -1;
     const float4 mr = r_ok ? meta[a] : make_float4(0.f, 0.f, 0.f, 1.f);
-    const float n2r = mr.x, xr = mr.y, er = mr.z, cr = mr.w;
-    const float xer = xr + er;
-    const bool fast = METRIC == FGIM_L2SQ && (BYTES || exact_rows);
+    const float cAB = METRIC == FGIM_L2SQ ? 2.2f : 1.1f;
+    const float er = !BYTES && r_ok ? tcm[cid[a]].z * (METRIC == FGIM_COSINE ? mr.w : 1.f) : 0.f;
+    const float Ar = cAB * er, Br = cAB * (mr.y + er);
+    const float c1 = 1.1f * (2.f * u32 + g);
+    const float cT = METRIC == FGIM_L2SQ ? 2.f * (1.f - c1) : 1.f;
+    const float K = 1.f - 1.1f * g - 10.f * u32;
     const unsigned lt = (1u << lane) - 1u;
     unsigned long long my_pairs = 0;
     // TMEM address of this warp's lane quarter
     auto trow_of = [&](int w) -> uint32_t { return tmem + ((uint32_t)(32 * (w & 3)) << 16); };
     // lo, a lower bound of the exact value of pair {a, b}, from its Gram entry
     auto lower = [&](int b, float dot, const float4& cc) -> float {
-        if (FP8) dot = dot * (sr * cc.w);   // sum q_a q_b -> s_a s_b sum q_a q_b (two roundings, in the bound)
-        if (fast) return fmaf(-2.f, dot, Pr + cc.x);
+        if (BYTES && METRIC == FGIM_L2SQ) return fmaf(-2.f, dot, Pr + cc.x);
         const float4 mc = meta[b];
-        const float cs = er * mc.y + mc.z * xer + g * xer * (mc.y + mc.z);
-        float val, bound;
-        if (METRIC == FGIM_L2SQ) {
-            const float s2 = n2r + mc.x;
-            val = s2 - 2.f * dot;
-            bound = 1.1f * (2.f * cs + g * s2 + (2.f * 5.9604645e-8f + g) * fabsf(val) +
-                            4.f * 5.9604645e-8f * (s2 + 2.f * fabsf(dot)));
-        } else if (METRIC == FGIM_IP) {
-            val = 1.f - dot;
-            bound = 1.1f * (cs + g * fabsf(val)) + 2.4e-7f;
-        } else {
-            const float ccv = cr * mc.w;
-            val = 1.f - dot * ccv;
-            bound = 1.1f * (cs * ccv + g * fabsf(val)) + 4.8e-7f;
-        }
-        return val - bound;
+        const float T = dot * (wr * cc.w);
+        const float base = METRIC == FGIM_L2SQ ? Pr + cc.x : K;
+        return fmaf(-Br, mc.z, fmaf(-Ar, mc.y, fmaf(-cT, T, base)));
     };
     // survivors go to this warp's own segment of the queue (a register count, no atomics)
     const int seg = kTCQueue / NW;
@@ -1738,7 +1828,7 @@ cudaError_t refine_join(const ShardTable& t, const float* X, const float* inv_no
     for (int q = 0; q < kOut; ++q) hb[q] = b.host_i32[q];
     const int32_t cm = hb[0], cmn = hb[1];
     if (cm < 2) return cudaSuccess;
-    const int du = b.fp8 ? t.dim / 2 : t.dim;   // staged row length in 2-byte units
+    const int du = b.fp8 ? b.dp / 2 : b.dp;   // staged row length in 2-byte units
     bool use_tc = b.join_filter != 1 && b.Xb && du % 16 == 0 && cmn <= 128 && cm <= 256;
     if (use_tc)
         for (int q = 0; q < kTCLists; ++q)
@@ -1766,7 +1856,7 @@ cudaError_t refine_join(const ShardTable& t, const float* X, const float* inv_no
         if (e != cudaSuccess) break;                                                                              \
         LaunchScope ls("k_join", s);                                                                              \
         k_join_tc<MT, BY, LG, F8><<<(unsigned)count, (BY) ? 256 : kTCThreads, smem, s>>>(                           \
-            t, X, reinterpret_cast<const __nv_bfloat16*>(b.Xb), b.X8, b.tcm, inv_norm, g.k, g.ids, b.wk, b.cand,  \
+            t, X, reinterpret_cast<const __nv_bfloat16*>(b.Xb), b.dp, b.f16, b.X8, b.tcm, inv_norm, g.k, g.ids, b.wk, b.cand,  \
             b.nn, b.no, b.cmax, cmq, cols, list, b.prop_tgt, b.prop_key, b.prop_count, b.prop_cap, b.pending,     \
             pairs, cands, status);                                                                                \
         e = cudaGetLastError();                                                                                   \
