@@ -199,7 +199,8 @@ static inline void need(bool ok, fgim_status st, const char* what) {
     }
 }
 
-// counters on the device: [0] ndc, [1] hops, [2] pairs, [3] repaired, [4] attached
+// counters on the device: [0] ndc, [1] hops, [2] pairs, [3] repaired, [4] attached, [5] candidates joined,
+// [6] zero-indegree vertices of the last repair, [8] the beam searches' item counter
 struct Ctx {
     cudaStream_t s;
     Scratch sc;
@@ -266,6 +267,7 @@ struct Ctx {
             st->repaired += (int64_t)hc[3];
             st->attached += (int64_t)hc[4];
             st->join_cands += (int64_t)hc[5];
+            st->zero_indegree = (int64_t)hc[6];   // of the call's last repair
         }
         if (hs[0] & kErrTimeout) need(false, FGIM_ETIMEOUT, "a bounded device loop ran out");
         if (hs[0] & kErrBounds) need(false, FGIM_EINVAL, "an input index is out of range (graph ids or entry)");
@@ -534,12 +536,12 @@ static RefineBuffers refine_buffers(Ctx& c, const Problem& P, const fgim_params*
     const int rev_cap = resolve_rev_cap(p);
     RefineBuffers b;
     std::memset(&b, 0, sizeof(b));
-    b.cntN = c.alloc<int32_t>(N);
-    b.cntO = c.alloc<int32_t>(N);
+    b.cntN = c.alloc<int32_t>(4 * N);
+    b.cntO = b.cntN + N;
+    b.fillN = b.cntN + 2 * N;
+    b.fillO = b.cntN + 3 * N;
     b.offN = c.alloc<long long>(N + 1);
     b.offO = c.alloc<long long>(N + 1);
-    b.fillN = c.alloc<int32_t>(N);
-    b.fillO = c.alloc<int32_t>(N);
     b.rev_capacity = N * k;
     b.revN = c.alloc<uint64_t>(N * k);
     b.revO = c.alloc<uint64_t>(N * k);
@@ -564,9 +566,9 @@ static RefineBuffers refine_buffers(Ctx& c, const Problem& P, const fgim_params*
     b.prop_key = c.alloc<uint64_t>(cap);
     b.prop_sorted = c.alloc<uint64_t>(cap);
     b.prop_count = c.alloc<unsigned long long>(1);
-    b.pcnt = c.alloc<int32_t>(N);
+    b.pcnt = c.alloc<int32_t>(2 * N);
+    b.pfill = b.pcnt + N;
     b.poff = c.alloc<long long>(N + 1);
-    b.pfill = c.alloc<int32_t>(N);
     b.pending = c.alloc<uint8_t>(N);
     b.pend_flag = c.alloc<int32_t>(N);
     b.pend_list = c.alloc<int32_t>(N);
@@ -640,13 +642,11 @@ static void refine_pass(Ctx& c, const Problem& P, const fgim_params* p, fgim_knn
     // merged lists: a proposal that would have entered a list still beats its (only lower)
     // worst key and is still absent, so the merged result is the same
     long long prev_pending = -1;
-    for (int rerun = 0;; ++rerun) {
+    while (cnt > (unsigned long long)cap) {   // only a full buffer leaves vertices pending
         ck(launch_nonzero_flags(b.pending, N, b.pend_flag, c.s));
         ck(compact_flags(b.pend_flag, N, b.pend_list, b.pend_off, b.scan_tmp, b.scan_bytes, c.s));
         const long long np = c.read_ll(b.pend_off + N);
-        if (np == 0) break;
-        need(!(cnt <= (unsigned long long)cap && np == prev_pending), FGIM_EINTERNAL,
-             "pending vertices without a proposal overflow");
+        need(np > 0 && np != prev_pending, FGIM_EINTERNAL, "proposal overflow does not shrink");
         prev_pending = np;
         st->join_reruns += 1;
         need(st->join_reruns < 10000, FGIM_EINTERNAL, "proposal overflow does not shrink");
@@ -661,7 +661,7 @@ static void refine_pass(Ctx& c, const Problem& P, const fgim_params* p, fgim_knn
     st->proposals += total;
 }
 
-static void repair(Ctx& c, const Problem& P, fgim_knng* g, int32_t* T, fgim_stats* st) {
+static void repair(Ctx& c, const Problem& P, fgim_knng* g, int32_t* T) {
     StageRange range("fgim stage b: indegree repair (Alg. 4)");
     const long long N = P.N;
     ck(launch_indegree(g->ids, N, g->k, T, true, g->flags, c.s));
@@ -672,24 +672,10 @@ static void repair(Ctx& c, const Problem& P, fgim_knng* g, int32_t* T, fgim_stat
     unsigned char* tmp = c.alloc<unsigned char>((long long)sb);
     ck(launch_zero_flags(T, N, flag, c.s));
     ck(compact_flags(flag, N, zeros, off, tmp, sb, c.s));
-    const long long nz = c.read_ll(off + N);
-    if (st) st->zero_indegree = nz;
-    if (nz == 0) return;
     unsigned long long* owner = c.alloc<unsigned long long>(N);
-    long long* ff = c.alloc<long long>(nz + 2);   // first uncommitted index after each round (one round commits >= 1)
-    ck(cudaMemsetAsync(owner, 0xff, sizeof(unsigned long long) * N, c.s));
-    ck(cudaMemsetAsync(ff, 0, sizeof(long long), c.s));
-    long long start = 0, rho = 1;
-    constexpr int kBatch = 16;   // rounds between host reads of the progress
-    while (start < nz) {
-        need(rho <= nz, FGIM_EINTERNAL, "indegree repair made no progress");
-        const int rounds = (int)std::min<long long>(kBatch, nz + 1 - rho);
-        ck(launch_repair_rounds(*g, T, zeros, nz, rho, rounds, ff, owner, c.ctr + 3, c.status, c.s));
-        rho += rounds;
-        const long long next = c.read_ll(ff + (rho - 1));
-        need(next > start, FGIM_EINTERNAL, "indegree repair made no progress");
-        start = next;
-    }
+    long long* ff = c.alloc<long long>(3);
+    int4* plan = c.alloc<int4>(kRepairWindow);
+    ck(launch_repair(*g, T, zeros, off + N, ff, owner, plan, c.ctr + 3, c.ctr + 6, c.status, c.s));
 }
 
 static void prune(Ctx& c, const Problem& P, const fgim_params* p, const fgim_knng* g, const int32_t* T, int32_t* e_ids,
@@ -725,17 +711,9 @@ struct Entries {
 
 // BFS from the entry (or entries); returns the number of reached vertices
 static long long bfs(Ctx& c, const fgim_graph* g, const Entries& E, int32_t* visited, int32_t* fa, int32_t* fb,
-                     int32_t* counts) {
-    const long long N = g->n;
-    if (E.ent) ck(launch_bfs_init_multi(visited, N, fa, counts, E.ent, E.nm, c.status, c.s));
-    else ck(launch_bfs_init(visited, N, fa, counts, g->entry, c.s));
-    constexpr int kBatch = 8;   // levels between host reads of the frontier size
-    for (int level = 1; level <= N; level += kBatch) {
-        ck(launch_bfs_levels(g->ids, g->R, N, visited, fa, fb, counts, level, kBatch, c.s));
-        const int last = level + kBatch - 1;   // its output frontier size is counts[(last + 1) % 3]
-        if (c.read_i32(counts + (last + 1) % 3) == 0) break;
-    }
-    return c.read_ll(reinterpret_cast<const long long*>(counts + 4));
+                     int32_t* st) {
+    ck(launch_bfs(g->ids, g->R, g->n, g->entry, E.ent, E.nm, visited, fa, fb, st, c.status, c.s));
+    return c.read_ll(reinterpret_cast<const long long*>(st + 4));
 }
 
 static void reach_fix(Ctx& c, const Problem& P, const fgim_params* p, fgim_graph* g, fgim_stats* st,
@@ -754,25 +732,17 @@ static void reach_fix(Ctx& c, const Problem& P, const fgim_params* p, fgim_graph
     long long* off = c.alloc<long long>(N + 1);
     const size_t sb = scan_scratch_bytes(N);
     unsigned char* tmp = c.alloc<unsigned char>((long long)sb);
-    int32_t* changed = c.alloc<int32_t>(1);
     int32_t* npar = c.alloc<int32_t>(N);
     unsigned long long* owner = c.alloc<unsigned long long>(N);
-    long long* ff = c.alloc<long long>(N + 2);   // first uncommitted index after each round (one round commits >= 1)
+    long long* ff = c.alloc<long long>(3);
     int4* plan = c.alloc<int4>(kReachWindow);    // the actions planned in a round
     int32_t* cand = nullptr;
     float* cdist = nullptr;
     int32_t* starts = nullptr;
     long long cand_cap = 0;
-    long long reached = 0;
-    for (int round = 0; round < 16; ++round) {
-        reached = bfs(c, g, E, visited, fa, fb, counts);
-        if (reached >= N) break;
-        ck(launch_cc_init(visited, N, label, c.s));
-        for (long long it = 0; it <= N; ++it) {
-            ck(cudaMemsetAsync(changed, 0, sizeof(int32_t), c.s));
-            ck(launch_cc_step(g->ids, R, N, visited, label, changed, c.s));
-            if (c.read_i32(changed) == 0) break;
-        }
+    long long reached = bfs(c, g, E, visited, fa, fb, counts);
+    for (int round = 0; round < 16 && reached < N; ++round) {
+        ck(launch_cc(g->ids, R, N, visited, label, fa, counts, c.s));
         ck(launch_rep_flags(visited, label, N, flag, c.s));
         ck(compact_flags(flag, N, reps, off, tmp, sb, c.s));
         const long long nr = c.read_ll(off + N);
@@ -788,23 +758,12 @@ static void reach_fix(Ctx& c, const Problem& P, const fgim_params* p, fgim_graph
         ck(launch_search(P.X, P.X8, P.inv, N, P.d, P.metric, g->ids, R, g->entry, nullptr, nullptr, reps, nr, beam, beam,
                          cand, cdist, c.ctr + 0, c.status, c.s, P.Xh, E.ent ? starts : nullptr));
         ck(launch_bfs_parents(g->ids, R, N, visited, npar, c.s));
-        // rounds run in batches between host reads of the progress; ff[0] = 0 starts round 1
         ck(cudaMemsetAsync(owner, 0xff, sizeof(unsigned long long) * N, c.s));
-        ck(cudaMemsetAsync(ff, 0, sizeof(long long), c.s));
-        long long start = 0, rho = 1;
-        constexpr int kBatch = 64;   // rounds per cooperative launch (it stops early once all are done)
-        while (start < nr) {
-            need(rho <= nr, FGIM_EINTERNAL, "reachability fix made no progress");
-            const int rounds = (int)std::min<long long>(kBatch, nr + 1 - rho);
-            ck(launch_reach_rounds(g->ids, g->dist, g->deg, visited, npar, R, reps, nr, rho, rounds, ff, cand, cdist,
-                                   beam, owner, plan, c.ctr + 4, c.s));
-            rho += rounds;
-            const long long next = c.read_ll(ff + (rho - 1));
-            need(next > start, FGIM_EINTERNAL, "reachability fix made no progress");
-            start = next;
-        }
+        ck(cudaMemsetAsync(ff, 0, sizeof(long long), c.s));   // ff[0] = 0 starts round 1
+        ck(launch_reach_rounds(g->ids, g->dist, g->deg, visited, npar, R, reps, nr, ff, cand, cdist, beam, owner, plan,
+                               c.ctr + 4, c.status, c.s));
+        reached = bfs(c, g, E, visited, fa, fb, counts);
     }
-    reached = bfs(c, g, E, visited, fa, fb, counts);
     if (st) st->unreached = N - reached;
 }
 
@@ -897,7 +856,7 @@ fgim_status fgim_indegree_repair(const fgim_shard* shards, int32_t h, const fgim
         Problem P;
         P.N = knng->n;
         int32_t* T = T_out ? T_out : c.alloc<int32_t>(P.N);
-        repair(c, P, knng, T, &t_stats);
+        repair(c, P, knng, T);
         c.finish(&t_stats);
     });
     end_call();
@@ -985,7 +944,7 @@ static void merge_impl(Ctx& c, const fgim_shard* shards, int32_t h, const fgim_p
     if (params->iters > 0) b = refine_buffers(c, P, params, k);
     for (int it = 0; it < params->iters; ++it) {
         refine_pass(c, P, params, &g, &t_stats, b);
-        repair(c, P, &g, T, &t_stats);
+        repair(c, P, &g, T);
     }
     if (params->iters == 0) ck(launch_indegree(g.ids, N, k, T, false, nullptr, c.s));
     int32_t* e_ids = c.alloc<int32_t>(N * params->R);
@@ -1102,7 +1061,7 @@ static void merge_union(Ctx& c, const fgim_shard* const* shards, const int32_t* 
     if (p->iters > 0) b = refine_buffers(c, P, p, k);
     for (int it = 0; it < p->iters; ++it) {
         refine_pass(c, P, p, &g, &t_stats, b);
-        repair(c, P, &g, T, &t_stats);
+        repair(c, P, &g, T);
     }
     if (p->iters == 0) ck(launch_indegree(g.ids, N, k, T, false, nullptr, c.s));
     int32_t* e_ids = c.alloc<int32_t>(N * R);

@@ -26,10 +26,38 @@ cudaError_t launch_search(const float* X, const uint8_t* X8, const float* inv_no
 // X8[i] = X[i] as a byte; *flag |= 1 unless every X[i] is an integer in [0, 255] (n_elems % 4 == 0)
 cudaError_t launch_narrow_u8(const float* X, long long n_elems, uint8_t* X8, int* flag, cudaStream_t s);
 
+// the grid of a cooperative launch: `want` blocks, at most as many as are resident at once (the grid-wide
+// barriers wait for all of them)
+template <typename K>
+cudaError_t coop_grid(K kernel, int threads, long long want, int* blocks) {
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
+    const long long most = (long long)per_sm * sms;
+    *blocks = (int)(want < 1 ? 1 : want < most ? want : most);
+    return cudaSuccess;
+}
+
+// Rounds that commit a prefix of a window (indegree repair, reachability fix): blocks of 16 warps, so that a
+// full window has a warp per item in at most 128 blocks (a grid-wide barrier costs less the fewer blocks
+// arrive: the 1M merge's reachability rounds 13.5 ms with 512 blocks of 4 warps, 8.3 ms so, 8.9 ms with 64 blocks
+// of 32); the next round looks at four times the items the last one committed, within [256, most] (what
+// lies past the first conflict is planned for nothing). The window changes no result.
+constexpr int kRoundThreads = 512;
+__device__ __forceinline__ long long round_window(long long committed, long long most) {
+    const long long w = 4 * committed;
+    return w < 256 ? 256 : w < most ? w : most;
+}
+
 // ---- k_util.cu
 // exclusive scan of n int32 counts into n + 1 int64 offsets (out[n] = total)
 cudaError_t scan_counts(const int32_t* in, long long n, long long* out, void* scratch, size_t scratch_bytes,
                         cudaStream_t s);
+cudaError_t scan_counts2(const int32_t* in0, const int32_t* in1, long long n, long long* out0, long long* out1,
+                         void* scratch, size_t scratch_bytes, cudaStream_t s);   // two arrays of n at once
 size_t scan_scratch_bytes(long long n);
 cudaError_t launch_inv_norms(const float* X, long long n, int d, float* inv, cudaStream_t s);
 // out[i] = the FP32 value of the bfloat16 encoding in[i]
@@ -48,12 +76,12 @@ cudaError_t compact_flags(const int32_t* flag, long long n, int32_t* out, long l
 // ---- k_refine.cu
 struct RefineBuffers {
     // reverse lists
-    int32_t* cntN;
+    int32_t* cntN;            // cntN, cntO, fillN, fillO: one block of 4 N
     int32_t* cntO;
-    long long* offN;
-    long long* offO;
     int32_t* fillN;
     int32_t* fillO;
+    long long* offN;
+    long long* offO;
     uint64_t* revN;
     uint64_t* revO;
     long long rev_capacity;   // entries of revN / revO (N * k each)
@@ -72,9 +100,9 @@ struct RefineBuffers {
     long long prop_cap;
     unsigned long long* prop_count;   // device counter
     uint64_t* prop_sorted;
-    int32_t* pcnt;
-    long long* poff;
+    int32_t* pcnt;            // proposals per target (counted by the join), pcnt and pfill: one block of 2 N
     int32_t* pfill;
+    long long* poff;
     uint8_t* pending;
     int32_t* pend_flag;
     int32_t* pend_list;
@@ -123,12 +151,12 @@ cudaError_t launch_prep_f16(const float* X, long long N, int d, int dp, void* Xb
                             cudaStream_t s);
 cudaError_t launch_indegree(const int32_t* ids, long long N, int k, int32_t* T, bool clear_replaced, uint8_t* flags,
                             cudaStream_t s);
-// rounds rho0 .. rho0 + rounds - 1 of the Alg. 4 repair; ff[rho0 - 1] holds the first pending
-// index, ff[rho] the first index after round rho
+// Alg. 4 for the vertices zeros[0 .. *nz) (ascending), in one cooperative launch; ff: 3 words, plan: scratch of
+// kRepairWindow entries, owner [g.n]; *zero_count = *nz
 constexpr int kRepairWindow = 2048;
-cudaError_t launch_repair_rounds(fgim_knng& g, int32_t* T, const int32_t* zeros, long long nz, long long rho0,
-                                 int rounds, long long* ff, unsigned long long* owner, unsigned long long* repaired,
-                                 int* status, cudaStream_t s);
+cudaError_t launch_repair(fgim_knng& g, int32_t* T, const int32_t* zeros, const long long* nz, long long* ff,
+                          unsigned long long* owner, int4* plan, unsigned long long* repaired,
+                          unsigned long long* zero_count, int* status, cudaStream_t s);
 cudaError_t launch_zero_flags(const int32_t* T, long long N, int32_t* flag, cudaStream_t s);
 cudaError_t launch_nonzero_flags(const uint8_t* v, long long N, int32_t* flag, cudaStream_t s);
 
@@ -150,36 +178,31 @@ struct ReverseBuffers {
 cudaError_t launch_reverse_insert(long long N, int R, const int32_t* e_ids, const float* e_dist, const int32_t* e_cnt,
                                   ReverseBuffers& b, int32_t* out_ids, float* out_dist, int32_t* out_deg,
                                   cudaStream_t s);
-// reachability fix helpers
-cudaError_t launch_bfs_init(int32_t* visited, long long N, int32_t* frontier, int32_t* st, int entry,
-                            cudaStream_t s);
-// the same from the ne sources entries[] (device)
-cudaError_t launch_bfs_init_multi(int32_t* visited, long long N, int32_t* frontier, int32_t* st,
-                                  const int32_t* entries, int ne, int* status, cudaStream_t s);
 // batches run as one problem: start[r] = entries[m] of the merge m (id range off[m] .. off[m+1]-1)
 // holding reps[r]; the rows of one merge copied out of the union graph, ids minus base
 cudaError_t launch_rep_starts(const int32_t* reps, long long nr, const long long* off, const int32_t* entries, int nm,
                               int32_t* start, cudaStream_t s);
 cudaError_t launch_split_rows(const int32_t* ids, const float* dist, const int32_t* deg, long long n, int R,
                               int32_t base, int32_t* out_ids, float* out_dist, int32_t* out_deg, cudaStream_t s);
-// BFS levels level0 .. level0 + levels - 1 (state st: 8 ints, see k_prune.cu; level 1 reads fa)
-cudaError_t launch_bfs_levels(const int32_t* graph, int R, long long N, int32_t* visited, int32_t* fa, int32_t* fb,
-                              int32_t* st, int level0, int levels, cudaStream_t s);
+// BFS from `entry` (entries == nullptr) or from the ne sources `entries` (device), in one cooperative launch:
+// visited[y] = level (sources 1, unreached 0); fa, fb [N]; st: 8 ints, reached vertices (int64) at st[4]
+cudaError_t launch_bfs(const int32_t* graph, int R, long long N, int entry, const int32_t* entries, int ne,
+                       int32_t* visited, int32_t* fa, int32_t* fb, int32_t* st, int* status, cudaStream_t s);
 cudaError_t launch_bfs_parents(const int32_t* graph, int R, long long N, const int32_t* level, int32_t* npar,
                                cudaStream_t s);
-cudaError_t launch_cc_init(const int32_t* visited, long long N, int32_t* label, cudaStream_t s);
-cudaError_t launch_cc_step(const int32_t* graph, int R, long long N, const int32_t* visited, int32_t* label,
-                           int32_t* changed, cudaStream_t s);
+// label[x] = the smallest id of x's weak component among the unreached vertices (-1: reached), in one
+// cooperative launch; list [N], st: 4 ints
+cudaError_t launch_cc(const int32_t* graph, int R, long long N, const int32_t* visited, int32_t* label, int32_t* list,
+                      int32_t* st, cudaStream_t s);
 cudaError_t launch_rep_flags(const int32_t* visited, const int32_t* label, long long N, int32_t* flag,
                              cudaStream_t s);
-// `rounds` rounds of the representative attachment (rounds rho0 .. rho0 + rounds - 1) in one
-// cooperative launch; ff[rho0 - 1] holds the first pending index, ff[rho] the first index
-// after round rho; plan: scratch of kReachWindow entries
+// the attachment of the nr representatives in one cooperative launch; ff: 3 words, ff[0] = 0; plan: scratch of
+// kReachWindow entries, owner all ones
 constexpr int kReachWindow = 2048;
 cudaError_t launch_reach_rounds(int32_t* graph, float* gdist, int32_t* deg, const int32_t* level, int32_t* npar,
-                                int R, const int32_t* reps, long long nr, long long rho0, int rounds, long long* ff,
-                                const int32_t* cand, const float* cdist, int beam, unsigned long long* owner,
-                                int4* plan, unsigned long long* attached, cudaStream_t s);
+                                int R, const int32_t* reps, long long nr, long long* ff, const int32_t* cand,
+                                const float* cdist, int beam, unsigned long long* owner, int4* plan,
+                                unsigned long long* attached, int* status, cudaStream_t s);
 
 // ---- k_hnsw.cu (HNSW-adaptive merging, Sec. 4.3.3)
 constexpr int kMaxHnswLevels = 16;

@@ -7,9 +7,6 @@
 
 #include <cooperative_groups.h>
 
-#include <map>
-#include <mutex>
-
 #include "fgim_launch.h"
 
 namespace fgim {
@@ -97,109 +94,69 @@ cudaError_t launch_reverse_insert(long long N, int R, const int32_t* e_ids, cons
 
 // ---------------------------------------------------------------------------- reachability fix
 // BFS state: st[0..2] frontier sizes (level L reads st[L % 3], writes st[(L + 1) % 3] and
-// clears st[(L + 2) % 3] for the level after), st[4..5] the number of reached vertices (int64)
-__global__ void k_bfs_init(int32_t* visited, long long N, int32_t* frontier, int32_t* st, int entry) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N) visited[i] = (i == entry) ? 1 : 0;
-    if (i == 0) {
-        frontier[0] = entry;
-        st[1] = 1;   // level 1 reads st[1]
-        st[2] = 0;
-        st[0] = 0;
-        *reinterpret_cast<long long*>(st + 4) = 1;
+// clears st[(L + 2) % 3] for the level after), st[4..5] the number of reached vertices (int64).
+// All levels in one cooperative launch, a grid-wide barrier per level: the levels are short (a launch each
+// and a host read every eight cost 0.3 of the 4.4 ms of a 20,000-vertex merge).
+__global__ void __launch_bounds__(512) k_bfs(const int32_t* __restrict__ graph, int R, long long N, int entry,
+                                             const int32_t* __restrict__ entries, int ne, int32_t* visited,
+                                             int32_t* fa, int32_t* fb, int32_t* st, int* status) {
+    cg::grid_group grid = cg::this_grid();
+    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
+    const int lane = lane_id();
+    for (long long i = tid; i < N; i += nt) visited[i] = 0;
+    if (tid == 0) {
+        st[0] = st[2] = 0;
+        st[1] = entries ? ne : 1;
+        *reinterpret_cast<long long*>(st + 4) = entries ? ne : 1;
     }
-}
-
-cudaError_t launch_bfs_init(int32_t* visited, long long N, int32_t* frontier, int32_t* st, int entry,
-                            cudaStream_t s) {
-    LaunchScope ls("k_bfs_init", s);
-    k_bfs_init<<<(unsigned)cdivl(N, 256), 256, 0, s>>>(visited, N, frontier, st, entry);
-    return cudaGetLastError();
-}
-
-// BFS from several sources at once (the entries of the merges of a batch, each in its own
-// component of the union graph): every entry is at level 1 and in the first frontier
-__global__ void k_bfs_init_multi(int32_t* visited, long long N, int32_t* frontier, int32_t* st,
-                                 const int32_t* __restrict__ entries, int ne) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N) visited[i] = 0;
-    if (i == 0) {
-        st[1] = ne;
-        st[2] = 0;
-        st[0] = 0;
-        *reinterpret_cast<long long*>(st + 4) = ne;
-    }
-}
-__global__ void k_bfs_seed(int32_t* visited, long long N, int32_t* frontier, const int32_t* __restrict__ entries,
-                           int ne, int* status) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= ne) return;
-    const int32_t e = entries[i];
-    if (e < 0 || e >= N) {
-        atomicOr(status, kErrBounds);
-        frontier[i] = 0;
-        return;
-    }
-    visited[e] = 1;
-    frontier[i] = e;
-}
-
-cudaError_t launch_bfs_init_multi(int32_t* visited, long long N, int32_t* frontier, int32_t* st,
-                                  const int32_t* entries, int ne, int* status, cudaStream_t s) {
-    {
-        LaunchScope ls("k_bfs_init", s);
-        k_bfs_init_multi<<<(unsigned)cdivl(N, 256), 256, 0, s>>>(visited, N, frontier, st, entries, ne);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    LaunchScope ls("k_bfs_init", s);
-    k_bfs_seed<<<(unsigned)cdivl(ne, 256), 256, 0, s>>>(visited, N, frontier, entries, ne, status);
-    return cudaGetLastError();
-}
-
-// one level L (grid-stride over (frontier vertex, neighbour slot)); visited[y] = BFS level
-// (entry = 1); a level whose frontier is empty does nothing, so several levels can be
-// queued without reading the frontier size on the host
-__global__ void k_bfs_step(const int32_t* __restrict__ graph, int R, long long N, int32_t* __restrict__ visited,
-                           const int32_t* __restrict__ fin, int32_t* __restrict__ fout, int32_t* __restrict__ st,
-                           int level) {
-    const long long nf = st[level % 3];
-    if (blockIdx.x == 0 && threadIdx.x == 0) st[(level + 2) % 3] = 0;
-    const int32_t next_level = level + 1;
-    int added = 0;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nf * R;
-         i += (long long)gridDim.x * blockDim.x) {
-        const long long fi = div_idx(i, R);
-        const int32_t x = fin[fi];
-        const int32_t y = graph[(long long)x * R + (i - fi * R)];
-        if (y < 0 || y >= N) continue;
-        if (visited[y] == 0 && atomicCAS(visited + y, 0, next_level) == 0) {
-            fout[atomicAdd(st + (level + 1) % 3, 1)] = y;
-            ++added;
+    grid.sync();
+    for (long long i = tid; i < (entries ? ne : 1); i += nt) {
+        int32_t e = entries ? entries[i] : entry;
+        if (e < 0 || e >= N) {
+            atomicOr(status, kErrBounds);
+            e = 0;
         }
+        visited[e] = 1;
+        fa[i] = e;
     }
-    const unsigned m = __ballot_sync(kFull, added > 0);
-    int sum = added;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
-    if ((threadIdx.x & 31) == 0 && m) atomicAdd(reinterpret_cast<unsigned long long*>(st + 4), (unsigned long long)sum);
-}
-
-cudaError_t launch_bfs_levels(const int32_t* graph, int R, long long N, int32_t* visited, int32_t* fa, int32_t* fb,
-                              int32_t* st, int level0, int levels, cudaStream_t s) {
-    const long long work = N * (long long)R;
-    const unsigned blocks = (unsigned)std::min<long long>(cdivl(work, 256), 152LL * 16);
-    for (int q = 0; q < levels; ++q) {
-        const int level = level0 + q;
-        // level L reads the frontier written by level L - 1: fa for odd L, fb for even L
+    grid.sync();
+    int sum = 0;
+    for (int level = 1; level <= N; ++level) {
+        const long long work = (long long)__ldcg(st + level % 3) * R;
+        if (work == 0) break;
+        if (tid == 0) st[(level + 2) % 3] = 0;
         const int32_t* fin = (level & 1) ? fa : fb;
         int32_t* fout = (level & 1) ? fb : fa;
-        LaunchScope ls("k_bfs_step", s);
-        k_bfs_step<<<blocks, 256, 0, s>>>(graph, R, N, visited, fin, fout, st, level);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+        int32_t* nout = st + (level + 1) % 3;
+        for (long long i0 = tid - lane; i0 < work; i0 += nt) {   // whole warps
+            const long long i = i0 + lane;
+            int32_t y = -1;
+            if (i < work) {
+                const long long fi = div_idx(i, R);
+                y = graph[(long long)__ldcg(fin + fi) * R + (i - fi * R)];
+            }
+            const bool add = y >= 0 && y < N && __ldcg(visited + y) == 0 && atomicCAS(visited + y, 0, level + 1) == 0;
+            const unsigned m = __ballot_sync(kFull, add);
+            if (m == 0u) continue;
+            int base = 0;
+            if (lane == 0) base = atomicAdd(nout, __popc(m));
+            base = __shfl_sync(kFull, base, 0);
+            if (add) fout[base + __popc(m & ((1u << lane) - 1u))] = y;
+            sum += __popc(m);
+        }
+        grid.sync();
     }
-    return cudaSuccess;
+    if (lane == 0 && sum) atomicAdd(reinterpret_cast<unsigned long long*>(st + 4), (unsigned long long)sum);
+}
+
+cudaError_t launch_bfs(const int32_t* graph, int R, long long N, int entry, const int32_t* entries, int ne,
+                       int32_t* visited, int32_t* fa, int32_t* fb, int32_t* st, int* status, cudaStream_t s) {
+    int blocks = 0;
+    const cudaError_t e = coop_grid(k_bfs, 512, std::min<long long>(cdivl(N * (long long)R, 512 * 4), 608), &blocks);
+    if (e != cudaSuccess) return e;
+    LaunchScope ls("k_bfs", s);
+    void* args[] = {&graph, &R, &N, &entry, &entries, &ne, &visited, &fa, &fb, &st, &status};
+    return cudaLaunchCooperativeKernel((const void*)k_bfs, dim3(blocks), dim3(512), args, 0, s);
 }
 
 // number of BFS parents of every reached vertex: in-neighbours at a smaller level
@@ -222,39 +179,55 @@ cudaError_t launch_bfs_parents(const int32_t* graph, int R, long long N, const i
     return cudaGetLastError();
 }
 
-__global__ void k_cc_init(const int32_t* __restrict__ visited, long long N, int32_t* __restrict__ label) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N) label[i] = visited[i] ? -1 : (int32_t)i;
-}
-
-cudaError_t launch_cc_init(const int32_t* visited, long long N, int32_t* label, cudaStream_t s) {
-    LaunchScope ls("k_cc_init", s);
-    k_cc_init<<<(unsigned)cdivl(N, 256), 256, 0, s>>>(visited, N, label);
-    return cudaGetLastError();
-}
-
-// min-label propagation over the undirected edges between unreached vertices
-__global__ void k_cc_step(const int32_t* __restrict__ graph, int R, long long N, const int32_t* __restrict__ visited,
-                          int32_t* __restrict__ label, int32_t* __restrict__ changed) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N * R) return;
-    const long long x = div_idx(i, R);
-    if (visited[x]) return;
-    const int32_t y = graph[i];
-    if (y < 0 || y >= N || visited[y]) return;
-    const int32_t lx = label[x], ly = label[y];
-    if (lx < ly) {
-        if (atomicMin(label + y, lx) > lx) *changed = 1;
-    } else if (ly < lx) {
-        if (atomicMin(label + x, ly) > ly) *changed = 1;
+// min-label propagation over the undirected edges between unreached vertices, all passes in one
+// cooperative launch over the list of the unreached vertices (one launch per pass over every vertex's
+// edges, and a host read after each, before). st[0]: their number, st[1 + it % 3]: pass it changed a label.
+__global__ void __launch_bounds__(512) k_cc(const int32_t* __restrict__ graph, int R, long long N,
+                                            const int32_t* __restrict__ visited, int32_t* label, int32_t* list,
+                                            int32_t* st) {
+    cg::grid_group grid = cg::this_grid();
+    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
+    const int lane = lane_id();
+    for (long long i0 = tid - lane; i0 < N; i0 += nt) {
+        const long long i = i0 + lane;
+        const bool un = i < N && visited[i] == 0;
+        if (i < N) label[i] = un ? (int32_t)i : -1;
+        const unsigned m = __ballot_sync(kFull, un);
+        if (m == 0u) continue;
+        int base = 0;
+        if (lane == 0) base = atomicAdd(st, __popc(m));
+        base = __shfl_sync(kFull, base, 0);
+        if (un) list[base + __popc(m & ((1u << lane) - 1u))] = (int32_t)i;
+    }
+    grid.sync();
+    const long long work = (long long)__ldcg(st) * R;
+    for (long long it = 0; it <= N; ++it) {
+        bool changed = false;
+        if (tid == 0) st[1 + (it + 1) % 3] = 0;
+        for (long long i = tid; i < work; i += nt) {
+            const long long li = div_idx(i, R);
+            const int32_t x = __ldcg(list + li);
+            const int32_t y = graph[(long long)x * R + (i - li * R)];
+            if (y < 0 || y >= N || visited[y]) continue;
+            const int32_t lx = __ldcg(label + x), ly = __ldcg(label + y);
+            if (lx < ly) changed |= atomicMin(label + y, lx) > lx;
+            else if (ly < lx) changed |= atomicMin(label + x, ly) > ly;
+        }
+        if (__any_sync(kFull, changed) && lane == 0) st[1 + it % 3] = 1;
+        grid.sync();
+        if (__ldcg(st + 1 + it % 3) == 0) break;
     }
 }
 
-cudaError_t launch_cc_step(const int32_t* graph, int R, long long N, const int32_t* visited, int32_t* label,
-                           int32_t* changed, cudaStream_t s) {
-    LaunchScope ls("k_cc_step", s);
-    k_cc_step<<<(unsigned)cdivl(N * R, 256), 256, 0, s>>>(graph, R, N, visited, label, changed);
-    return cudaGetLastError();
+cudaError_t launch_cc(const int32_t* graph, int R, long long N, const int32_t* visited, int32_t* label, int32_t* list,
+                      int32_t* st, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(st, 0, 4 * sizeof(int32_t), s);
+    if (e != cudaSuccess) return e;
+    int blocks = 0;
+    if ((e = coop_grid(k_cc, 512, std::min<long long>(cdivl(N * (long long)R, 512 * 4), 304), &blocks)) != cudaSuccess) return e;
+    LaunchScope ls("k_cc", s);
+    void* args[] = {&graph, &R, &N, &visited, &label, &list, &st};
+    return cudaLaunchCooperativeKernel((const void*)k_cc, dim3(blocks), dim3(512), args, 0, s);
 }
 
 __global__ void k_rep_flags(const int32_t* __restrict__ visited, const int32_t* __restrict__ label, long long N,
@@ -281,8 +254,8 @@ cudaError_t launch_rep_flags(const int32_t* visited, const int32_t* label, long 
 // longest ascending prefix of the round's window holding its reservations is committed,
 // the rest recomputed in the next round.
 //
-// Round rho works on the window [ff[rho - 1], min(ff[rho - 1] + W, nr)) and leaves in ff[rho]
-// the first index it did not commit (the next round's start). Tags of later rounds are
+// Round rho works on the window [start, min(start + W, nr)), start = ff[(rho - 1) % 3], and leaves in
+// ff[rho % 3] the first index it did not commit (the next round's start). Tags of later rounds are
 // smaller than those of earlier ones, so owner needs no reset between rounds.
 __device__ __forceinline__ unsigned long long reach_tag(long long rho, long long r) {
     return ((unsigned long long)(0xFFFFFFFFu - (uint32_t)rho) << 32) | (unsigned long long)(uint32_t)r;
@@ -333,33 +306,31 @@ __device__ __forceinline__ int4 reach_plan(const int32_t* __restrict__ graph, co
     return make_int4(p, pos, t_sel, victim);
 }
 
-// The rounds of one batch in one cooperative launch (warps stride over the window): plan
+// The rounds in one cooperative launch (warps stride over the window): plan
 // (the action of every item and its reservations), check (the first item that lost one
 // bounds the prefix), commit (the prefix); phases are separated by grid-wide barriers and an
-// item's plan is computed once per round.
-__global__ void __launch_bounds__(128) k_reach_rounds(int32_t* __restrict__ graph, float* __restrict__ gdist,
-                                                      int32_t* __restrict__ deg, const int32_t* __restrict__ level,
-                                                      int32_t* __restrict__ npar, int R,
-                                                      const int32_t* __restrict__ reps, long long nr, long long rho0,
-                                                      int rounds, long long window, long long* __restrict__ ff,
-                                                      const int32_t* __restrict__ cand,
+// item's plan is computed once per round. Every round commits at least one item.
+__global__ void __launch_bounds__(kRoundThreads) k_reach_rounds(int32_t* graph, float* gdist, int32_t* deg,
+                                                      const int32_t* __restrict__ level, int32_t* npar, int R,
+                                                      const int32_t* __restrict__ reps, long long nr, long long window,
+                                                      long long* ff, const int32_t* __restrict__ cand,
                                                       const float* __restrict__ cdist, int beam,
-                                                      unsigned long long* __restrict__ owner, int4* __restrict__ plan,
-                                                      unsigned long long* attached) {
+                                                      unsigned long long* owner, int4* plan,
+                                                      unsigned long long* attached, int* status) {
     cg::grid_group grid = cg::this_grid();
     const int lane = lane_id();
     const long long gw = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
-    for (int q = 0; q < rounds; ++q) {
-        const long long rho = rho0 + q;
-        const long long start = ff[rho - 1];   // written before the last barrier
-        if (start >= nr) {                     // the same for every thread: all leave together
-            if (blockIdx.x == 0 && threadIdx.x == 0)
-                for (int t = q; t < rounds; ++t) ff[rho0 + t] = nr;
-            return;
+    long long win = window;
+    for (long long rho = 1;; ++rho) {
+        const long long start = __ldcg(ff + (rho - 1) % 3);   // written before the last barrier
+        if (start >= nr) break;                               // the same for every thread: all leave together
+        if (rho > nr) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, kErrTimeout);
+            break;
         }
-        const long long wend = start + window < nr ? start + window : nr;
-        if (blockIdx.x == 0 && threadIdx.x == 0) ff[rho] = wend;
+        const long long wend = start + win < nr ? start + win : nr;
+        if (blockIdx.x == 0 && threadIdx.x == 0) ff[rho % 3] = wend;
         for (long long r = start + gw; r < wend; r += nw) {
             const int4 pl = reach_plan(graph, deg, level, npar, R, cand + r * beam, beam, lane);
             if (lane == 0) {
@@ -376,10 +347,11 @@ __global__ void __launch_bounds__(128) k_reach_rounds(int32_t* __restrict__ grap
             const int4 pl = plan[r - start];
             const unsigned long long tag = reach_tag(rho, r);
             if (pl.x >= 0 && (owner[pl.x] != tag || (pl.w >= 0 && owner[pl.w] != tag)))
-                atomicMin((unsigned long long*)(ff + rho), (unsigned long long)r);
+                atomicMin((unsigned long long*)(ff + rho % 3), (unsigned long long)r);
         }
         grid.sync();
-        const long long cend = ff[rho];
+        const long long cend = __ldcg(ff + rho % 3);
+        win = round_window(cend - start, window);
         for (long long r = start + gw * 32 + lane; r < cend; r += nw * 32) {
             const int4 pl = plan[r - start];
             if (pl.x < 0) continue;
@@ -410,38 +382,16 @@ __global__ void __launch_bounds__(128) k_reach_rounds(int32_t* __restrict__ grap
 }
 
 cudaError_t launch_reach_rounds(int32_t* graph, float* gdist, int32_t* deg, const int32_t* level, int32_t* npar,
-                                int R, const int32_t* reps, long long nr, long long rho0, int rounds, long long* ff,
-                                const int32_t* cand, const float* cdist, int beam, unsigned long long* owner,
-                                int4* plan, unsigned long long* attached, cudaStream_t s) {
-    // a cooperative grid: every block resident at once (the barriers wait for all of them);
-    // the largest such grid is worked out once per device (devices may differ in SM count)
-    static std::mutex mu;
-    static std::map<int, int> max_blocks_of;
-    cudaError_t e = cudaSuccess;
-    int dev = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    int max_blocks = 0;
-    {
-        std::lock_guard<std::mutex> lk(mu);
-        auto it = max_blocks_of.find(dev);
-        if (it != max_blocks_of.end()) {
-            max_blocks = it->second;
-        } else {
-            int per_sm = 0, sms = 0;
-            if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_reach_rounds, 128, 0)) != cudaSuccess)
-                return e;
-            max_blocks = per_sm * sms;
-            if (max_blocks < 1) return cudaErrorCooperativeLaunchTooLarge;
-            max_blocks_of[dev] = max_blocks;
-        }
-    }
+                                int R, const int32_t* reps, long long nr, long long* ff, const int32_t* cand,
+                                const float* cdist, int beam, unsigned long long* owner, int4* plan,
+                                unsigned long long* attached, int* status, cudaStream_t s) {
     long long window = kReachWindow;
-    const int blocks = (int)std::min<long long>(cdivl(window, 4), max_blocks);
+    int blocks = 0;
+    const cudaError_t e = coop_grid(k_reach_rounds, kRoundThreads, cdivl(std::min(window, nr), kRoundThreads / 32), &blocks);
+    if (e != cudaSuccess) return e;
     LaunchScope ls("k_reach_rounds", s);
-    void* args[] = {&graph, &gdist, &deg, &level, &npar, &R, &reps, &nr, &rho0, &rounds, &window, &ff,
-                    &cand, &cdist, &beam, &owner, &plan, &attached};
-    return cudaLaunchCooperativeKernel((const void*)k_reach_rounds, dim3(blocks), dim3(128), args, 0, s);
+    void* args[] = {&graph, &gdist, &deg, &level, &npar, &R, &reps, &nr, &window, &ff, &cand, &cdist, &beam, &owner, &plan, &attached, &status};
+    return cudaLaunchCooperativeKernel((const void*)k_reach_rounds, dim3(blocks), dim3(kRoundThreads), args, 0, s);
 }
 
 }  // namespace fgim

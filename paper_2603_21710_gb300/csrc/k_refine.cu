@@ -18,6 +18,7 @@
 // against the updated lists), which yields the same final lists.
 #include <algorithm>
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
@@ -26,6 +27,8 @@
 #include "tc_sm100.cuh"
 
 namespace fgim {
+
+namespace cg = cooperative_groups;
 
 static inline long long cdivll(long long a, long long b) { return (a + b - 1) / b; }
 
@@ -82,10 +85,19 @@ __global__ void k_rev_fill(const int32_t* __restrict__ ids, const float* __restr
 
 // the `cap` smallest (delta, source) keys of every reverse segment (warp per vertex), as a set:
 // in segment order when the segment has at most `cap` entries, else ascending
-__global__ void __launch_bounds__(128) k_rev_select(const long long* __restrict__ off, const uint64_t* __restrict__ rev,
-                                                    long long N, int cap, int32_t* __restrict__ top,
-                                                    int32_t* __restrict__ ntop) {
+// (blockIdx.y: the new or the old entries)
+struct RevLists {
+    const long long* off[2];
+    const uint64_t* rev[2];
+    int32_t* top[2];
+    int32_t* ntop[2];
+};
+__global__ void __launch_bounds__(128) k_rev_select(RevLists lists, long long N, int cap) {
     extern __shared__ __align__(16) unsigned char smem[];
+    const long long* __restrict__ off = lists.off[blockIdx.y];
+    const uint64_t* __restrict__ rev = lists.rev[blockIdx.y];
+    int32_t* __restrict__ top = lists.top[blockIdx.y];
+    int32_t* __restrict__ ntop = lists.ntop[blockIdx.y];
     const int warp = threadIdx.x >> 5;
     const int lane = lane_id();
     const long long v = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
@@ -187,18 +199,14 @@ cudaError_t refine_visit(const fgim_knng& g, int rev_cap, RefineBuffers& b, cuda
     const int k = g.k;
     const long long total = N * k;
     cudaError_t e;
-    if ((e = cudaMemsetAsync(b.cntN, 0, sizeof(int32_t) * N, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(b.cntO, 0, sizeof(int32_t) * N, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(b.fillN, 0, sizeof(int32_t) * N, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(b.fillO, 0, sizeof(int32_t) * N, s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(b.cntN, 0, sizeof(int32_t) * 4 * N, s)) != cudaSuccess) return e;   // cntN .. fillO
     const unsigned gb = (unsigned)cdivll(total, 256);
     {
         LaunchScope ls("k_rev_count", s);
         k_rev_count<<<gb, 256, 0, s>>>(g.ids, g.flags, total, b.cntN, b.cntO);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if ((e = scan_counts(b.cntN, N, b.offN, b.scan_tmp, b.scan_bytes, s)) != cudaSuccess) return e;
-    if ((e = scan_counts(b.cntO, N, b.offO, b.scan_tmp, b.scan_bytes, s)) != cudaSuccess) return e;
+    if ((e = scan_counts2(b.cntN, b.cntO, N, b.offN, b.offO, b.scan_tmp, b.scan_bytes, s)) != cudaSuccess) return e;
     {
         LaunchScope ls("k_rev_fill", s);
         k_rev_fill<<<gb, 256, 0, s>>>(g.ids, g.dist, g.flags, total, k, b.offN, b.offO, b.fillN, b.fillO, b.revN,
@@ -209,12 +217,8 @@ cudaError_t refine_visit(const fgim_knng& g, int rev_cap, RefineBuffers& b, cuda
     const unsigned wb = (unsigned)cdivll(N, wpb);
     {
         LaunchScope ls("k_rev_select", s);
-        k_rev_select<<<wb, wpb * 32, (size_t)wpb * rev_cap * 8, s>>>(b.offN, b.revN, N, rev_cap, b.topN, b.ntopN);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    {
-        LaunchScope ls("k_rev_select", s);
-        k_rev_select<<<wb, wpb * 32, (size_t)wpb * rev_cap * 8, s>>>(b.offO, b.revO, N, rev_cap, b.topO, b.ntopO);
+        const RevLists lists = {{b.offN, b.offO}, {b.revN, b.revO}, {b.topN, b.topO}, {b.ntopN, b.ntopO}};
+        k_rev_select<<<dim3(wb, 2), wpb * 32, (size_t)wpb * rev_cap * 8, s>>>(lists, N, rev_cap);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     {
@@ -322,7 +326,7 @@ __global__ void __launch_bounds__(kJThreads, 2) k_join_staged(
     const int32_t* __restrict__ ids, const float* __restrict__ dist, const int32_t* __restrict__ cand,
     const int32_t* __restrict__ nn_arr, const int32_t* __restrict__ no_arr, int cmax, int cm,
     const int32_t* __restrict__ vlist, int32_t* __restrict__ prop_tgt, uint64_t* __restrict__ prop_key,
-    unsigned long long* prop_count, long long prop_cap, uint8_t* __restrict__ pending,
+    unsigned long long* prop_count, long long prop_cap, int32_t* __restrict__ pcnt, uint8_t* __restrict__ pending,
     unsigned long long* pairs_count, unsigned long long* cands_count, int* status) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int tid = threadIdx.x;
@@ -523,6 +527,7 @@ __global__ void __launch_bounds__(kJThreads, 2) k_join_staged(
                             const unsigned long long pos = atomicAdd(prop_count, 1ull);
                             if (pos < (unsigned long long)prop_cap) {
                                 prop_tgt[pos] = cid[a];
+                                atomicAdd(pcnt + (cid[a]), 1);
                                 prop_key[pos] = key;
                             } else {
                                 pending[v] = 1;
@@ -549,6 +554,7 @@ __global__ void __launch_bounds__(kJThreads, 2) k_join_staged(
             const unsigned long long pos = base + i;
             if (pos < (unsigned long long)prop_cap) {
                 prop_tgt[pos] = pb_tgt[i];
+                atomicAdd(pcnt + (pb_tgt[i]), 1);
                 prop_key[pos] = pb_key[i];
             } else {
                 pending[v] = 1;
@@ -818,7 +824,7 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
     const uint8_t* __restrict__ X8, const float4* __restrict__ tcm, const float* __restrict__ inv_norm, int k, const int32_t* __restrict__ ids,
     const uint64_t* __restrict__ wk, const int32_t* __restrict__ cand, const int32_t* __restrict__ nn_arr, const int32_t* __restrict__ no_arr, int cmax,
     int cm, uint32_t tmem_cols, const int32_t* __restrict__ vlist, int32_t* __restrict__ prop_tgt,
-    uint64_t* __restrict__ prop_key, unsigned long long* prop_count, long long prop_cap, uint8_t* __restrict__ pending,
+    uint64_t* __restrict__ prop_key, unsigned long long* prop_count, long long prop_cap, int32_t* __restrict__ pcnt, uint8_t* __restrict__ pending,
     unsigned long long* pairs_count, unsigned long long* cands_count, int* status) {
     constexpr int NT = BYTES ? 256 : 128;   // threads (byte rows: eight warps, two per TMEM lane quarter)
     constexpr int NW = NT / 32;
@@ -1263,6 +1269,7 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
                         const unsigned long long pos = atomicAdd(prop_count, 1ull);
                         if (pos < (unsigned long long)prop_cap) {
                             prop_tgt[pos] = tgt[dir];
+                            atomicAdd(pcnt + (tgt[dir]), 1);
                             prop_key[pos] = key[dir];
                         } else {
                             pending[v] = 1;
@@ -1368,6 +1375,7 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
             const unsigned long long pos = base + q;
             if (pos < (unsigned long long)prop_cap) {
                 prop_tgt[pos] = pb_tgt[q];
+                atomicAdd(pcnt + (pb_tgt[q]), 1);
                 prop_key[pos] = pb_key[q];
             } else {
                 pending[v] = 1;
@@ -1454,7 +1462,7 @@ __global__ void __launch_bounds__(kSparseWarps * 32, 8) k_join_sparse(
     const long long* __restrict__ offN, const uint64_t* __restrict__ revO, const long long* __restrict__ offO,
     const int32_t* __restrict__ cand, const int32_t* __restrict__ nn_arr, const int32_t* __restrict__ no_arr,
     int cmax, int cm, int nnm, const int32_t* __restrict__ vlist, long long nv, int32_t* __restrict__ prop_tgt,
-    uint64_t* __restrict__ prop_key, unsigned long long* prop_count, long long prop_cap,
+    uint64_t* __restrict__ prop_key, unsigned long long* prop_count, long long prop_cap, int32_t* __restrict__ pcnt,
     uint8_t* __restrict__ pending, unsigned long long* pairs_count, unsigned long long* cands_count, int* status) {
     extern __shared__ __align__(16) unsigned char smem_sp[];
     const int lane = lane_id();
@@ -1729,6 +1737,7 @@ __global__ void __launch_bounds__(kSparseWarps * 32, 8) k_join_sparse(
                 const unsigned long long pos = pos0 + (dir == 0 ? __popc(va & lt) : na + __popc(vb & lt));
                 if (pos < (unsigned long long)prop_cap) {
                     prop_tgt[pos] = dir == 0 ? ci : cj;
+                    atomicAdd(pcnt + (dir == 0 ? ci : cj), 1);
                     prop_key[pos] = dir == 0 ? kA : kB;
                 } else {
                     pending[v] = 1;
@@ -1808,7 +1817,9 @@ cudaError_t refine_join(const ShardTable& t, const float* X, const float* inv_no
                         unsigned long long* cands, int* status, cudaStream_t s) {
     for (int q = 0; q < 5; ++q) b.class_count[q] = 0;
     if (nv <= 0) return cudaSuccess;
-    cudaError_t e = cudaSuccess;
+    // the proposals of this run per target (counted as they are written), and their places in the merge
+    cudaError_t e = cudaMemsetAsync(b.pcnt, 0, sizeof(int32_t) * 2 * g.n, s);   // pcnt, pfill
+    if (e != cudaSuccess) return e;
     // the warp-per-vertex form works on byte rows, in the first run of a pass only (its
     // membership bits come from the reverse lists of Visit; a re-run reads merged lists)
     const bool bytes = b.X8 != nullptr && byte_rows_ok(t.dim) && !b.fp8;
@@ -1857,7 +1868,7 @@ cudaError_t refine_join(const ShardTable& t, const float* X, const float* inv_no
         LaunchScope ls("k_join", s);                                                                              \
         k_join_tc<MT, BY, LG, F8><<<(unsigned)count, (BY) ? 256 : kTCThreads, smem, s>>>(                           \
             t, X, reinterpret_cast<const __nv_bfloat16*>(b.Xb), b.dp, b.f16, b.X8, b.tcm, inv_norm, g.k, g.ids, b.wk, b.cand,  \
-            b.nn, b.no, b.cmax, cmq, cols, list, b.prop_tgt, b.prop_key, b.prop_count, b.prop_cap, b.pending,     \
+            b.nn, b.no, b.cmax, cmq, cols, list, b.prop_tgt, b.prop_key, b.prop_count, b.prop_cap, b.pcnt, b.pending,     \
             pairs, cands, status);                                                                                \
         e = cudaGetLastError();                                                                                   \
     } while (0)
@@ -1903,7 +1914,7 @@ cudaError_t refine_join(const ShardTable& t, const float* X, const float* inv_no
         LaunchScope ls("k_join_sparse", s);                                                                       \
         k_join_sparse<MT><<<grid, kSparseWarps * 32, smem, s>>>(                                                  \
             t, b.X8, inv_norm, g.k, g.ids, b.wk, b.revN, b.offN, b.revO, b.offO, b.cand, b.nn, b.no, b.cmax,      \
-            cms, nnm, list, count, b.prop_tgt, b.prop_key, b.prop_count, b.prop_cap, b.pending, pairs, cands,     \
+            cms, nnm, list, count, b.prop_tgt, b.prop_key, b.prop_count, b.prop_cap, b.pcnt, b.pending, pairs, cands,     \
             status);                                                                                              \
         e = cudaGetLastError();                                                                                   \
     } while (0)
@@ -1927,7 +1938,7 @@ cudaError_t refine_join(const ShardTable& t, const float* X, const float* inv_no
         LaunchScope ls("k_join", s);                                                                              \
         k_join_staged<MT, ST><<<(unsigned)nv, kJThreads, smem, s>>>(t, X, inv_norm, g.k, g.ids, g.dist, b.cand,    \
                                                                     b.nn, b.no, b.cmax, cm, vlist, b.prop_tgt,    \
-                                                                    b.prop_key, b.prop_count, b.prop_cap,         \
+                                                                    b.prop_key, b.prop_count, b.prop_cap, b.pcnt, \
                                                                     b.pending, pairs, cands, status);             \
         e = cudaGetLastError();                                                                                   \
     } while (0)
@@ -1945,11 +1956,6 @@ cudaError_t refine_join(const ShardTable& t, const float* X, const float* inv_no
 }
 
 // ---------------------------------------------------------------------------- Merge
-__global__ void k_prop_count(const int32_t* __restrict__ tgt, long long P, int32_t* __restrict__ cnt) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < P) atomicAdd(cnt + tgt[i], 1);
-}
-
 __global__ void k_prop_scatter(const int32_t* __restrict__ tgt, const uint64_t* __restrict__ key, long long P,
                                const long long* __restrict__ off, int32_t* __restrict__ fill,
                                uint64_t* __restrict__ sorted) {
@@ -2011,14 +2017,7 @@ cudaError_t refine_merge(const fgim_knng& g, RefineBuffers& b, long long P, cuda
     if (P <= 0) return cudaSuccess;
     const long long N = g.n;
     cudaError_t e;
-    if ((e = cudaMemsetAsync(b.pcnt, 0, sizeof(int32_t) * N, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(b.pfill, 0, sizeof(int32_t) * N, s)) != cudaSuccess) return e;
     const unsigned gp = (unsigned)cdivll(P, 256);
-    {
-        LaunchScope ls("k_prop_count", s);
-        k_prop_count<<<gp, 256, 0, s>>>(b.prop_tgt, P, b.pcnt);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
     if ((e = scan_counts(b.pcnt, N, b.poff, b.scan_tmp, b.scan_bytes, s)) != cudaSuccess) return e;
     {
         LaunchScope ls("k_prop_scatter", s);
@@ -2068,45 +2067,22 @@ cudaError_t launch_nonzero_flags(const uint8_t* v, long long N, int32_t* flag, c
 // and each was computed on the state the sequential loop would have given it. The
 // rest is recomputed in the next round. The lowest pending index always holds its
 // reservations, so every round commits at least one action.
-enum { kPlan = 0, kCheck = 1, kCommit = 2 };
-
-// Round rho works on the window [ff[rho - 1], min(ff[rho - 1] + W, nz)) and leaves in ff[rho]
-// the first index it did not commit (the next round's start). Reservations carry a tag
+//
+// All rounds run in one cooperative launch, the phases of a round separated by grid-wide barriers (three
+// launches per round, in batches of 16 rounds between host reads, took 0.8 of the 4.4 ms of a 20,000-vertex
+// merge). Round rho works on the window [start, min(start + W, nz)), start = ff[(rho - 1) % 3], and leaves
+// in ff[rho % 3] the first index it did not commit (the next round's start). Reservations carry a tag
 // ordered by (round, index) with later rounds smaller, so owner needs no reset.
 __device__ __forceinline__ unsigned long long round_tag(long long rho, long long i) {
     return ((unsigned long long)(0xFFFFFFFFu - (uint32_t)rho) << 32) | (unsigned long long)(uint32_t)i;
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(128) k_repair_round(int32_t* __restrict__ ids, float* __restrict__ dist,
-                                                      uint8_t* __restrict__ flags, long long N, int k,
-                                                      int32_t* __restrict__ T, const int32_t* __restrict__ zeros,
-                                                      long long nz, long long rho, long long window,
-                                                      long long* __restrict__ ff,
-                                                      unsigned long long* __restrict__ owner,
-                                                      unsigned long long* repaired, int* status) {
-    const int warp = threadIdx.x >> 5;
-    const int lane = lane_id();
-    const long long start = ff[rho - 1];
-    const long long wend = start + window < nz ? start + window : nz;
-    if (MODE == kPlan && blockIdx.x == 0 && threadIdx.x == 0) ff[rho] = wend;
-    const long long i = start + (long long)blockIdx.x * (blockDim.x >> 5) + warp;
-    if (i >= wend) return;
-    if (MODE == kCommit && i >= ff[rho]) return;
-    const unsigned long long tag = round_tag(rho, i);
-    bool ok = true;
-    auto touch = [&](int32_t x) {
-        if (MODE == kPlan) atomicMin(owner + x, tag);
-        else if (MODE == kCheck) ok = ok && owner[x] == tag;
-    };
-    const long long vs = zeros[i];
-    if (vs < 0 || vs >= N) {
-        if (lane == 0) atomicOr(status, kErrBounds);
-        return;
-    }
+// the action of v* = vs (warp): (neighbour v, entry of N(v) replaced, index of v in N(v*), -), v = -1: none;
+// touch(x) is called by one lane for every vertex id x the action reads or writes
+template <typename TOUCH>
+__device__ __forceinline__ int4 repair_plan(const int32_t* ids, const uint8_t* flags, const int32_t* T, long long N,
+                                            int k, long long vs, int lane, TOUCH touch) {
     if (lane == 0) touch((int32_t)vs);
-    int a_sel = -1, best = -1;
-    int32_t v_sel = -1;
     for (int a = 0; a < k; ++a) {
         const int32_t v = ids[vs * k + a];
         if (v < 0 || v >= N) break;
@@ -2125,67 +2101,105 @@ __global__ void __launch_bounds__(128) k_repair_round(int32_t* __restrict__ ids,
             if (m) bst = r * 32 + 31 - __clz(m);
             if (e >= 0 && e < N && (bst < 0 || s >= bst)) touch(e);
         }
-        if (bst >= 0) {
-            a_sel = a;
-            best = bst;
-            v_sel = v;
+        if (bst >= 0) return make_int4(v, bst, a, 0);
+    }
+    return make_int4(-1, -1, -1, 0);
+}
+
+__global__ void __launch_bounds__(kRoundThreads) k_repair(int32_t* ids, float* dist, uint8_t* flags, long long N, int k,
+                                                int32_t* T, const int32_t* __restrict__ zeros,
+                                                const long long* __restrict__ nz_at, long long window, long long* ff,
+                                                unsigned long long* owner, int4* plan, unsigned long long* repaired,
+                                                unsigned long long* zero_count, int* status) {
+    cg::grid_group grid = cg::this_grid();
+    const int lane = lane_id();
+    const long long gw = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
+    const long long nz = *nz_at;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *zero_count = (unsigned long long)nz;
+    long long win = window;
+    for (long long rho = 1;; ++rho) {
+        const long long start = __ldcg(ff + (rho - 1) % 3);   // written before the last barrier
+        if (start >= nz) break;                               // the same for every thread: all leave together
+        if (rho > nz) {   // every round commits at least one action
+            if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, kErrTimeout);
             break;
         }
-    }
-    if (MODE == kCheck) {
-        if (__any_sync(kFull, !ok) && lane == 0) atomicMin((unsigned long long*)(ff + rho), (unsigned long long)i);
-        return;
-    }
-    if (MODE == kCommit && best >= 0 && lane == 0) {
-        int32_t* li = ids + (long long)v_sel * k;
-        float* ld = dist + (long long)v_sel * k;
-        uint8_t* lf = flags + (long long)v_sel * k;
-        const float dvs = dist[vs * k + a_sel];
-        const int32_t old = li[best];
-        T[old] -= 1;
-        T[vs] += 1;
-        const uint64_t key = mkkey(dvs, (int32_t)vs);
-        int pos = best;
-        while (pos > 0 && mkkey(ld[pos - 1], li[pos - 1]) > key) {
-            li[pos] = li[pos - 1];
-            ld[pos] = ld[pos - 1];
-            lf[pos] = lf[pos - 1];
-            --pos;
+        const long long wend = start + win < nz ? start + win : nz;
+        if (blockIdx.x == 0 && threadIdx.x == 0) ff[rho % 3] = wend;
+        for (long long i = start + gw; i < wend; i += nw) {
+            const long long vs = zeros[i];
+            if (vs < 0 || vs >= N) {
+                if (lane == 0) {
+                    atomicOr(status, kErrBounds);
+                    plan[i - start] = make_int4(-1, -1, -1, 0);
+                }
+                continue;
+            }
+            const unsigned long long tag = round_tag(rho, i);
+            const int4 pl = repair_plan(ids, flags, T, N, k, vs, lane, [&](int32_t x) { atomicMin(owner + x, tag); });
+            if (lane == 0) plan[i - start] = pl;
         }
-        while (pos + 1 < k && li[pos + 1] >= 0 && mkkey(ld[pos + 1], li[pos + 1]) < key) {
-            li[pos] = li[pos + 1];
-            ld[pos] = ld[pos + 1];
-            lf[pos] = lf[pos + 1];
-            ++pos;
+        grid.sync();
+        for (long long i = start + gw; i < wend; i += nw) {
+            const long long vs = zeros[i];
+            if (vs < 0 || vs >= N) continue;
+            const unsigned long long tag = round_tag(rho, i);
+            bool ok = true;
+            repair_plan(ids, flags, T, N, k, vs, lane, [&](int32_t x) { ok = ok && __ldcg(owner + x) == tag; });
+            if (__any_sync(kFull, !ok) && lane == 0)
+                atomicMin((unsigned long long*)(ff + rho % 3), (unsigned long long)i);
         }
-        li[pos] = (int32_t)vs;
-        ld[pos] = dvs;
-        lf[pos] = FGIM_FLAG_NEW | FGIM_FLAG_REPLACED;
-        atomicAdd(repaired, 1ull);
+        grid.sync();
+        const long long cend = __ldcg(ff + rho % 3);
+        win = round_window(cend - start, window);
+        for (long long i = start + gw * 32 + lane; i < cend; i += nw * 32) {   // disjoint vertices: one thread each
+            const int4 pl = plan[i - start];
+            if (pl.x < 0) continue;
+            const long long vs = zeros[i];
+            int32_t* li = ids + (long long)pl.x * k;
+            float* ld = dist + (long long)pl.x * k;
+            uint8_t* lf = flags + (long long)pl.x * k;
+            const float dvs = dist[vs * k + pl.z];
+            const int32_t old = li[pl.y];
+            T[old] -= 1;
+            T[vs] += 1;
+            const uint64_t key = mkkey(dvs, (int32_t)vs);
+            int pos = pl.y;
+            while (pos > 0 && mkkey(ld[pos - 1], li[pos - 1]) > key) {
+                li[pos] = li[pos - 1];
+                ld[pos] = ld[pos - 1];
+                lf[pos] = lf[pos - 1];
+                --pos;
+            }
+            while (pos + 1 < k && li[pos + 1] >= 0 && mkkey(ld[pos + 1], li[pos + 1]) < key) {
+                li[pos] = li[pos + 1];
+                ld[pos] = ld[pos + 1];
+                lf[pos] = lf[pos + 1];
+                ++pos;
+            }
+            li[pos] = (int32_t)vs;
+            ld[pos] = dvs;
+            lf[pos] = FGIM_FLAG_NEW | FGIM_FLAG_REPLACED;
+            atomicAdd(repaired, 1ull);
+        }
+        grid.sync();
     }
 }
 
-cudaError_t launch_repair_rounds(fgim_knng& g, int32_t* T, const int32_t* zeros, long long nz, long long rho0,
-                                 int rounds, long long* ff, unsigned long long* owner, unsigned long long* repaired,
-                                 int* status, cudaStream_t s) {
-    cudaError_t e = cudaSuccess;
-    const int wpb = 4;
-    const long long window = kRepairWindow;
-    const unsigned blocks = (unsigned)cdivll(window, wpb);
-    for (int q = 0; q < rounds; ++q) {
-        const long long rho = rho0 + q;
-        LaunchScope ls("k_repair_round", s);
-        k_repair_round<kPlan><<<blocks, wpb * 32, 0, s>>>(g.ids, g.dist, g.flags, g.n, g.k, T, zeros, nz, rho, window,
-                                                          ff, owner, repaired, status);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_repair_round<kCheck><<<blocks, wpb * 32, 0, s>>>(g.ids, g.dist, g.flags, g.n, g.k, T, zeros, nz, rho,
-                                                           window, ff, owner, repaired, status);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_repair_round<kCommit><<<blocks, wpb * 32, 0, s>>>(g.ids, g.dist, g.flags, g.n, g.k, T, zeros, nz, rho,
-                                                            window, ff, owner, repaired, status);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    return e;
+cudaError_t launch_repair(fgim_knng& g, int32_t* T, const int32_t* zeros, const long long* nz, long long* ff,
+                          unsigned long long* owner, int4* plan, unsigned long long* repaired,
+                          unsigned long long* zero_count, int* status, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(owner, 0xff, sizeof(unsigned long long) * g.n, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ff, 0, sizeof(long long), s);
+    int blocks = 0;
+    if (e == cudaSuccess) e = coop_grid(k_repair, kRoundThreads, cdivll(std::min<long long>(kRepairWindow, g.n), kRoundThreads / 32), &blocks);
+    if (e != cudaSuccess) return e;
+    long long N = g.n, window = kRepairWindow;
+    int k = g.k;
+    LaunchScope ls("k_repair", s);
+    void* args[] = {&g.ids, &g.dist, &g.flags, &N, &k, &T, &zeros, &nz, &window, &ff, &owner, &plan, &repaired, &zero_count, &status};
+    return cudaLaunchCooperativeKernel((const void*)k_repair, dim3(blocks), dim3(kRoundThreads), args, 0, s);
 }
 
 }  // namespace fgim

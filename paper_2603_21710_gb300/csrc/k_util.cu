@@ -1,4 +1,5 @@
-// Small building blocks: exclusive scans, compaction by flags, fills, inverse norms.
+// Small building blocks: exclusive scans (two launches: the tiles' sums, then every block adds up the sums
+// before its own; five launches before, most of a small merge's launches), compaction by flags, fills, inverse norms.
 #include <algorithm>
 
 #include "fgim_launch.h"
@@ -8,93 +9,164 @@ namespace fgim {
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 8;
 constexpr long long kScanTile = (long long)kScanThreads * kScanItems;
+// blocks up to which a block adds up the sums of all blocks before it by itself (8M entries); above, the block
+// sums are scanned first
+constexpr long long kScanFlat = 4096;
 
-template <typename TIN>
-__global__ void __launch_bounds__(kScanThreads) k_scan_block(const TIN* __restrict__ in, long long n,
-                                                             long long* __restrict__ out,
-                                                             long long* __restrict__ bsum) {
-    __shared__ long long sh[kScanThreads];
-    const int tid = threadIdx.x;
-    const long long base = (long long)blockIdx.x * kScanTile + (long long)tid * kScanItems;
-    long long v[kScanItems];
+// sum of v over the block, in every thread (sh: 8 words); a second call needs a barrier in between
+__device__ __forceinline__ long long block_sum(long long v, long long* sh) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    long long s = 0;
+#pragma unroll
+    for (int w = 0; w < kScanThreads / 32; ++w) s += sh[w];
+    return s;
+}
+
+// One or two arrays (blockIdx.y) are scanned at once.
+struct ScanJob {
+    const int32_t* in[2];
+    long long* out[2];
+};
+
+// sums[y * gridDim.x + b] = the sum of tile b of array y
+__global__ void __launch_bounds__(kScanThreads) k_scan_sums(ScanJob job, long long n, long long* __restrict__ sums) {
+    __shared__ long long sh[kScanThreads / 32];
+    const int32_t* in = job.in[blockIdx.y];
+    const long long base = (long long)blockIdx.x * kScanTile;
     long long s = 0;
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i) {
-        const long long idx = base + i;
-        v[i] = idx < n ? (long long)in[idx] : 0;
-        s += v[i];
+        const long long idx = base + i * kScanThreads + threadIdx.x;
+        if (idx < n) s += in[idx];
     }
-    sh[tid] = s;
-    __syncthreads();
-    for (int off = 1; off < kScanThreads; off <<= 1) {
-        long long add = tid >= off ? sh[tid - off] : 0;
-        __syncthreads();
-        sh[tid] += add;
-        __syncthreads();
+    s = block_sum(s, sh);
+    if (threadIdx.x == 0) sums[(long long)blockIdx.y * gridDim.x + blockIdx.x] = s;
+}
+
+// out = exclusive prefix sums of in, out[n] = the total. FLAT: pre holds the tiles' sums, and each block adds
+// up those before its own; else pre holds their exclusive prefix sums.
+template <bool FLAT>
+__global__ void __launch_bounds__(kScanThreads) k_scan_write(ScanJob job, long long n, const long long* __restrict__ pre) {
+    __shared__ long long sh[kScanThreads / 32];
+    __shared__ long long warp_sum[kScanThreads / 32];
+    const int32_t* in = job.in[blockIdx.y];
+    long long* out = job.out[blockIdx.y];
+    const long long* p = pre + (long long)blockIdx.y * gridDim.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    long long before = 0;
+    if (FLAT) {
+        for (long long b = tid; b < blockIdx.x; b += kScanThreads) before += p[b];
+        before = block_sum(before, sh);
+    } else {
+        before = p[blockIdx.x];
     }
-    long long run = sh[tid] - s;
+    const long long base = (long long)blockIdx.x * kScanTile + (long long)tid * kScanItems;
+    int32_t v[kScanItems];
+    long long s = 0;
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i) {
-        const long long idx = base + i;
-        if (idx < n) out[idx] = run;
-        run += v[i];
+        v[i] = base + i < n ? in[base + i] : 0;
+        s += v[i];
     }
-    if (tid == kScanThreads - 1) bsum[blockIdx.x] = sh[tid];
+    long long inc = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) warp_sum[warp] = inc;
+    __syncthreads();
+    long long run = before + inc - s;
+#pragma unroll
+    for (int w = 0; w < kScanThreads / 32; ++w)
+        if (w < warp) run += warp_sum[w];
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+        if (base + i < n) out[base + i] = run;
+        run += v[i];
+        if (base + i == n - 1) out[n] = run;
+    }
 }
 
-__global__ void k_scan_add(long long* __restrict__ out, long long n, const long long* __restrict__ boff) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] += boff[i / kScanTile];
+// exclusive prefix sums of n words by one block (the tiles' sums of very long arrays)
+__global__ void __launch_bounds__(kScanThreads) k_scan_one(const long long* __restrict__ in, long long n,
+                                                           long long* __restrict__ out) {
+    __shared__ long long warp_sum[kScanThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    long long carry = 0;
+    for (long long b = 0; b < n; b += kScanThreads) {
+        const long long v = b + tid < n ? in[b + tid] : 0;
+        long long inc = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long y = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) warp_sum[warp] = inc;
+        __syncthreads();
+        long long run = carry + inc - v;
+#pragma unroll
+        for (int w = 0; w < kScanThreads / 32; ++w) {
+            if (w < warp) run += warp_sum[w];
+            carry += warp_sum[w];
+        }
+        if (b + tid < n) out[b + tid] = run;
+        __syncthreads();
+    }
 }
-
-__global__ void k_copy1(long long* dst, const long long* src) { *dst = *src; }
 
 static long long cdiv(long long a, long long b) { return (a + b - 1) / b; }
 
-size_t scan_scratch_bytes(long long n) {
-    size_t words = 0;
-    long long m = n;
-    do {
-        long long blocks = cdiv(m > 0 ? m : 1, kScanTile);
-        words += 2 * blocks + 1;
-        m = blocks;
-    } while (m > 1);
-    return (words + 8) * sizeof(long long);
-}
+size_t scan_scratch_bytes(long long n) { return (size_t)(4 * cdiv(n > 0 ? n : 1, kScanTile) + 8) * sizeof(long long); }
 
-template <typename TIN>
-static cudaError_t scan_impl(const TIN* in, long long n, long long* out, long long* scratch, cudaStream_t s) {
-    const long long blocks = cdiv(n > 0 ? n : 1, kScanTile);
-    long long* bsum = scratch;
-    long long* boff = scratch + blocks;
+static cudaError_t scan_job(const ScanJob& job, int arrays, long long n, long long* scratch, cudaStream_t s) {
+    if (n <= 0) {
+        for (int y = 0; y < arrays; ++y) {
+            const cudaError_t e = cudaMemsetAsync(job.out[y], 0, sizeof(long long), s);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
+    const long long blocks = cdiv(n, kScanTile);
+    const dim3 grid((unsigned)blocks, (unsigned)arrays);
     {
-        LaunchScope ls("k_scan_block", s);
-        k_scan_block<TIN><<<(unsigned)blocks, kScanThreads, 0, s>>>(in, n, out, bsum);
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (blocks == 1) {
-        LaunchScope ls("k_copy1", s);
-        k_copy1<<<1, 1, 0, s>>>(out + n, bsum);
-        return cudaGetLastError();
-    }
-    e = scan_impl<long long>(bsum, blocks, boff, scratch + 2 * blocks + 1, s);
-    if (e != cudaSuccess) return e;
-    if (n > 0) {
-        LaunchScope ls("k_scan_add", s);
-        k_scan_add<<<(unsigned)cdiv(n, 256), 256, 0, s>>>(out, n, boff);
-        e = cudaGetLastError();
+        LaunchScope ls("k_scan_sums", s);
+        k_scan_sums<<<grid, kScanThreads, 0, s>>>(job, n, scratch);
+        const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    LaunchScope ls("k_copy1", s);
-    k_copy1<<<1, 1, 0, s>>>(out + n, boff + blocks);
+    if (blocks <= kScanFlat) {
+        LaunchScope ls("k_scan_write", s);
+        k_scan_write<true><<<grid, kScanThreads, 0, s>>>(job, n, scratch);
+        return cudaGetLastError();
+    }
+    long long* pre = scratch + arrays * blocks;
+    for (int y = 0; y < arrays; ++y) {
+        LaunchScope ls("k_scan_one", s);
+        k_scan_one<<<1, kScanThreads, 0, s>>>(scratch + y * blocks, blocks, pre + y * blocks);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    LaunchScope ls("k_scan_write", s);
+    k_scan_write<false><<<grid, kScanThreads, 0, s>>>(job, n, pre);
     return cudaGetLastError();
 }
 
 cudaError_t scan_counts(const int32_t* in, long long n, long long* out, void* scratch, size_t scratch_bytes,
                         cudaStream_t s) {
     if (scratch_bytes < scan_scratch_bytes(n)) return cudaErrorInvalidValue;
-    return scan_impl<int32_t>(in, n, out, reinterpret_cast<long long*>(scratch), s);
+    const ScanJob job = {{in, nullptr}, {out, nullptr}};
+    return scan_job(job, 1, n, reinterpret_cast<long long*>(scratch), s);
+}
+
+cudaError_t scan_counts2(const int32_t* in0, const int32_t* in1, long long n, long long* out0, long long* out1,
+                         void* scratch, size_t scratch_bytes, cudaStream_t s) {
+    if (scratch_bytes < scan_scratch_bytes(n)) return cudaErrorInvalidValue;
+    const ScanJob job = {{in0, in1}, {out0, out1}};
+    return scan_job(job, 2, n, reinterpret_cast<long long*>(scratch), s);
 }
 
 __global__ void k_compact(const int32_t* __restrict__ flag, long long n, const long long* __restrict__ off,
