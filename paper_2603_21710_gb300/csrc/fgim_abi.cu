@@ -202,23 +202,23 @@ static inline void need(bool ok, fgim_status st, const char* what) {
 // counters on the device: [0] ndc, [1] hops, [2] pairs, [3] repaired, [4] attached, [5] candidates joined,
 // [6] zero-indegree vertices of the last repair, [8] the beam searches' item counter
 struct Ctx {
+    static constexpr int kCtxWords = 18;
     cudaStream_t s;
     Scratch sc;
     int* status = nullptr;
     unsigned long long* ctr = nullptr;
     long long* host = nullptr;   // pinned readback slot
     explicit Ctx(cudaStream_t st) : s(st), sc(st) {
-        status = sc.alloc<int>(4);
-        ctr = sc.alloc<unsigned long long>(16);
+        ctr = sc.alloc<unsigned long long>(kCtxWords);   // 16 counters, then the status words
         need(sc.ok(), FGIM_ENOMEM, "scratch allocation failed");
-        ck(cudaMemsetAsync(status, 0, 4 * sizeof(int), s));
-        ck(cudaMemsetAsync(ctr, 0, 16 * sizeof(unsigned long long), s));
+        status = reinterpret_cast<int*>(ctr + 16);
+        ck(cudaMemsetAsync(ctr, 0, kCtxWords * sizeof(unsigned long long), s));
         const int hop_budget = g_test_hop_budget.load(std::memory_order_relaxed);
         if (hop_budget > 0)   // status[1]: the beam searches' expansion budget (test hook)
             ck(cudaMemcpyAsync(status + 1, &hop_budget, sizeof(int), cudaMemcpyHostToDevice, s));
         host = pinned_slot();
     }
-    // One pinned 128-byte readback slot per host thread, made once and kept for the thread's
+    // One pinned 512-byte readback slot per host thread, made once and kept for the thread's
     // life: pinning and releasing host memory on every call costs milliseconds now and then
     // (and the release synchronizes the device).
     static long long* pinned_slot() {
@@ -229,7 +229,7 @@ struct Ctx {
             }
         };
         thread_local Slot slot;
-        if (!slot.p) ck(cudaMallocHost(&slot.p, 128));
+        if (!slot.p) ck(cudaMallocHost(&slot.p, 512));
         return slot.p;
     }
     template <typename T>
@@ -255,11 +255,11 @@ struct Ctx {
     }
     // drain the stream, then report device-side errors and counters
     void finish(fgim_stats* st) {
+        // counters and status in one copy to the pinned slot, one synchronization
+        unsigned long long* hc = reinterpret_cast<unsigned long long*>(host + 16);
+        ck(cudaMemcpyAsync(hc, ctr, kCtxWords * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
         ck(cudaStreamSynchronize(s));
-        int hs[4];
-        unsigned long long hc[16];
-        ck(cudaMemcpy(hs, status, sizeof(hs), cudaMemcpyDeviceToHost));
-        ck(cudaMemcpy(hc, ctr, sizeof(hc), cudaMemcpyDeviceToHost));
+        const int* hs = reinterpret_cast<const int*>(hc + 16);
         if (st) {
             st->ndc += (int64_t)hc[0];
             st->hops += (int64_t)hc[1];
@@ -576,7 +576,7 @@ static RefineBuffers refine_buffers(Ctx& c, const Problem& P, const fgim_params*
     b.scan_bytes = scan_scratch_bytes(N);
     b.scan_tmp = c.alloc<unsigned char>((long long)b.scan_bytes);
     b.max_nc = c.alloc<int32_t>(12);
-    b.host_i32 = reinterpret_cast<int32_t*>(c.host + 4);   // 24 ints of the 128-byte pinned slot
+    b.host_i32 = reinterpret_cast<int32_t*>(c.host + 4);   // 24 ints of the pinned slot
     b.blist = c.alloc<int32_t>(4 * N);
     b.wk = c.alloc<uint64_t>(N);
     b.blist_cap = N;
@@ -1426,6 +1426,74 @@ fgim_status fgim_build_pg(const void* vectors, int64_t n, int32_t dim, int32_t d
 }
 
 
+}  // extern "C"
+
+// Alg. 1 for nq queries over a graph, with or without HNSW layers above it (live: the non-empty ones, top first)
+static void search_graph(Ctx& c, const void* base, long long n, int dim, int dtype, int metric, const int32_t* graph_ids,
+                         int R, const fgim_layer* live, int n_live, int entry, const void* queries, int nq, int topk,
+                         int beam, int ef_up, int32_t* out_ids, float* out_dist, int32_t* out_start) {
+    // wide BF16 rows are read as they are; others are decoded first
+    const bool wide16 = dtype == FGIM_BF16 && dim > 128 && ((uintptr_t)base & 7u) == 0;
+    const uint16_t* Xh = dtype == FGIM_BF16 ? static_cast<const uint16_t*>(base) : nullptr;
+    const float* X = nullptr;
+    const bool few = n_live > 0 ? nq <= kTeamLayered : dim > 128 && nq <= kTeamQueries;
+    if (few && !(wide16 && ((uintptr_t)queries & 7u) != 0)) {   // one block per query, the layers in the same launch
+        const void* rows = base;
+        const void* Q = queries;
+        if (dtype == FGIM_BF16 && !wide16) {
+            rows = f32_rows(c, base, n, dim, dtype);
+            Q = f32_rows(c, queries, nq, dim, dtype);
+        }
+        TeamLayers ls;
+        ls.count = n_live;
+        for (int i = 0; i < n_live; ++i) ls.l[i] = {live[i].members, live[i].adj, (int)live[i].n, live[i].M};
+        ck(launch_search_team(rows, wide16, nullptr, n, dim, metric, graph_ids, R, entry, nullptr, ls, ef_up, Q,
+                              nullptr, nq, topk, beam, out_ids, out_dist, out_start, c.ctr + 0, c.status, c.s));
+        return;
+    }
+    if (!wide16 || n_live > 0) X = f32_rows(c, base, n, dim, dtype);
+    const float* Q = f32_rows(c, queries, nq, dim, dtype);
+    float* inv = nullptr;
+    float* qinv = nullptr;
+    if (metric == FGIM_COSINE) {
+        inv = c.alloc<float>(n);
+        qinv = c.alloc<float>(nq);
+        if (X) ck(launch_inv_norms(X, n, dim, inv, c.s));
+        else ck(launch_inv_norms_bf16(Xh, n, dim, inv, c.s));
+        ck(launch_inv_norms(Q, nq, dim, qinv, c.s));
+    }
+    int32_t* start = nullptr;
+    if (out_start || n_live > 0) {
+        start = out_start ? out_start : c.alloc<int32_t>(nq);
+        int32_t* qpos = c.alloc<int32_t>(nq);
+        int32_t* best = c.alloc<int32_t>(nq);
+        float* bdist = c.alloc<float>(nq);
+        // every query starts at the entry's position in the top layer; each layer is searched
+        // with Alg. 1 (pool ef_up) and its nearest result starts the layer below
+        ck(launch_hnsw_next(nullptr, nullptr, 0, n_live ? live[0].members : nullptr, n_live ? live[0].n : 0, nq, 1, entry,
+                            qpos, start, c.status, c.s));
+        for (int i = 0; i < n_live; ++i) {
+            const fgim_layer& ly = live[i];
+            float* Xl = c.alloc<float>(ly.n * dim);
+            ck(launch_gather_rows(X, ly.members, ly.n, dim, Xl, c.s));
+            float* invl = nullptr;
+            if (metric == FGIM_COSINE) {
+                invl = c.alloc<float>(ly.n);
+                ck(launch_inv_norms(Xl, ly.n, dim, invl, c.s));
+            }
+            ck(launch_search(Xl, nullptr, invl, ly.n, dim, metric, ly.adj, ly.M, 0, Q, qinv, nullptr, nq, 1, ef_up, best,
+                             bdist, c.ctr + 0, c.status, c.s, nullptr, qpos));
+            const fgim_layer* nx = i + 1 < n_live ? &live[i + 1] : nullptr;
+            ck(launch_hnsw_next(best, ly.members, ly.n, nx ? nx->members : nullptr, nx ? nx->n : 0, nq, 0, entry, qpos,
+                                start, c.status, c.s));
+        }
+    }
+    ck(launch_search(X, nullptr, inv, n, dim, metric, graph_ids, R, entry, Q, qinv, nullptr, nq, topk, beam, out_ids,
+                     out_dist, c.ctr + 0, c.status, c.s, wide16 ? Xh : nullptr, start));
+}
+
+extern "C" {
+
 fgim_status fgim_search_hnsw(const void* base, int64_t n, int32_t dim, int32_t dtype, int32_t metric,
                              const int32_t* graph_ids, int32_t R, const fgim_layer* layers, int32_t n_layers,
                              int32_t entry, const void* queries, int32_t nq, int32_t topk, int32_t beam, int32_t ef_up,
@@ -1455,46 +1523,10 @@ fgim_status fgim_search_hnsw(const void* base, int64_t n, int32_t dim, int32_t d
         }
         if (nq == 0) return;
         Ctx c((cudaStream_t)stream);
-        const float* X = f32_rows(c, base, n, dim, dtype);
-        const float* Q = f32_rows(c, queries, nq, dim, dtype);
-        float* inv = nullptr;
-        float* qinv = nullptr;
-        if (metric == FGIM_COSINE) {
-            inv = c.alloc<float>(n);
-            qinv = c.alloc<float>(nq);
-            ck(launch_inv_norms(X, n, dim, inv, c.s));
-            ck(launch_inv_norms(Q, nq, dim, qinv, c.s));
-        }
-        int32_t* start = out_start ? out_start : c.alloc<int32_t>(nq);
-        int32_t* qpos = c.alloc<int32_t>(nq);
-        int32_t* best = c.alloc<int32_t>(nq);
-        float* bdist = c.alloc<float>(nq);
-        if (live.empty()) {
-            ck(launch_hnsw_next(nullptr, nullptr, 0, nullptr, 0, nq, 1, entry, qpos, start, c.status, c.s));
-        } else {
-            // every query starts at the entry's position in the top layer; each layer is searched
-            // with Alg. 1 (pool ef_up) and its nearest result starts the layer below
-            const fgim_layer& t0 = layers[live[0]];
-            ck(launch_hnsw_next(nullptr, nullptr, 0, t0.members, t0.n, nq, 1, entry, qpos, start, c.status, c.s));
-            for (size_t i = 0; i < live.size(); ++i) {
-                const fgim_layer& ly = layers[live[i]];
-                float* Xl = c.alloc<float>(ly.n * dim);
-                ck(launch_gather_rows(X, ly.members, ly.n, dim, Xl, c.s));
-                float* invl = nullptr;
-                if (metric == FGIM_COSINE) {
-                    invl = c.alloc<float>(ly.n);
-                    ck(launch_inv_norms(Xl, ly.n, dim, invl, c.s));
-                }
-                ck(launch_search(Xl, nullptr, invl, ly.n, dim, metric, ly.adj, ly.M, 0, Q, qinv, nullptr, nq, 1, ef_up,
-                                 best, bdist, c.ctr + 0, c.status, c.s, nullptr, qpos));
-                const fgim_layer* nx = i + 1 < live.size() ? &layers[live[i + 1]] : nullptr;
-                ck(launch_hnsw_next(best, ly.members, ly.n, nx ? nx->members : nullptr, nx ? nx->n : 0, nq, 0, entry,
-                                    qpos, start, c.status, c.s));
-            }
-        }
-        ck(launch_search(X, nullptr, inv, n, dim, metric, graph_ids, R, entry, Q, qinv, nullptr, nq, topk, beam, out_ids,
-                         out_dist, c.ctr + 0, c.status, c.s,
-                         dtype == FGIM_BF16 ? static_cast<const uint16_t*>(base) : nullptr, start));
+        std::vector<fgim_layer> lv;
+        for (int l : live) lv.push_back(layers[l]);
+        search_graph(c, base, n, dim, dtype, metric, graph_ids, R, lv.data(), (int)lv.size(), entry, queries, nq, topk, beam,
+                     ef_up, out_ids, out_dist, out_start);
         c.finish(&t_stats);
     });
     end_call();
@@ -1520,27 +1552,8 @@ fgim_status fgim_search(const void* base, int64_t n, int32_t dim, int32_t dtype,
              "vectors must be 16-byte (FP32) or 2-byte (BF16) aligned");
         if (nq == 0) return;
         Ctx c((cudaStream_t)stream);
-        const float* X = static_cast<const float*>(base);
-        const float* Q = static_cast<const float*>(queries);
-        if (dtype == FGIM_BF16) {
-            float* Xf = c.alloc<float>(n * dim);
-            float* Qf = c.alloc<float>((long long)nq * dim);
-            ck(launch_bf16_to_f32(static_cast<const uint16_t*>(base), n * dim, Xf, c.s));
-            ck(launch_bf16_to_f32(static_cast<const uint16_t*>(queries), (long long)nq * dim, Qf, c.s));
-            X = Xf;
-            Q = Qf;
-        }
-        float* inv = nullptr;
-        float* qinv = nullptr;
-        if (metric == FGIM_COSINE) {
-            inv = c.alloc<float>(n);
-            qinv = c.alloc<float>(nq);
-            ck(launch_inv_norms(X, n, dim, inv, c.s));
-            ck(launch_inv_norms(Q, nq, dim, qinv, c.s));
-        }
-        ck(launch_search(X, nullptr, inv, n, dim, metric, graph_ids, R, entry, Q, qinv, nullptr, nq, topk, beam, out_ids,
-                         out_dist, c.ctr + 0, c.status, c.s,
-                         dtype == FGIM_BF16 ? static_cast<const uint16_t*>(base) : nullptr));
+        search_graph(c, base, n, dim, dtype, metric, graph_ids, R, nullptr, 0, entry, queries, nq, topk, beam, 1, out_ids,
+                     out_dist, nullptr);
         c.finish(&t_stats);
     });
     end_call();

@@ -23,6 +23,32 @@ cudaError_t launch_search(const float* X, const uint8_t* X8, const float* inv_no
                           const int32_t* qids, long long nq, int topk, int L, int32_t* out_ids, float* out_dist,
                           unsigned long long* counters, int* status, cudaStream_t s, const uint16_t* Xh = nullptr,
                           const int32_t* qentry = nullptr);
+// ---- k_team.cu: one block per query (few queries). X and Q: FP32 rows, or BF16 ones (bf16: d > 128,
+// 8-byte aligned); Q == nullptr: queries are the rows qids of X; inv_norm == nullptr (cosine): formed from the rows.
+// layers: the non-empty HNSW layers, top first (count 0: the search starts at `entry`), searched with pool ef_up
+constexpr int kTeamThreads = 256;            // half of them above kTeamWide queries
+constexpr long long kTeamWide = 304;         // two blocks per SM
+// Queries up to which a block each is faster than a warp each. Wide rows (100k, d = 768 BF16, cosine): 100
+// queries 0.74 -> 0.33 ms, 300: 0.69 -> 0.38, 1,000: 0.73 and 0.69 (and the FP32 d = 960 form slower). Rows of up to
+// 128 coordinates: never (one query 0.122 and 0.132 ms, 1,000: 0.26 and 0.31): there the leader's own steps
+// are the chain. With HNSW layers the single launch counts: 1,001 queries over six layers 0.34 -> 0.25 ms.
+constexpr long long kTeamQueries = 608;
+constexpr long long kTeamLayered = 1216;
+struct TeamLayer {
+    const int32_t* members;
+    const int32_t* adj;
+    int n;
+    int M;
+};
+struct TeamLayers {
+    TeamLayer l[FGIM_MAX_LEVELS];
+    int count;
+};
+cudaError_t launch_search_team(const void* X, bool bf16, const float* inv_norm, long long n, int d, int metric,
+                               const int32_t* graph, int R, int entry, const int32_t* qentry, const TeamLayers& layers,
+                               int ef_up, const void* Q, const int32_t* qids, long long nq, int topk, int L, int32_t* out_ids,
+                               float* out_dist, int32_t* out_start, unsigned long long* counters, int* status,
+                               cudaStream_t s);
 // X8[i] = X[i] as a byte; *flag |= 1 unless every X[i] is an integer in [0, 255] (n_elems % 4 == 0)
 cudaError_t launch_narrow_u8(const float* X, long long n_elems, uint8_t* X8, int* flag, cudaStream_t s);
 
@@ -60,6 +86,8 @@ cudaError_t scan_counts2(const int32_t* in0, const int32_t* in1, long long n, lo
                          void* scratch, size_t scratch_bytes, cudaStream_t s);   // two arrays of n at once
 size_t scan_scratch_bytes(long long n);
 cudaError_t launch_inv_norms(const float* X, long long n, int d, float* inv, cudaStream_t s);
+// the same of BF16 rows (8-byte aligned), without an FP32 copy
+cudaError_t launch_inv_norms_bf16(const uint16_t* X, long long n, int d, float* inv, cudaStream_t s);
 // out[i] = the FP32 value of the bfloat16 encoding in[i]
 cudaError_t launch_bf16_to_f32(const uint16_t* in, long long n, float* out, cudaStream_t s);
 // flag[i] = (mask == nullptr || mask[i] != 0)

@@ -131,6 +131,35 @@ __device__ __forceinline__ Query load_query(const float* __restrict__ src, float
     return Q;
 }
 
+// one row as the query of rows_delta (the values of load_query, read from the row storage in use)
+template <bool SMALLD, typename RT>
+__device__ __forceinline__ Query row_query(const RT* __restrict__ row, float* qs, int d, int lane) {
+    Query Q;
+    if constexpr (sizeof(RT) == 1) {
+        const int lsh = byte_lanes_log2(d);
+        const int part = lane & ((1 << lsh) - 1);
+        Q.w = make_uint4(0u, 0u, 0u, 0u);
+        if (part < (d >> 4)) Q.w = reinterpret_cast<const uint4*>(row)[part];
+        uint32_t s = __dp4a(Q.w.x, Q.w.x, 0u);
+        s = __dp4a(Q.w.y, Q.w.y, s);
+        s = __dp4a(Q.w.z, Q.w.z, s);
+        s = __dp4a(Q.w.w, Q.w.w, s);
+        Q.q2 = row_group_sum(s, lsh);
+    } else if constexpr (SMALLD) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int c = (lane & 7) + 8 * i;
+            Q.c[i] = c < (d >> 2) ? row_chunk(row, c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    } else {
+        float4* q4 = reinterpret_cast<float4*>(qs);
+        for (int c = lane; c < (d >> 2); c += 32) q4[c] = row_chunk(row, c);
+        Q.q = qs;
+        __syncwarp();
+    }
+    return Q;
+}
+
 // The sums of four partials per lane over the eight lanes of a row (offsets 4, 2, 1, the last
 // three levels of the butterfly), all four together: each exchange step halves the values a lane
 // keeps, so lane p of row group s ends with the total of partial p / 2. Lane r then takes the total of
@@ -306,6 +335,71 @@ __device__ __forceinline__ float rows_delta(const RT* __restrict__ base, const i
     }
 }
 
+constexpr int kPoolSlots = 4;
+__host__ __device__ inline int pool_entries(int L) { return L <= 32 ? 32 : L <= 64 ? 64 : 128; }
+
+// the id of the pool's first entry not yet expanded (slot, lane src, low word lo), or -1
+template <int MAXS>
+__device__ __forceinline__ int pool_next(const uint64_t (&pk)[MAXS], int& slot, int& src, uint32_t& lo) {
+    slot = -1;
+    unsigned open = 0u;
+#pragma unroll
+    for (int s = 0; s < MAXS; ++s) {
+        if (slot < 0) {
+            open = __ballot_sync(kFull, ((uint32_t)pk[s] & 1u) == 0u);
+            if (open) slot = s;
+        }
+    }
+    if (slot < 0) return -1;
+    src = __ffs(open) - 1;
+    lo = (uint32_t)pk[0];
+#pragma unroll
+    for (int s = 1; s < MAXS; ++s)
+        if (slot == s) lo = (uint32_t)pk[s];
+    return (int)(__shfl_sync(kFull, lo, src) >> 1);
+}
+
+// One candidate key per lane (the empty key: none) into the pool of beam_search: those that beat entry
+// L - 1 enter together. pk and pool: the pool's registers and its copy in shared memory.
+template <int MAXS>
+__device__ __forceinline__ void pool_insert(uint64_t (&pk)[MAXS], uint64_t* pool, uint64_t cand, int L, int lane) {
+    bool valid = cand < pool[L - 1];
+    __syncwarp();
+    if (__ballot_sync(kFull, valid) == 0u) return;
+    // rank of the candidate among the pool's entries: halving steps over its 32, 64 or 128
+    // slots (a valid candidate ranks below the last one: it beats entry L - 1). An entry
+    // equal but for the mark means it is pooled already (the lossy table let it in).
+    int pos = 0;
+#pragma unroll
+    for (int st = 16 * MAXS; st > 0; st >>= 1)
+        if (pool[pos + st - 1] < cand) pos += st;
+    if (valid && (pool[pos] | 1ull) == (cand | 1ull)) valid = false;
+    unsigned vm = __ballot_sync(kFull, valid);
+    if (vm == 0u) return;
+    // the candidates are distinct: rank among them, and each pool entry's shift
+    int crank = pos, shift[MAXS];
+#pragma unroll
+    for (int s = 0; s < MAXS; ++s) shift[s] = 0;
+    do {
+        const uint64_t cj = shfl64(cand, __ffs(vm) - 1);
+        vm &= vm - 1;
+        crank += cj < cand ? 1 : 0;
+#pragma unroll
+        for (int s = 0; s < MAXS; ++s) shift[s] += cj < pk[s] ? 1 : 0;
+    } while (vm);
+    // merged order: pool entry e goes to e + shift, a candidate to its rank among both
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < MAXS; ++s) {
+        const int e = 32 * s + lane + shift[s];
+        if (shift[s] != 0 && pk[s] != kEmptyKey && e < L) pool[e] = pk[s];
+    }
+    if (valid && crank < L) pool[crank] = cand;
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < MAXS; ++s) pk[s] = pool[32 * s + lane];
+}
+
 // Alg. 1 over one graph whose rows are Xt[v] / adj[v * M] for local ids v < nt. Keys carry
 // global ids (local + id_off). The pool C (<= L <= 32 * MAXS entries, sorted by (delta, id)) lives in
 // registers: entry e = 32 s + lane is pk[s] of that lane; pool[] in shared memory holds a copy. An
@@ -319,9 +413,6 @@ __device__ __forceinline__ float rows_delta(const RT* __restrict__ base, const i
 // kernel's instructions at L = 48.)
 // Returns the pool size and leaves the keys (delta, id) in pool[0 .. size).
 // scratch: 32 ints of shared memory for the compacted neighbour ids.
-constexpr int kPoolSlots = 4;
-__host__ __device__ inline int pool_entries(int L) { return L <= 32 ? 32 : L <= 64 ? 64 : 128; }
-
 template <int METRIC, bool SMALLD, typename RT, int MAXS, bool SKIP>
 __device__ __forceinline__ int beam_search(const RT* __restrict__ Xt, const float* __restrict__ invt, const int32_t* __restrict__ adj,
                            int M, int nt, int ep, int id_off, const Query& Q, float qinv, int d, int L, uint64_t* pool,
@@ -360,27 +451,15 @@ __device__ __forceinline__ int beam_search(const RT* __restrict__ Xt, const floa
     const unsigned budget = hop_budget > 0 ? (unsigned)hop_budget : (unsigned)nt + 1u;
     unsigned it = 0, ndc = 1;
     for (; it <= (unsigned)nt; ++it) {
-        // the first entry not yet expanded
-        int slot = -1;
-        unsigned open = 0u;
-#pragma unroll
-        for (int s = 0; s < MAXS; ++s) {
-            if (slot < 0) {
-                open = __ballot_sync(kFull, ((uint32_t)pk[s] & 1u) == 0u);
-                if (open) slot = s;
-            }
-        }
-        if (slot < 0) {
+        int slot, src;
+        uint32_t lo;
+        const int id = pool_next<MAXS>(pk, slot, src, lo);
+        if (id < 0) {
             done = true;
             break;
         }
         if (it >= budget) break;
-        const int src = __ffs(open) - 1;
-        uint32_t lo = (uint32_t)pk[0];
-#pragma unroll
-        for (int s = 1; s < MAXS; ++s)
-            if (slot == s) lo = (uint32_t)pk[s];
-        const int u = (int)(__shfl_sync(kFull, lo, src) >> 1) - id_off;
+        const int u = id - id_off;
         if (lane == src) {
 #pragma unroll
             for (int s = 0; s < MAXS; ++s)
@@ -414,41 +493,8 @@ __device__ __forceinline__ int beam_search(const RT* __restrict__ Xt, const floa
                 cand = mkkey(delta_finish<METRIC>(dd, inv), (int32_t)((uint32_t)(w + id_off) << 1));
             }
             ndc += (unsigned)U;
-            bool valid = cand < pool[L - 1];
-            __syncwarp();   // scratch has been read, pool[L - 1] too
-            if (__ballot_sync(kFull, valid) == 0u) continue;
-            // rank of the candidate among the pool's entries: halving steps over its 32, 64 or 128
-            // slots (a valid candidate ranks below the last one: it beats entry L - 1). An entry
-            // equal but for the mark means it is pooled already (the lossy table let it in).
-            int pos = 0;
-#pragma unroll
-            for (int st = 16 * MAXS; st > 0; st >>= 1)
-                if (pool[pos + st - 1] < cand) pos += st;
-            if (valid && (pool[pos] | 1ull) == (cand | 1ull)) valid = false;
-            unsigned vm = __ballot_sync(kFull, valid);
-            if (vm == 0u) continue;
-            // the candidates are distinct: rank among them, and each pool entry's shift
-            int crank = pos, shift[MAXS];
-#pragma unroll
-            for (int s = 0; s < MAXS; ++s) shift[s] = 0;
-            do {
-                const uint64_t cj = shfl64(cand, __ffs(vm) - 1);
-                vm &= vm - 1;
-                crank += cj < cand ? 1 : 0;
-#pragma unroll
-                for (int s = 0; s < MAXS; ++s) shift[s] += cj < pk[s] ? 1 : 0;
-            } while (vm);
-            // merged order: pool entry e goes to e + shift, a candidate to its rank among both
-            __syncwarp();
-#pragma unroll
-            for (int s = 0; s < MAXS; ++s) {
-                const int e = 32 * s + lane + shift[s];
-                if (shift[s] != 0 && pk[s] != kEmptyKey && e < L) pool[e] = pk[s];
-            }
-            if (valid && crank < L) pool[crank] = cand;
-            __syncwarp();
-#pragma unroll
-            for (int s = 0; s < MAXS; ++s) pk[s] = pool[32 * s + lane];
+            __syncwarp();   // scratch has been read
+            pool_insert<MAXS>(pk, pool, cand, L, lane);
         }
     }
     if (!done && lane == 0) atomicOr(status, kErrTimeout);

@@ -52,6 +52,12 @@ cudaError_t launch_search(const float* X, const uint8_t* X8, const float* inv_no
                           const int32_t* qentry) {
     const bool bytes = X8 && qids && byte_rows_ok(d);
     const bool bf16 = !bytes && Xh && d > 128 && (reinterpret_cast<uintptr_t>(Xh) & 7u) == 0;
+    if (d > 128 && nq <= kTeamQueries && (!bf16 || qids)) {   // few queries: a block each (BF16 rows: queries that are rows too)
+        TeamLayers none;
+        none.count = 0;
+        return launch_search_team(bf16 ? (const void*)Xh : (const void*)X, bf16, inv_norm, n, d, metric, graph, R, entry,
+                                  qentry, none, 1, Q, qids, nq, topk, L, out_ids, out_dist, nullptr, counters, status, s);
+    }
     int htbits = ht_bits_for(L), wpb = beam_warps(d);   // the autotuner's choice for this workload, if any
     tuned_beam_shape(beam_shape_key(metric, bytes ? 1 : bf16 ? 2 : 4, d, L), &wpb, &htbits);
     const WarpLayout lay = warp_layout(d, L, htbits, 0, d > 128);

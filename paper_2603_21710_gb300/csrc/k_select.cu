@@ -61,35 +61,6 @@ __host__ __device__ inline SelectLayout select_layout(int k, int R, int d, int n
     return l;
 }
 
-// one row as the query of rows_delta (the values of load_query, read from the row storage in use)
-template <bool SMALLD, typename RT>
-__device__ __forceinline__ Query row_query(const RT* __restrict__ row, float* qs, int d, int lane) {
-    Query Q;
-    if constexpr (sizeof(RT) == 1) {
-        const int lsh = byte_lanes_log2(d);
-        const int part = lane & ((1 << lsh) - 1);
-        Q.w = make_uint4(0u, 0u, 0u, 0u);
-        if (part < (d >> 4)) Q.w = reinterpret_cast<const uint4*>(row)[part];
-        uint32_t s = __dp4a(Q.w.x, Q.w.x, 0u);
-        s = __dp4a(Q.w.y, Q.w.y, s);
-        s = __dp4a(Q.w.z, Q.w.z, s);
-        s = __dp4a(Q.w.w, Q.w.w, s);
-        Q.q2 = row_group_sum(s, lsh);
-    } else if constexpr (SMALLD) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int c = (lane & 7) + 8 * i;
-            Q.c[i] = c < (d >> 2) ? row_chunk(row, c) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    } else {
-        float4* q4 = reinterpret_cast<float4*>(qs);
-        for (int c = lane; c < (d >> 2); c += 32) q4[c] = row_chunk(row, c);
-        Q.q = qs;
-        __syncwarp();
-    }
-    return Q;
-}
-
 // NW warps per vertex: 1 (four vertices per block), or 4 when there are too few vertices to fill the
 // GPU with one warp each; warp w of a vertex then holds the candidates at positions w, w + 4, ..., all in
 // one window, and the warps agree on the next kept neighbour (the smallest position left) once per step.

@@ -196,15 +196,24 @@ cudaError_t launch_fill_i32(int32_t* p, long long n, int32_t v, cudaStream_t s) 
     return cudaGetLastError();
 }
 
+// float4 chunk c of an FP32 row, or of a BF16 row (decoded exactly)
+__device__ __forceinline__ float4 norm_chunk(const float* row, int c) { return reinterpret_cast<const float4*>(row)[c]; }
+__device__ __forceinline__ float4 norm_chunk(const uint16_t* row, int c) {
+    const uint2 w = reinterpret_cast<const uint2*>(row)[c];
+    return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
+                       __uint_as_float(w.y & 0xffff0000u));
+}
+
 // 1 / ||x|| of every row (warp per row), used by the cosine metric
-__global__ void k_inv_norms(const float* __restrict__ X, long long n, int d, float* __restrict__ inv) {
+template <typename RT>
+__global__ void k_inv_norms(const RT* __restrict__ X, long long n, int d, float* __restrict__ inv) {
     const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (row >= n) return;
-    const float4* x = reinterpret_cast<const float4*>(X + row * d);
+    const RT* x = X + row * d;
     float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
     for (int c = lane; c < (d >> 2); c += 32) {
-        float4 v = x[c];
+        float4 v = norm_chunk(x, c);
         s0 = fmaf(v.x, v.x, s0);
         s1 = fmaf(v.y, v.y, s1);
         s2 = fmaf(v.z, v.z, s2);
@@ -216,11 +225,18 @@ __global__ void k_inv_norms(const float* __restrict__ X, long long n, int d, flo
     if (lane == 0) inv[row] = s > 0.f ? __fdiv_rn(1.f, __fsqrt_rn(s)) : 0.f;
 }
 
-cudaError_t launch_inv_norms(const float* X, long long n, int d, float* inv, cudaStream_t s) {
+template <typename RT>
+static cudaError_t inv_norms(const RT* X, long long n, int d, float* inv, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     LaunchScope ls("k_inv_norms", s);
-    k_inv_norms<<<(unsigned)cdiv(n * 32, 256), 256, 0, s>>>(X, n, d, inv);
+    k_inv_norms<RT><<<(unsigned)cdiv(n * 32, 256), 256, 0, s>>>(X, n, d, inv);
     return cudaGetLastError();
+}
+cudaError_t launch_inv_norms(const float* X, long long n, int d, float* inv, cudaStream_t s) {
+    return inv_norms(X, n, d, inv, s);
+}
+cudaError_t launch_inv_norms_bf16(const uint16_t* X, long long n, int d, float* inv, cudaStream_t s) {
+    return inv_norms(X, n, d, inv, s);
 }
 
 __global__ void k_bf16_to_f32(const uint16_t* __restrict__ in, long long n, float* __restrict__ out) {

@@ -82,3 +82,25 @@ def test_float_rows_give_the_canonical_distance(d, metric):
         p = p[:, :, :o] + p[:, :, o:2 * o]
     s = p[:, :, 0]
     assert np.array_equal(dist, s if metric == L2 else np.float32(1) - s)
+
+
+@pytest.mark.parametrize("nq", [1, 304, 305, 608, 609, 1216, 1217])
+@pytest.mark.parametrize("d,dtype", [(20, "f32"), (132, "f32"), (768, "bf16"), (772, "bf16")])
+def test_few_and_many_queries_agree(d, dtype, nq):
+    """A query's result does not depend on how many come with it (a block per query, or a warp), cosine and
+    layered searches included."""
+    import paper_2603_21710_gb300 as fg
+    dev = _dev()
+    g = torch.Generator(device=dev).manual_seed(d)
+    t = torch.bfloat16 if dtype == "bf16" else torch.float32
+    X = torch.randn((3000, d), generator=g, device=dev).to(t)
+    Q = torch.randn((1300, d), generator=g, device=dev).to(t)
+    X[17] = 0   # a row without a norm
+    adj, entry = fg.build_pg(X, M=12, ef=24, metric="cos")
+    ly = fg.build_layers(X, M=8, ef=16, seed=3, metric="cos")
+    a = fg.search(X, adj, entry, Q, topk=10, beam=40, metric="cos")
+    b = fg.search(X, adj, entry, Q[:nq], topk=10, beam=40, metric="cos")
+    c = fg.search_hnsw(X, adj, ly["layers"], ly["entry"], Q, topk=10, beam=40, metric="cos")
+    e = fg.search_hnsw(X, adj, ly["layers"], ly["entry"], Q[:nq], topk=10, beam=40, metric="cos")
+    for x, y in zip(a + c, b + e):
+        assert torch.equal(x[:nq], y)
