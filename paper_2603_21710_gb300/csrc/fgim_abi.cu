@@ -1340,14 +1340,16 @@ fgim_status fgim_build_pg(const void* vectors, int64_t n, int32_t dim, int32_t d
         finish_problem(c, P, &lp);   // byte rows when the data allow, cosine norms
         // the medoid and the insertion order
         double* mean = c.alloc<double>(dim);
-        unsigned long long* dbits = c.alloc<unsigned long long>(n);
+        unsigned long long* dbits = c.alloc<unsigned long long>(std::max<long long>(n, dim));
         unsigned long long* best = c.alloc<unsigned long long>(1);
         int* medoid_d = c.alloc<int>(1);
-        ck(launch_pg_medoid(P.X, n, dim, mean, dbits, best, medoid_d, c.s));
+        ck(launch_pg_medoid(P.X, P.X8, n, dim, mean, dbits, best, medoid_d, c.s));
         int32_t* order = c.alloc<int32_t>(n);
         float* nd = c.alloc<float>(n * M);
         int32_t* zeros = c.alloc<int32_t>(n);
-        ck(launch_pg_init(n, M, medoid_d, order, adj, nd, deg, zeros, c.s));
+        int32_t* cin = c.alloc<int32_t>(n);
+        int32_t* fill = c.alloc<int32_t>(n);
+        ck(launch_pg_init(n, M, medoid_d, order, adj, nd, deg, zeros, cin, fill, c.s));
         const int medoid = c.read_i32(medoid_d);
         need(medoid >= 0 && medoid < n, FGIM_EINTERNAL, "medoid out of range");
         // per-batch scratch
@@ -1358,20 +1360,14 @@ fgim_status fgim_build_pg(const void* vectors, int64_t n, int32_t dim, int32_t d
         int32_t* e_ids = c.alloc<int32_t>(bmax * M);
         float* e_dist = c.alloc<float>(bmax * M);
         int32_t* e_cnt = c.alloc<int32_t>(bmax);
-        int32_t* cin = c.alloc<int32_t>(n);
-        int32_t* fill = c.alloc<int32_t>(n);
-        long long* off = c.alloc<long long>(n + 1);
+        int32_t* off = c.alloc<int32_t>(n);
         uint64_t* rev = c.alloc<uint64_t>(bmax * M);
-        int32_t* flag = c.alloc<int32_t>(n);
-        int32_t* targets = c.alloc<int32_t>(n);
-        long long* toff = c.alloc<long long>(n + 1);
-        const size_t sb = scan_scratch_bytes(n);
-        unsigned char* tmp = c.alloc<unsigned char>((long long)sb);
         const long long tmax = std::min<long long>(n, bmax * M);
+        int32_t* targets = c.alloc<int32_t>(tmax);
         int32_t* ov_ids = c.alloc<int32_t>(tmax * W);
         float* ov_dist = c.alloc<float>(tmax * W);
         int32_t* ov_tgt = c.alloc<int32_t>(tmax);
-        int* n_ov = c.alloc<int>(1);
+        int* pg_ctr = c.alloc<int>(kPgCounters);
         int32_t* o_ids = c.alloc<int32_t>(tmax * M);
         float* o_dist = c.alloc<float>(tmax * M);
         int32_t* o_cnt = c.alloc<int32_t>(tmax);
@@ -1391,20 +1387,11 @@ fgim_status fgim_build_pg(const void* vectors, int64_t n, int32_t dim, int32_t d
             g1.n = b;
             g1.k = ef;
             ck(launch_prune(P.X, P.X8, P.Xh, P.inv, n, dim, metric, g1, zeros, M, heur, e_ids, e_dist, e_cnt, c.status, c.s));
-            // 2. the batch's lists go in, their entries are reverse edges of their targets
-            ck(cudaMemsetAsync(cin, 0, sizeof(int32_t) * n, c.s));
-            ck(cudaMemsetAsync(fill, 0, sizeof(int32_t) * n, c.s));
-            ck(launch_pg_install(order + done, b, M, e_ids, e_dist, e_cnt, adj, nd, deg, cin, c.s));
-            ck(scan_counts(cin, n, off, tmp, sb, c.s));
-            ck(launch_pg_rev_fill(order + done, b, M, e_ids, e_dist, e_cnt, off, fill, rev, c.s));
-            ck(launch_pos_flags(cin, n, flag, c.s));
-            ck(compact_flags(flag, n, targets, toff, tmp, sb, c.s));
-            const long long nt = c.read_ll(toff + n);
-            // 3. every target keeps its list and its new edges, or the heuristic's M of them
-            ck(cudaMemsetAsync(n_ov, 0, sizeof(int), c.s));
-            ck(launch_pg_rev_merge(targets, nt, off, rev, M, M + (int)b, adj, nd, deg, ov_ids, ov_dist, ov_tgt, n_ov,
-                                   c.s));
-            const long long nov = c.read_i32(n_ov);
+            // 2. the batch's lists go in; every target of theirs keeps its list and its new edges, or the
+            //    heuristic's M of them
+            ck(launch_pg_edges(order + done, b, M, e_ids, e_dist, e_cnt, adj, nd, deg, cin, fill, off, targets, rev, ov_ids,
+                               ov_dist, ov_tgt, pg_ctr, c.s));
+            const long long nov = c.read_i32(pg_ctr + kPgOverflow);
             if (nov > 0) {
                 fgim_knng g2;
                 std::memset(&g2, 0, sizeof(g2));

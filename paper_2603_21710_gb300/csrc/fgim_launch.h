@@ -256,22 +256,17 @@ cudaError_t launch_hnsw_next(const int32_t* best, const int32_t* mem, long long 
                              int* status, cudaStream_t s);
 
 // ---- k_pgbuild.cu: input PGs by batch-incremental insertion (see the file comment)
-cudaError_t launch_pg_medoid(const float* X, long long n, int d, double* mean, unsigned long long* dist_bits,
+cudaError_t launch_pg_medoid(const float* X, const uint8_t* X8, long long n, int d, double* mean, unsigned long long* dist_bits,
                              unsigned long long* best, int* medoid, cudaStream_t s);
 cudaError_t launch_pg_init(long long n, int M, const int* medoid, int32_t* order, int32_t* nbr, float* nd, int32_t* cnt,
-                           int32_t* zeros, cudaStream_t s);
-cudaError_t launch_pg_install(const int32_t* rows, long long b, int M, const int32_t* e_ids, const float* e_dist,
-                              const int32_t* e_cnt, int32_t* nbr, float* nd, int32_t* cnt, int32_t* cin,
-                              cudaStream_t s);
-cudaError_t launch_pg_rev_fill(const int32_t* rows, long long b, int M, const int32_t* e_ids, const float* e_dist,
-                               const int32_t* e_cnt, const long long* off, int32_t* fill, uint64_t* rev,
-                               cudaStream_t s);
-cudaError_t launch_pg_rev_merge(const int32_t* targets, long long nt, const long long* off, const uint64_t* rev, int M,
-                                int W, int32_t* nbr, float* nd, int32_t* cnt, int32_t* ov_ids, float* ov_dist,
-                                int32_t* ov_tgt, int* n_ov, cudaStream_t s);
+                           int32_t* zeros, int32_t* cin, int32_t* fill, cudaStream_t s);
+constexpr int kPgCounters = 3, kPgOverflow = 2;   // ints of launch_pg_edges' counters; the overflow lists' number
+cudaError_t launch_pg_edges(const int32_t* rows, long long b, int M, const int32_t* e_ids, const float* e_dist,
+                            const int32_t* e_cnt, int32_t* nbr, float* nd, int32_t* cnt, int32_t* cin, int32_t* fill,
+                            int32_t* off, int32_t* targets, uint64_t* rev, int32_t* ov_ids, float* ov_dist,
+                            int32_t* ov_tgt, int* counters, cudaStream_t s);
 cudaError_t launch_pg_write_back(const int32_t* ov_tgt, long long nov, int M, const int32_t* e_ids, const float* e_dist,
                                  const int32_t* e_cnt, int32_t* nbr, float* nd, int32_t* cnt, cudaStream_t s);
-cudaError_t launch_pos_flags(const int32_t* c, long long n, int32_t* flag, cudaStream_t s);
 
 // ---- fgim_abi.cu: launch shapes chosen by the autotuner (fgim_autotune)
 // Beam-search kernels (cross query, searches): warps per block and visited-table bits, keyed by

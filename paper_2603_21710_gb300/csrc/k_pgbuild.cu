@@ -13,19 +13,67 @@
 // all of them when they are at most M and otherwise the heuristic's M. The mean and the medoid
 // distances are summed in the same sequential FP64 order as a plain loop, so the medoid is that
 // of the plain loop bit for bit.
+#include <cstddef>
+
 #include "fgim_launch.h"
 
 namespace fgim {
 
 static inline long long cdivp(long long a, long long b) { return (a + b - 1) / b; }
 
-// mean[t] = (sum over rows i, in order, of X[i][t]) / n, in FP64 (one thread per dimension)
-__global__ void k_col_mean(const float* __restrict__ X, long long n, int d, double* __restrict__ mean) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+// mean[t] = (sum over rows i, in order, of X[i][t]) / n, in FP64. One warp per 32 dimensions, one lane each: a
+// chain of n additions, bound by their latency as long as the rows arrive in time, so the next kMeanRows rows
+// are read while the current ones are added (one row at a time, 60,000 rows took 4.9 ms).
+constexpr int kMeanRows = 32;
+__global__ void __launch_bounds__(32) k_col_mean(const float* __restrict__ X, long long n, int d, double* __restrict__ mean) {
+    const int t = blockIdx.x * 32 + threadIdx.x;
     if (t >= d) return;
+    const float* p = X + t;
+    float cur[kMeanRows], nxt[kMeanRows];
     double s = 0.0;
-    for (long long i = 0; i < n; ++i) s = __dadd_rn(s, (double)X[i * d + t]);
+    const long long full = n / kMeanRows;
+    if (full > 0) {
+#pragma unroll
+        for (int r = 0; r < kMeanRows; ++r) cur[r] = p[(long long)r * d];
+    }
+    for (long long b = 0; b < full; ++b) {
+        p += (long long)kMeanRows * d;
+        if (b + 1 < full) {
+#pragma unroll
+            for (int r = 0; r < kMeanRows; ++r) nxt[r] = p[(long long)r * d];
+        }
+#pragma unroll
+        for (int r = 0; r < kMeanRows; ++r) s = __dadd_rn(s, (double)cur[r]);
+#pragma unroll
+        for (int r = 0; r < kMeanRows; ++r) cur[r] = nxt[r];
+    }
+    for (long long i = full * kMeanRows; i < n; ++i) s = __dadd_rn(s, (double)X[i * d + t]);
     mean[t] = __ddiv_rn(s, (double)n);
+}
+
+// The same from byte rows: every partial sum is an integer below 255 n < 2^39, exact in FP64, so the sum over any
+// order is the sequential one's. Block (x, y): 32 dimensions, rows y * rows ..; sums[t] += its part.
+__global__ void __launch_bounds__(256) k_col_sums_u8(const uint8_t* __restrict__ X8, long long n, int d, long long rows,
+                                                     unsigned long long* __restrict__ sums) {
+    __shared__ unsigned long long part[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int t = blockIdx.x * 32 + lane;
+    const long long r0 = blockIdx.y * rows, r1 = min(n, r0 + rows);
+    unsigned long long s = 0;
+    if (t < d)
+#pragma unroll 8
+        for (long long i = r0 + warp; i < r1; i += 8) s += X8[i * d + t];
+    part[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0 && t < d) {
+        for (int w = 1; w < 8; ++w) s += part[w][lane];
+        atomicAdd(sums + t, s);
+    }
+}
+
+__global__ void k_col_mean_u8(const unsigned long long* __restrict__ sums, long long n, int d, double* __restrict__ mean) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < d) mean[t] = __ddiv_rn((double)sums[t], (double)n);
 }
 
 // squared FP64 distance of every row to the mean (sequential over the dimensions), the smallest
@@ -54,13 +102,15 @@ __global__ void k_medoid_pick(const unsigned long long* __restrict__ dist_bits, 
 // insertion order: the medoid, then every other row in id order; and the empty graph
 __global__ void k_pg_init(long long n, int M, const int* medoid, int32_t* __restrict__ order,
                           int32_t* __restrict__ nbr, float* __restrict__ nd, int32_t* __restrict__ cnt,
-                          int32_t* __restrict__ zeros) {
+                          int32_t* __restrict__ zeros, int32_t* __restrict__ cin, int32_t* __restrict__ fill) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int m = *medoid;
     if (i < n) {
         order[i] = i == 0 ? m : (i - 1 < m ? (int32_t)(i - 1) : (int32_t)i);
         cnt[i] = 0;
         zeros[i] = 0;
+        cin[i] = 0;
+        fill[i] = 0;
     }
     if (i < n * M) {
         nbr[i] = -1;
@@ -68,11 +118,20 @@ __global__ void k_pg_init(long long n, int M, const int* medoid, int32_t* __rest
     }
 }
 
+// The reverse edges of a batch are grouped by target without a pass over all n vertices (two prefix sums, a
+// compaction and two fills over n took seven launches and a host read per batch): the first edge to a
+// vertex puts it in the list of targets, every target takes its segment of rev from a counter, and the merge
+// leaves cin and fill zero for the next batch. The order of targets and segments is arbitrary; a target's keys
+// are put in order when they are merged.
+struct PgCounters {   // of one batch, zeroed before it
+    int targets, edges, overflow;
+};
+
 // the batch's lists go in; their entries become reverse-edge candidates of their targets
 __global__ void k_pg_install(const int32_t* __restrict__ rows, long long b, int M, const int32_t* __restrict__ e_ids,
                              const float* __restrict__ e_dist, const int32_t* __restrict__ e_cnt,
                              int32_t* __restrict__ nbr, float* __restrict__ nd, int32_t* __restrict__ cnt,
-                             int32_t* __restrict__ cin) {
+                             int32_t* __restrict__ cin, int32_t* __restrict__ targets, PgCounters* ctr) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= b * M) return;
     const long long bi = i / M;
@@ -82,12 +141,19 @@ __global__ void k_pg_install(const int32_t* __restrict__ rows, long long b, int 
     if (t == 0) cnt[p] = c;
     nbr[(long long)p * M + t] = t < c ? e_ids[i] : -1;
     nd[(long long)p * M + t] = t < c ? e_dist[i] : __int_as_float(0x7f800000);
-    if (t < c) atomicAdd(cin + e_ids[i], 1);
+    if (t < c && atomicAdd(cin + e_ids[i], 1) == 0) targets[atomicAdd(&ctr->targets, 1)] = e_ids[i];
+}
+
+__global__ void k_pg_segments(const int32_t* __restrict__ targets, const int32_t* __restrict__ cin,
+                              int32_t* __restrict__ off, PgCounters* ctr) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= ctr->targets) return;
+    off[targets[i]] = atomicAdd(&ctr->edges, cin[targets[i]]);
 }
 
 __global__ void k_pg_rev_fill(const int32_t* __restrict__ rows, long long b, int M, const int32_t* __restrict__ e_ids,
                               const float* __restrict__ e_dist, const int32_t* __restrict__ e_cnt,
-                              const long long* __restrict__ off, int32_t* __restrict__ fill,
+                              const int32_t* __restrict__ off, int32_t* __restrict__ fill,
                               uint64_t* __restrict__ rev) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= b * M) return;
@@ -102,22 +168,25 @@ constexpr int kMergeCap = 128;   // the longest list warp_merge can hold
 
 // Per target v (warp per target): its list and its new reverse edges in ascending (distance, id);
 // at most M of them stay as they are, more go to the overflow lists for the heuristic.
-__global__ void __launch_bounds__(128) k_pg_rev_merge(const int32_t* __restrict__ targets, long long nt,
-                                                      const long long* __restrict__ off,
+__global__ void __launch_bounds__(128) k_pg_rev_merge(const int32_t* __restrict__ targets,
+                                                      const int32_t* __restrict__ off, int32_t* __restrict__ cin,
+                                                      int32_t* __restrict__ fill,
                                                       const uint64_t* __restrict__ rev, int M, int W,
                                                       int32_t* __restrict__ nbr, float* __restrict__ nd,
                                                       int32_t* __restrict__ cnt, int32_t* __restrict__ ov_ids,
                                                       float* __restrict__ ov_dist, int32_t* __restrict__ ov_tgt,
-                                                      int* __restrict__ n_ov) {
+                                                      PgCounters* ctr) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5;
     const int lane = lane_id();
     const long long ti = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
-    if (ti >= nt) return;
+    if (ti >= ctr->targets) return;
     const int32_t v = targets[ti];
     uint64_t* list = reinterpret_cast<uint64_t*>(smem) + (size_t)warp * W;
     const int c0 = cnt[v];
-    const long long b0 = off[v], m = off[v + 1] - off[v];
+    const long long b0 = off[v], m = cin[v];
+    __syncwarp();
+    if (lane == 0) cin[v] = fill[v] = 0;
     if (c0 + m > kMergeCap) {
         // a hub: more keys than a merged list may hold (the keys are distinct and at most W, more than M):
         // each key's place is the number of smaller ones, written straight to the overflow list
@@ -126,7 +195,7 @@ __global__ void __launch_bounds__(128) k_pg_rev_merge(const int32_t* __restrict_
             list[s] = s < c0 ? mkkey(nd[(long long)v * M + s], nbr[(long long)v * M + s]) : rev[b0 + (s - c0)];
         __syncwarp();
         int slot = 0;
-        if (lane == 0) slot = atomicAdd(n_ov, 1);
+        if (lane == 0) slot = atomicAdd(&ctr->overflow, 1);
         slot = __shfl_sync(kFull, slot, 0);
         for (int s = lane; s < total; s += 32) {
             const uint64_t key = list[s];
@@ -161,7 +230,7 @@ __global__ void __launch_bounds__(128) k_pg_rev_merge(const int32_t* __restrict_
         return;
     }
     int slot = 0;
-    if (lane == 0) slot = atomicAdd(n_ov, 1);
+    if (lane == 0) slot = atomicAdd(&ctr->overflow, 1);
     slot = __shfl_sync(kFull, slot, 0);
     for (int s = lane; s < W; s += 32) {
         ov_ids[(long long)slot * W + s] = s < n ? key_id(list[s]) : -1;
@@ -185,25 +254,25 @@ __global__ void k_pg_write_back(const int32_t* __restrict__ ov_tgt, long long no
     nd[(long long)v * M + t] = e_dist[i];
 }
 
-__global__ void k_pos_flags(const int32_t* __restrict__ c, long long n, int32_t* __restrict__ flag) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) flag[i] = c[i] > 0 ? 1 : 0;
-}
-
-cudaError_t launch_pos_flags(const int32_t* c, long long n, int32_t* flag, cudaStream_t s) {
-    LaunchScope ls("k_pos_flags", s);
-    k_pos_flags<<<(unsigned)cdivp(n, 256), 256, 0, s>>>(c, n, flag);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pg_medoid(const float* X, long long n, int d, double* mean, unsigned long long* dist_bits,
+cudaError_t launch_pg_medoid(const float* X, const uint8_t* X8, long long n, int d, double* mean, unsigned long long* dist_bits,
                              unsigned long long* best, int* medoid, cudaStream_t s) {
     cudaError_t e;
     if ((e = cudaMemsetAsync(best, 0xff, sizeof(unsigned long long), s)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(medoid, 0x7f, sizeof(int), s)) != cudaSuccess) return e;
-    {
+    if (X8) {   // the sums stand where the distances go afterwards (dist_bits has room for n and for d of them)
+        if ((e = cudaMemsetAsync(dist_bits, 0, sizeof(unsigned long long) * d, s)) != cudaSuccess) return e;
+        const long long rows = std::max(512LL, cdivp(n, 4096));
+        {
+            LaunchScope ls("k_col_sums_u8", s);
+            k_col_sums_u8<<<dim3((unsigned)cdivp(d, 32), (unsigned)cdivp(n, rows)), 256, 0, s>>>(X8, n, d, rows, dist_bits);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
         LaunchScope ls("k_col_mean", s);
-        k_col_mean<<<(unsigned)cdivp(d, 128), 128, 0, s>>>(X, n, d, mean);
+        k_col_mean_u8<<<(unsigned)cdivp(d, 128), 128, 0, s>>>(dist_bits, n, d, mean);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    } else {
+        LaunchScope ls("k_col_mean", s);
+        k_col_mean<<<(unsigned)cdivp(d, 32), 32, 0, s>>>(X, n, d, mean);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     {
@@ -217,39 +286,46 @@ cudaError_t launch_pg_medoid(const float* X, long long n, int d, double* mean, u
 }
 
 cudaError_t launch_pg_init(long long n, int M, const int* medoid, int32_t* order, int32_t* nbr, float* nd, int32_t* cnt,
-                           int32_t* zeros, cudaStream_t s) {
+                           int32_t* zeros, int32_t* cin, int32_t* fill, cudaStream_t s) {
     LaunchScope ls("k_pg_init", s);
-    k_pg_init<<<(unsigned)cdivp(n * M, 256), 256, 0, s>>>(n, M, medoid, order, nbr, nd, cnt, zeros);
+    k_pg_init<<<(unsigned)cdivp(n * M, 256), 256, 0, s>>>(n, M, medoid, order, nbr, nd, cnt, zeros, cin, fill);
     return cudaGetLastError();
 }
 
-cudaError_t launch_pg_install(const int32_t* rows, long long b, int M, const int32_t* e_ids, const float* e_dist,
-                              const int32_t* e_cnt, int32_t* nbr, float* nd, int32_t* cnt, int32_t* cin,
-                              cudaStream_t s) {
-    LaunchScope ls("k_pg_install", s);
-    k_pg_install<<<(unsigned)cdivp(b * M, 256), 256, 0, s>>>(rows, b, M, e_ids, e_dist, e_cnt, nbr, nd, cnt, cin);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pg_rev_fill(const int32_t* rows, long long b, int M, const int32_t* e_ids, const float* e_dist,
-                               const int32_t* e_cnt, const long long* off, int32_t* fill, uint64_t* rev,
-                               cudaStream_t s) {
-    LaunchScope ls("k_pg_rev_fill", s);
-    k_pg_rev_fill<<<(unsigned)cdivp(b * M, 256), 256, 0, s>>>(rows, b, M, e_ids, e_dist, e_cnt, off, fill, rev);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pg_rev_merge(const int32_t* targets, long long nt, const long long* off, const uint64_t* rev, int M,
-                                int W, int32_t* nbr, float* nd, int32_t* cnt, int32_t* ov_ids, float* ov_dist,
-                                int32_t* ov_tgt, int* n_ov, cudaStream_t s) {
-    if (nt <= 0) return cudaSuccess;
-    const int wpb = 4;
-    const size_t smem = (size_t)wpb * W * 8;
-    cudaError_t e = cudaFuncSetAttribute(k_pg_rev_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+// The batch's lists into the graph, and its reverse edges into their targets' lists; counters (kPgCounters ints)
+// [kPgOverflow] becomes the number of overflow lists.
+cudaError_t launch_pg_edges(const int32_t* rows, long long b, int M, const int32_t* e_ids, const float* e_dist,
+                            const int32_t* e_cnt, int32_t* nbr, float* nd, int32_t* cnt, int32_t* cin, int32_t* fill,
+                            int32_t* off, int32_t* targets, uint64_t* rev, int32_t* ov_ids, float* ov_dist,
+                            int32_t* ov_tgt, int* counters, cudaStream_t s) {
+    static_assert(sizeof(PgCounters) == kPgCounters * sizeof(int) && offsetof(PgCounters, overflow) == kPgOverflow * sizeof(int));
+    PgCounters* ctr = reinterpret_cast<PgCounters*>(counters);
+    cudaError_t e = cudaMemsetAsync(ctr, 0, sizeof(PgCounters), s);
     if (e != cudaSuccess) return e;
+    const long long edges = b * M;   // no more targets than edges
+    const unsigned blocks = (unsigned)cdivp(edges, 256);
+    {
+        LaunchScope ls("k_pg_install", s);
+        k_pg_install<<<blocks, 256, 0, s>>>(rows, b, M, e_ids, e_dist, e_cnt, nbr, nd, cnt, cin, targets, ctr);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    {
+        LaunchScope ls("k_pg_segments", s);
+        k_pg_segments<<<blocks, 256, 0, s>>>(targets, cin, off, ctr);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    {
+        LaunchScope ls("k_pg_rev_fill", s);
+        k_pg_rev_fill<<<blocks, 256, 0, s>>>(rows, b, M, e_ids, e_dist, e_cnt, off, fill, rev);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    const int wpb = 4, W = M + (int)b;
+    const size_t smem = (size_t)wpb * W * 8;
+    if ((e = cudaFuncSetAttribute(k_pg_rev_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+        return e;
     LaunchScope ls("k_pg_rev_merge", s);
-    k_pg_rev_merge<<<(unsigned)cdivp(nt, wpb), wpb * 32, smem, s>>>(targets, nt, off, rev, M, W, nbr, nd, cnt, ov_ids,
-                                                                   ov_dist, ov_tgt, n_ov);
+    k_pg_rev_merge<<<(unsigned)cdivp(edges, wpb), wpb * 32, smem, s>>>(targets, off, cin, fill, rev, M, W, nbr, nd, cnt,
+                                                                      ov_ids, ov_dist, ov_tgt, ctr);
     return cudaGetLastError();
 }
 
