@@ -191,10 +191,13 @@ __device__ __forceinline__ T take_row_totals(const T (&v)[4], int r0, T mine, in
 // integer below 128 * 255^2 < 2^24, so it is exact and the canonical value is the exact
 // integer result. Lanes take 16 bytes each (32 / lanes-per-row rows per warp load) and form
 // |q|^2 + |x|^2 - 2 q.x with four-way byte dot products, summed over the row's lanes.
-// SKIP (FP32 rows up to 128 coordinates): the chunks past the row's end are left out by a branch (the same for
-// every lane) instead of adding zeros. Faster where many warps share an SM (cross query at d = 96:
-// 16.8 -> 15.0 ms, d = 32: 0.46 -> 0.42 ms), slower where few searches wait for each other's chain
-// (k_search of 10,000 queries 0.90 -> 0.99 ms), so k_search leaves it off.
+// SKIP (FP32 rows up to 128 coordinates; many warps share an SM): the loads are unconditional (past the last
+// row its chunks again, past a row's end its last chunk, left out of the sum by a branch), and the second
+// eight rows of a step are left out together when there are none. Loads under a lane's own condition made
+// each row's a branch of its own: cross query 300k d = 96 15.1 -> 13.0 ms, d = 32 0.445 -> 0.398 ms. k_search,
+// where few searches wait for each other's chain, is slower so (10,000 queries 0.86 -> 0.96 ms) and
+// leaves it off, as is reading the next entry's adjacency row ahead there (held in a register 1.6 ms,
+// as a prefetch 0.94).
 template <int METRIC, bool SMALLD, typename RT, bool SKIP = true>
 __device__ __forceinline__ float rows_delta(const RT* __restrict__ base, const int32_t* rid, int U, const Query& Q,
                                             int d, int lane) {
@@ -254,10 +257,20 @@ __device__ __forceinline__ float rows_delta(const RT* __restrict__ base, const i
             float sv[4];
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf) {
+                if (SKIP && hf && r0 + 8 >= U) {
+                    sv[2] = sv[3] = 0.f;
+                    continue;
+                }
                 float4 y[2][4];
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
                     const int r = r0 + 8 * hf + 4 * t + sub;
+                    if (SKIP) {
+                        const RT* row = base + (long long)rid[min(r, U - 1)] * d;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) y[t][i] = row_chunk(row, min(part + 8 * i, nc4 - 1));
+                        continue;
+                    }
                     const bool ok = r < U;
                     const RT* row = base + (long long)(ok ? rid[r] : 0) * d;
 #pragma unroll
@@ -271,7 +284,7 @@ __device__ __forceinline__ float rows_delta(const RT* __restrict__ base, const i
                     float pt[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        if (!SKIP || 8 * i < nc4) pt[i] = chunk_part<METRIC>(Q.c[i], y[t][i]);
+                        if (!SKIP || part + 8 * i < nc4) pt[i] = chunk_part<METRIC>(Q.c[i], y[t][i]);
                     sv[2 * hf + t] = __fadd_rn(__fadd_rn(pt[0], pt[2]), __fadd_rn(pt[1], pt[3]));
                 }
             }
