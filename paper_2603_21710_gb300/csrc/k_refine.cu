@@ -754,12 +754,19 @@ cudaError_t launch_fp8_coarse(const fgim_knng& g, const float4* tcm, const float
     return cudaGetLastError();
 }
 
-// Tile row of candidate i for candidate sets of up to 128: candidates i = 4 m + q go to TMEM
-// lane quarter q (row 32 q + m), so every lane quarter holds an even share of the new and old
+// Tile row of candidate i for candidate sets of up to 128: candidates i = 4 m + q go to row m of
+// TMEM lane quarter q, so every lane quarter holds an even share of the new and old
 // candidates and the warps of the four quarters get similar work. The columns of D follow
-// the same order (both MMA operands are the one staged tile); the inverse is the same formula.
-__host__ __device__ __forceinline__ int tc_row(int i) { return 32 * (i & 3) + (i >> 2); }
-__host__ __device__ __forceinline__ int tc_cand(int row) { return 4 * (row & 31) + (row >> 5); }
+// the same order (both MMA operands are the one staged tile). A quarter has 2^qs rows: 32 (M = 128) or, for
+// sets of up to 64 (kTCSmall) joined without byte rows, 16 (M = 64, whose rows 16 q + m go to TMEM lanes
+// 32 q + m). That tile takes 64 TMEM columns and half the shared memory, and with re-rank steps of four
+// pairs instead of eight (80 registers) six CTAs fit on an SM instead of four: each is a chain of a few
+// memory round trips, and four kept the SM's schedulers 48 % busy. Join of 300k d = 96: 12.4 -> 10.0 ms,
+// 120k d = 768 BF16 12.4 -> 9.9, 50k d = 100 4.0 -> 3.3, 20k d = 32 0.78 -> 0.62. (Byte rows keep eight warps of
+// 64 registers per CTA, which fill an SM at four; nearly all of their sets are larger anyway.)
+constexpr int kTCSmall = 64;
+__host__ __device__ __forceinline__ int tc_row(int i, int qs) { return ((i & 3) << qs) + (i >> 2); }
+__host__ __device__ __forceinline__ int tc_cand(int lane_row) { return 4 * (lane_row & 31) + (lane_row >> 5); }
 
 // Shared memory of one k_join_tc CTA (offsets from the first 1024-byte boundary of the
 // dynamic shared memory; `bytes` includes the slack for that alignment).
@@ -767,17 +774,18 @@ struct TCLayout {
     int op, rows_alloc, dpad, meta, colf, thr, pb_key, cid, hkv, mask, queue, pb_tgt, misc, bytes, hs, words;
 };
 
-__host__ __device__ inline TCLayout tc_layout(int cm, int d) {
+// small: the M = 64 tile (cm <= kTCSmall)
+__host__ __device__ inline TCLayout tc_layout(int cm, int d, bool small) {
     TCLayout l;
     int hs = 64;   // id -> index table, load factor <= 1/4: two probes find nearly every key
     while (hs < 4 * cm) hs <<= 1;
     l.hs = hs;
     const int npad = ((cm + 15) / 16) * 16;
-    // membership bits per TMEM lane row in TMEM column order: 128 columns (interleaved order) or npad
-    l.words = cm <= 128 ? 4 : (npad + 31) >> 5;
+    // membership bits per candidate in TMEM column order: 64 or 128 columns (interleaved order) or npad
+    l.words = small ? 2 : cm <= 128 ? 4 : (npad + 31) >> 5;
     // rows per panel (a multiple of 8: whole swizzle atoms); sets of up to 128 candidates are
-    // staged in the quarter-interleaved row order (tc_row), which spans all 128 rows
-    l.rows_alloc = cm <= 128 ? 128 : npad;
+    // staged in the quarter-interleaved row order (tc_row), which spans all 64 or 128 rows
+    l.rows_alloc = small ? 64 : cm <= 128 ? 128 : npad;
     // K is staged in chunks of at most kTCKChunk dimensions (whole 128-byte panels, zero beyond d);
     // the MMAs of successive chunks accumulate in TMEM, so d is not limited by shared memory
     l.dpad = ((d + 63) / 64) * 64;
@@ -806,10 +814,10 @@ __host__ __device__ inline TCLayout tc_layout(int cm, int d) {
     o += kTCPropBuf * 4;
     l.misc = o;
     o += 64;
-    // The A operand spans 128 rows of every panel even when fewer are staged: rows past the
+    // The A operand spans 128 (small: 64) rows of every panel even when fewer are staged: rows past the
     // staged ones read whatever follows (the next panel, the arrays above) and only produce
     // rows of D that are never used. Keep all of it inside the allocation.
-    const int a_end = (l.dpad / 64 - 1) * l.rows_alloc * 128 + 128 * 128;
+    const int a_end = (l.dpad / 64 - 1) * l.rows_alloc * 128 + (small ? 64 : 128) * 128;
     l.bytes = (o > a_end ? o : a_end) + 1024;
     return l;
 }
@@ -818,8 +826,8 @@ __host__ __device__ inline TCLayout tc_layout(int cm, int d) {
 // Xb: the staged operand, rows of dp BF16 or FP16 values, or (FP8) of dp E4M3 ones; each row has a
 // factor (tcm.w, 1 for BF16), so each Gram entry is scaled by the two rows' factors, and the filter's bound
 // takes their conversion errors.
-template <int METRIC, bool BYTES, bool LARGE, bool FP8>
-__global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
+template <int METRIC, bool BYTES, bool LARGE, bool FP8, bool SMALL>
+__global__ void __launch_bounds__(BYTES ? 256 : 128, SMALL ? 6 : 4) k_join_tc(
     ShardTable t, const float* __restrict__ X, const __nv_bfloat16* __restrict__ Xb, int dp, bool f16,
     const uint8_t* __restrict__ X8, const float4* __restrict__ tcm, const float* __restrict__ inv_norm, int k, const int32_t* __restrict__ ids,
     const uint64_t* __restrict__ wk, const int32_t* __restrict__ cand, const int32_t* __restrict__ nn_arr, const int32_t* __restrict__ no_arr, int cmax,
@@ -828,6 +836,7 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
     unsigned long long* pairs_count, unsigned long long* cands_count, int* status) {
     constexpr int NT = BYTES ? 256 : 128;   // threads (byte rows: eight warps, two per TMEM lane quarter)
     constexpr int NW = NT / 32;
+    constexpr int QS = SMALL ? 4 : 5;   // log2 of the rows of a lane quarter (tc_row)
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
     const int tid = threadIdx.x;
@@ -841,13 +850,13 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
     const int32_t cA = tid < cm ? cand[crow + tid] : -1;
     const int32_t cB = tid + NT < cm ? cand[crow + tid + NT] : -1;
     if (nn == 0 || nc < 2) return;
-    if (nc > cm || nn > 128 || cm > 2 * NT || (!LARGE && cm > 128)) {   // the host sized the launch
+    if (nc > cm || nn > 128 || cm > 2 * NT || (!LARGE && cm > (SMALL ? kTCSmall : 128))) {   // the host sized the launch
         if (tid == 0) atomicOr(status, kErrBounds);
         return;
     }
     const int d = t.dim;
     const int du = FP8 ? dp / 2 : dp;   // staged row in 2-byte units (a 16-bit value or an E4M3 pair; zeros past d)
-    const TCLayout L = tc_layout(cm, du);
+    const TCLayout L = tc_layout(cm, du, SMALL);
     unsigned char* op = smem + L.op;
     float4* meta = reinterpret_cast<float4*>(smem + L.meta);   // n2, y, z (see the filter), cosine 1/|x|
     float4* colf = reinterpret_cast<float4*>(smem + L.colf);   // P, worst distance, shard (bits), factor
@@ -900,7 +909,7 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
             const int r = kcp_sh >= 0 ? item >> kcp_sh : item / kcp;
             const int c = item - r * kcp;
             const int gc = ch * kcp + c;
-            unsigned char* dst = op + tc::sw_offset(LARGE ? r : tc_row(r), c, rows);
+            unsigned char* dst = op + tc::sw_offset(LARGE ? r : tc_row(r, QS), c, rows);
             if (gc < kc) cp_async16(dst, Xb + (long long)cid[r] * du + gc * 8, true);
             else *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
         }
@@ -1000,7 +1009,7 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
             }
         }
         if (j >= 0) {
-            const int cj = LARGE ? j : tc_row(j), ci = LARGE ? i : tc_row(i);
+            const int cj = LARGE ? j : tc_row(j, QS), ci = LARGE ? i : tc_row(i, QS);
             if (!LARGE || i < 128) atomicOr(mask + i * W + (cj >> 5), 1u << (cj & 31));
             if (!LARGE || j < 128) atomicOr(maskB + j * W + (ci >> 5), 1u << (ci & 31));
         }
@@ -1045,8 +1054,8 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
             tc::fence_after_sync();
         }
         if (tid == 0) {
-            const int n_cols = LARGE ? npad : 128;
-            const uint32_t idesc = FP8 ? tc::idesc_e4m3(128, n_cols) : f16 ? tc::idesc_f16(128, n_cols) : tc::idesc_bf16(128, n_cols);
+            const int n_cols = LARGE ? npad : 4 << QS, m_rows = SMALL ? 64 : 128;
+            const uint32_t idesc = FP8 ? tc::idesc_e4m3(m_rows, n_cols) : f16 ? tc::idesc_f16(m_rows, n_cols) : tc::idesc_bf16(m_rows, n_cols);
             const uint32_t base = tc::smem_u32(op);
             for (int s = 0; s < L.dpad / 16; ++s) {   // 32 bytes of every row per MMA
                 const uint64_t desc = tc::smem_desc_sw128(base + (uint32_t)((s >> 2) * rows * 128 + (s & 3) * 32));
@@ -1142,7 +1151,8 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
     //    warp's pairs fall in different banks).
     //  - otherwise the canonical FP32 additions, from the staged tile when every staged row is
     //    exact (the same values), else from the FP32 rows in global memory.
-    constexpr int kStep = BYTES ? 32 : 8;
+    constexpr int KP = SMALL ? 4 : 8;   // pairs whose rows are in flight together (FP32 rows)
+    constexpr int kStep = BYTES ? 32 : KP;
     auto rerank = [&](int nq) {
         if (BYTES && !rows_ready && nq > 0) {   // bounded wait for the byte rows (every lane)
             if (!tc::mbar_wait(rows_bar, 0u, 1 << 24)) atomicOr(status, kErrTimeout);
@@ -1176,25 +1186,25 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
                     }
                 }
             } else {
-                int ra[8], rb[8];
+                int ra[KP], rb[KP];
 #pragma unroll
-                for (int t8 = 0; t8 < 8; ++t8) {
+                for (int t8 = 0; t8 < KP; ++t8) {
                     const uint32_t e = wq[q0 + min(t8, U - 1)];
                     ra[t8] = (int)(e & 1023u);
                     rb[t8] = (int)((e >> 10) & 1023u);
                 }
-                float acc[8][4];
+                float acc[KP][4];
 #pragma unroll
-                for (int t8 = 0; t8 < 8; ++t8) acc[t8][0] = acc[t8][1] = acc[t8][2] = acc[t8][3] = 0.f;
+                for (int t8 = 0; t8 < KP; ++t8) acc[t8][0] = acc[t8][1] = acc[t8][2] = acc[t8][3] = 0.f;
                 for (int c = lane; c < vq; c += 32) {
-                    float4 xa[8], xb[8];
+                    float4 xa[KP], xb[KP];
                     if (exact) {
 #pragma unroll
-                        for (int t8 = 0; t8 < 8; ++t8) {
+                        for (int t8 = 0; t8 < KP; ++t8) {
                             const uint2 ua =
-                                *reinterpret_cast<const uint2*>(op + tc::sw_offset(LARGE ? ra[t8] : tc_row(ra[t8]), c >> 1, rows) + (c & 1) * 8);
+                                *reinterpret_cast<const uint2*>(op + tc::sw_offset(LARGE ? ra[t8] : tc_row(ra[t8], QS), c >> 1, rows) + (c & 1) * 8);
                             const uint2 ub =
-                                *reinterpret_cast<const uint2*>(op + tc::sw_offset(LARGE ? rb[t8] : tc_row(rb[t8]), c >> 1, rows) + (c & 1) * 8);
+                                *reinterpret_cast<const uint2*>(op + tc::sw_offset(LARGE ? rb[t8] : tc_row(rb[t8], QS), c >> 1, rows) + (c & 1) * 8);
                             xa[t8] = make_float4(__uint_as_float(ua.x << 16), __uint_as_float(ua.x & 0xffff0000u),
                                                  __uint_as_float(ua.y << 16), __uint_as_float(ua.y & 0xffff0000u));
                             xb[t8] = make_float4(__uint_as_float(ub.x << 16), __uint_as_float(ub.x & 0xffff0000u),
@@ -1202,13 +1212,13 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
                         }
                     } else {
 #pragma unroll
-                        for (int t8 = 0; t8 < 8; ++t8) {
+                        for (int t8 = 0; t8 < KP; ++t8) {
                             xa[t8] = reinterpret_cast<const float4*>(X + (long long)cid[ra[t8]] * d)[c];
                             xb[t8] = reinterpret_cast<const float4*>(X + (long long)cid[rb[t8]] * d)[c];
                         }
                     }
 #pragma unroll
-                    for (int t8 = 0; t8 < 8; ++t8) {
+                    for (int t8 = 0; t8 < KP; ++t8) {
                         const float4 x = xa[t8], y = xb[t8];
                         if (METRIC == FGIM_L2SQ) {
                             const float e0 = __fsub_rn(x.x, y.x), e1 = __fsub_rn(x.y, y.y);
@@ -1226,7 +1236,7 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
                     }
                 }
 #pragma unroll
-                for (int t8 = 0; t8 < 8; ++t8) {
+                for (int t8 = 0; t8 < KP; ++t8) {
                     const float tot = warp_butterfly(__fadd_rn(__fadd_rn(acc[t8][0], acc[t8][1]),
                                                                __fadd_rn(acc[t8][2], acc[t8][3])));
                     if (lane == t8) sc = tot;
@@ -1329,7 +1339,7 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
     };
     if (ok_mma) {
         // Column ranges. Interleaved order (up to 128 candidates): range rg = columns
-        // 32 rg + m', m' < |{b < nn : b % 4 = rg}|, candidate b = 4 m' + rg; lane (a = 4 lane + q)
+        // 2^QS rg + m', m' < |{b < nn : b % 4 = rg}|, candidate b = 4 m' + rg; lane (a = 4 lane + q)
         // pairs with b < a, i.e. m' < lane + [rg < q]. Natural order: columns b < min(nn, 32 q + 31)
         // with b < a, then, for lanes of new candidates, columns 128 .. nc - 1. The NW / 4 warps
         // of a lane quarter take every (NW / 4)-th block of the quarter's ranges.
@@ -1355,7 +1365,7 @@ __global__ void __launch_bounds__(BYTES ? 256 : 128, 4) k_join_tc(
 #pragma unroll 1
             for (int rg = 0; rg < 4; ++rg) {
                 const int cnt = nn > rg ? (nn - rg + 3) >> 2 : 0;
-                run(32 * rg, cnt, rg, 4, r_ok ? min(cnt, lane + (rg < q ? 1 : 0)) : 0);
+                run(rg << QS, cnt, rg, 4, r_ok ? min(cnt, lane + (rg < q ? 1 : 0)) : 0);
             }
         }
         rerank(qn);
@@ -1843,7 +1853,7 @@ cudaError_t refine_join(const ShardTable& t, const float* X, const float* inv_no
     bool use_tc = b.join_filter != 1 && b.Xb && du % 16 == 0 && cmn <= 128 && cm <= 256;
     if (use_tc)
         for (int q = 0; q < kTCLists; ++q)
-            if (hb[2 + q] > 0 && tc_layout(hb[2 + kJoinLists + q], du).bytes > 227 * 1024) use_tc = false;
+            if (hb[2 + q] > 0 && tc_layout(hb[2 + kJoinLists + q], du, !bytes && hb[2 + kJoinLists + q] <= kTCSmall).bytes > 227 * 1024) use_tc = false;
     if (use_tc) {
         {
             LaunchScope ls("k_worst_keys", s);
@@ -1854,34 +1864,36 @@ cudaError_t refine_join(const ShardTable& t, const float* X, const float* inv_no
             const int32_t count = hb[2 + q], cmq = hb[2 + kJoinLists + q];
             if (count <= 0) continue;
             b.class_count[q] += count;
-            const TCLayout TL = tc_layout(cmq, du);
-            const int ncols = cmq <= 128 ? 128 : ((cmq + 15) / 16) * 16;   // MMA N (interleaved order: 128)
+            const bool small = !bytes && cmq <= kTCSmall;
+            const TCLayout TL = tc_layout(cmq, du, small);
+            const int ncols = small ? 64 : cmq <= 128 ? 128 : ((cmq + 15) / 16) * 16;   // MMA N (interleaved order: 64 or 128)
             uint32_t cols = 32;
             while ((int)cols < ncols) cols <<= 1;
             const size_t smem = tc_launch_smem(TL, cols);
             const int32_t* list = b.blist + (long long)q * b.blist_cap;
-#define FGIM_LAUNCH_TC4(MT, BY, LG, F8)                                                                           \
+#define FGIM_LAUNCH_TC4(MT, BY, LG, F8, SM)                                                                         \
     do {                                                                                                          \
-        e = cudaFuncSetAttribute(k_join_tc<MT, BY, LG, F8>, cudaFuncAttributeMaxDynamicSharedMemorySize,          \
+        e = cudaFuncSetAttribute(k_join_tc<MT, BY, LG, F8, SM>, cudaFuncAttributeMaxDynamicSharedMemorySize,          \
                                  (int)smem);                                                                      \
         if (e != cudaSuccess) break;                                                                              \
         LaunchScope ls("k_join", s);                                                                              \
-        k_join_tc<MT, BY, LG, F8><<<(unsigned)count, (BY) ? 256 : kTCThreads, smem, s>>>(                           \
+        k_join_tc<MT, BY, LG, F8, SM><<<(unsigned)count, (BY) ? 256 : kTCThreads, smem, s>>>(                           \
             t, X, reinterpret_cast<const __nv_bfloat16*>(b.Xb), b.dp, b.f16, b.X8, b.tcm, inv_norm, g.k, g.ids, b.wk, b.cand,  \
             b.nn, b.no, b.cmax, cmq, cols, list, b.prop_tgt, b.prop_key, b.prop_count, b.prop_cap, b.pcnt, b.pending,     \
             pairs, cands, status);                                                                                \
         e = cudaGetLastError();                                                                                   \
     } while (0)
-#define FGIM_LAUNCH_TC3(MT, BY, LG) FGIM_LAUNCH_TC4(MT, BY, LG, false)
 #define FGIM_LAUNCH_TC(MT, BY)                                                                                    \
     do {                                                                                                          \
-        if (cmq > 128) FGIM_LAUNCH_TC3(MT, BY, true);                                                             \
-        else FGIM_LAUNCH_TC3(MT, BY, false);                                                                      \
+        if (cmq > 128) FGIM_LAUNCH_TC4(MT, BY, true, false, false);                                               \
+        else if (small) FGIM_LAUNCH_TC4(MT, false, false, false, true);                                           \
+        else FGIM_LAUNCH_TC4(MT, BY, false, false, false);                                                        \
     } while (0)
 #define FGIM_LAUNCH_TC8(MT)                                                                                       \
     do {                                                                                                          \
-        if (cmq > 128) FGIM_LAUNCH_TC4(MT, false, true, true);                                                    \
-        else FGIM_LAUNCH_TC4(MT, false, false, true);                                                             \
+        if (cmq > 128) FGIM_LAUNCH_TC4(MT, false, true, true, false);                                             \
+        else if (small) FGIM_LAUNCH_TC4(MT, false, false, true, true);                                            \
+        else FGIM_LAUNCH_TC4(MT, false, false, true, false);                                                      \
     } while (0)
             if (b.fp8) {
                 if (metric == FGIM_L2SQ) FGIM_LAUNCH_TC8(FGIM_L2SQ);
@@ -1896,7 +1908,6 @@ cudaError_t refine_join(const ShardTable& t, const float* X, const float* inv_no
             }
 #undef FGIM_LAUNCH_TC8
 #undef FGIM_LAUNCH_TC
-#undef FGIM_LAUNCH_TC3
 #undef FGIM_LAUNCH_TC4
             if (e != cudaSuccess) return e;
         }
