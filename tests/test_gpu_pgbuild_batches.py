@@ -27,3 +27,19 @@ def test_mean_and_reverse_edges(kind, d, n):
     assert entry == ref_entry
     if kind != "floats":
         assert np.array_equal(adj.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("scale", [1e-38, 1e-42, 1e30])
+def test_mean_of_zeros_and_subnormals(scale):
+    """Rows with zeros of either sign, subnormal and very large coordinates: the medoid is the host builder's."""
+    import paper_2603_21710_gb300 as fg
+    from synth import pgbuild
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    rng = np.random.default_rng(5)
+    X = rng.standard_normal((333, 36)).astype(np.float32)
+    X[::3, ::2] = (X[::3, ::2].astype(np.float64) * scale).astype(np.float32)
+    X[::7, ::5] = 0.0
+    X[1::7, ::5] = -0.0
+    _, entry = fg.build_pg(torch.from_numpy(X).cuda(), M=8, ef=16)
+    assert entry == pgbuild.build_pg(X, 8, 16, 0)[1]
