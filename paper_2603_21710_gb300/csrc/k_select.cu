@@ -61,6 +61,32 @@ __host__ __device__ inline SelectLayout select_layout(int k, int R, int d, int n
     return l;
 }
 
+// The list of a vertex: its entries before the first that is no vertex id (an empty or negative one, or one of N
+// or above, which is reported). Every lane gets their number; position s goes to cid[s] and dl[s] where this warp
+// (vw of the vertex's NW) holds it. Positions past the list are not to be read: they may hold anything.
+template <int NW>
+__device__ __forceinline__ int load_list(const int32_t* __restrict__ ids, const float* __restrict__ dist, int k, long long N,
+                                         int vw, int lane, int32_t* cid, float* dl, int* status) {
+    int nv = 0;
+    bool more = true;
+    for (int s0 = 0; s0 < k; s0 += 32) {
+        const int s = s0 + lane;
+        int32_t id = s < k ? ids[s] : -1;
+        if (id >= N) {
+            atomicOr(status, kErrBounds);
+            id = -1;
+        }
+        if (s < k && (s0 >> 5) % NW == vw) {
+            cid[s] = id;
+            dl[s] = dist[s];
+        }
+        const unsigned none = __ballot_sync(kFull, id < 0);
+        if (more) nv += none ? __ffs(none) - 1 : 32;
+        more = more && none == 0u;
+    }
+    return nv;
+}
+
 // NW warps per vertex: 1 (four vertices per block), or 4 when there are too few vertices to fill the
 // GPU with one warp each; warp w of a vertex then holds the candidates at positions w, w + 4, ..., all in
 // one window, and the warps agree on the next kept neighbour (the smallest position left) once per step.
@@ -95,36 +121,20 @@ __global__ void __launch_bounds__(128, sizeof(RT) == 1 ? 8 : SMALLD ? 5 : 4) k_p
         else __syncthreads();
     };
 
-    // the valid prefix of list(u)
-    int nv = 0;
-    for (int s0 = 0; s0 < k; s0 += 32) {
-        const int s = s0 + lane;
-        int32_t id = s < k ? ids[u * k + s] : -1;
-        if (id >= N) {
-            atomicOr(status, kErrBounds);
-            id = -1;
-        }
-        if (s < k && (s0 >> 5) % NW == vw) {
-            cid[s] = id;
-            dl[s] = dist[u * k + s];
-        }
-        nv += __popc(__ballot_sync(kFull, id >= 0));
-    }
+    const int nv = load_list<NW>(ids + u * k, dist + u * k, k, N, vw, lane, cid, dl, status);
     vsync();
     if (STAGE) {
         const int c16 = d * (int)sizeof(RT) >> 4;   // 16-byte pieces per row
         for (int i = lane; i < nv * c16; i += 32) {
             const int r = i / c16, c = i - r * c16;
-            if (cid[r] >= 0)
-                reinterpret_cast<uint4*>(rows)[i] = reinterpret_cast<const uint4*>(Xr + (long long)cid[r] * d)[c];
+            reinterpret_cast<uint4*>(rows)[i] = reinterpret_cast<const uint4*>(Xr + (long long)cid[r] * d)[c];
         }
     }
     // this warp's candidates
     const int total = nv > vw ? (nv - vw + NW - 1) / NW : 0;
     for (int i = lane; i < total; i += 32) {
         const int t = vw + i * NW;
-        const int32_t v = cid[t];
-        list[i] = (uint16_t)(t | (v >= 0 && T[v] == 1 ? kProtected : 0));
+        list[i] = (uint16_t)(t | (T[cid[t]] == 1 ? kProtected : 0));
     }
     __syncwarp();
     // the window: list[a0 .. m), tested against kept[0 .. ki); list[nxt .. total) has not been looked at
@@ -155,7 +165,7 @@ __global__ void __launch_bounds__(128, sizeof(RT) == 1 ? 8 : SMALLD ? 5 : 4) k_p
         }
         const int tw = kept[ki++];
         const int32_t w = cid[tw];
-        if (a0 == m || w < 0) continue;   // nothing to test, or a hole in the list
+        if (a0 == m) continue;   // nothing to test
         const Query Q = row_query<SMALLD, RT>(STAGE ? rows + tw * d : Xr + (long long)w * d, qs, d, lane);
         const float duw = dl[tw];
         const float inv_w = METRIC == FGIM_COSINE ? inv_norm[w] : 1.f;
@@ -164,8 +174,8 @@ __global__ void __launch_bounds__(128, sizeof(RT) == 1 ? 8 : SMALLD ? 5 : 4) k_p
             const bool has = i0 + lane < m;
             const int a = has ? list[i0 + lane] : 0;
             const int t = a & kListMask;
-            const int32_t v = has ? cid[t] : -1;
-            const bool test = v >= 0 && !(a & kProtected);
+            const int32_t v = has ? cid[t] : 0;
+            const bool test = has && !(a & kProtected);
             const unsigned tm = __ballot_sync(kFull, test);
             bool occ = false;
             if (tm) {
@@ -235,20 +245,7 @@ __global__ void __launch_bounds__(128, 5) k_prune_bytes(
     const int rpi = 32 >> lsh;   // rows per warp load
     const int sub = lane >> lsh, part = lane & ((1 << lsh) - 1);
 
-    int nv = 0;
-    for (int s0 = 0; s0 < k; s0 += 32) {
-        const int s = s0 + lane;
-        int32_t id = s < k ? ids[u * k + s] : -1;
-        if (id >= N) {
-            atomicOr(status, kErrBounds);
-            id = -1;
-        }
-        if (s < k) {
-            cid[s] = id;
-            dl[s] = dist[u * k + s];
-        }
-        nv += __popc(__ballot_sync(kFull, id >= 0));
-    }
+    const int nv = load_list<1>(ids + u * k, dist + u * k, k, N, 0, lane, cid, dl, status);
     __syncwarp();
     uint4 xr[8];   // this lane's row
     uint32_t x2 = 0u;
@@ -288,7 +285,7 @@ __global__ void __launch_bounds__(128, 5) k_prune_bytes(
             for (int q = 0; q < 4; ++q) {
                 const int r = r0 + q * rpi + sub;
                 x[q] = make_uint4(0u, 0u, 0u, 0u);
-                if (r < wn && part < c16n && cid[w0 + r] >= 0)
+                if (r < wn && part < c16n)
                     x[q] = *reinterpret_cast<const uint4*>(X8 + (long long)cid[w0 + r] * d + 16 * part);
             }
 #pragma unroll
@@ -305,8 +302,8 @@ __global__ void __launch_bounds__(128, 5) k_prune_bytes(
                 }
             }
         }
-        const int32_t own = lane < wn ? cid[w0 + lane] : -1;
-        const bool prot = own >= 0 && T[own] == 1;   // never occluded
+        const bool has = lane < wn;
+        const bool prot = has && T[cid[w0 + lane]] == 1;   // never occluded
         __syncwarp();
         if (nk > kManyKept && R <= 32) {
             const unsigned pm = __ballot_sync(kFull, prot);
@@ -328,8 +325,8 @@ __global__ void __launch_bounds__(128, 5) k_prune_bytes(
             __syncwarp();
             continue;
         }
-        unsigned left = __ballot_sync(kFull, own >= 0);
-        if (own >= 0) hold(w0 + lane);
+        unsigned left = __ballot_sync(kFull, has);
+        if (has) hold(w0 + lane);
         for (int ki = 0; left; ++ki) {
             if (ki == nk) {   // the first candidate left is kept
                 const int t = __ffs(left) - 1;
