@@ -640,14 +640,13 @@ static void refine_pass(Ctx& c, const Problem& P, const fgim_params* p, fgim_knn
     ck(refine_merge(*g, b, cnt < (unsigned long long)cap ? (long long)cnt : cap, c.s));
     // vertices whose proposals did not all fit (proposal buffer full) are re-run against the
     // merged lists: a proposal that would have entered a list still beats its (only lower)
-    // worst key and is still absent, so the merged result is the same
-    long long prev_pending = -1;
+    // worst key and is still absent, so the merged result is the same. Every run that fills the buffer
+    // improves lists, also when as many vertices are left as before (each may have lost its last proposals again)
     while (cnt > (unsigned long long)cap) {   // only a full buffer leaves vertices pending
         ck(launch_nonzero_flags(b.pending, N, b.pend_flag, c.s));
         ck(compact_flags(b.pend_flag, N, b.pend_list, b.pend_off, b.scan_tmp, b.scan_bytes, c.s));
         const long long np = c.read_ll(b.pend_off + N);
-        need(np > 0 && np != prev_pending, FGIM_EINTERNAL, "proposal overflow does not shrink");
-        prev_pending = np;
+        need(np > 0, FGIM_EINTERNAL, "proposals were dropped without a pending vertex");
         st->join_reruns += 1;
         need(st->join_reruns < 10000, FGIM_EINTERNAL, "proposal overflow does not shrink");
         ck(cudaMemsetAsync(b.pending, 0, N, c.s));
