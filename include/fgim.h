@@ -377,7 +377,9 @@ void fgim_trim_memory(void);
  *                       returns FGIM_ENOMEM); -1 = off (default).
  * fgim_test_get("pool_used_bytes"): bytes of the current device's scratch pool handed out
  * and not yet handed back (0 whenever no call is running); fgim_test_get("scratch_allocs"):
- * scratch allocations made by the last call on this host thread; -1 for an unknown name.
+ * scratch allocations made by the last call on this host thread; "rev_select_local_bytes" and
+ * "scan_local_bytes": local memory per thread of the reverse-list selection and of the prefix
+ * sums on the current device; -1 for an unknown name.
  */
 int32_t fgim_test_set(const char* knob, int64_t value);
 int64_t fgim_test_get(const char* what);

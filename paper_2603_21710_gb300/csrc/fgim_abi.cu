@@ -1731,6 +1731,14 @@ int64_t fgim_test_get(const char* what) {
         }
         return (int64_t)used;
     }
+    if (std::string(what) == "rev_select_local_bytes" || std::string(what) == "scan_local_bytes") {
+        size_t bytes = 0;
+        if ((what[0] == 'r' ? rev_select_local_bytes(&bytes) : scan_local_bytes(&bytes)) != cudaSuccess) {
+            cudaGetLastError();
+            return -1;
+        }
+        return (int64_t)bytes;
+    }
     return -1;
 }
 

@@ -85,6 +85,7 @@ cudaError_t scan_counts(const int32_t* in, long long n, long long* out, void* sc
 cudaError_t scan_counts2(const int32_t* in0, const int32_t* in1, long long n, long long* out0, long long* out1,
                          void* scratch, size_t scratch_bytes, cudaStream_t s);   // two arrays of n at once
 size_t scan_scratch_bytes(long long n);
+cudaError_t scan_local_bytes(size_t* bytes);   // local memory per thread of the scan kernels (test hook)
 cudaError_t launch_inv_norms(const float* X, long long n, int d, float* inv, cudaStream_t s);
 // the same of BF16 rows (8-byte aligned), without an FP32 copy
 cudaError_t launch_inv_norms_bf16(const uint16_t* X, long long n, int d, float* inv, cudaStream_t s);
@@ -161,6 +162,7 @@ struct RefineBuffers {
     const uint8_t* X8;
 };
 
+cudaError_t rev_select_local_bytes(size_t* bytes);   // local memory per thread of k_rev_select (test hook)
 cudaError_t refine_visit(const fgim_knng& g, int rev_cap, RefineBuffers& b, cudaStream_t s);
 cudaError_t refine_join(const ShardTable& t, const float* X, const float* inv_norm, int metric, const fgim_knng& g,
                         RefineBuffers& b, const int32_t* vlist, long long nv, unsigned long long* pairs,

@@ -25,7 +25,8 @@ __device__ __forceinline__ long long block_sum(long long v, long long* sh) {
     return s;
 }
 
-// One or two arrays (blockIdx.y) are scanned at once.
+// One or two arrays (blockIdx.y) are scanned at once. The arrays are selected, not indexed by blockIdx.y: an index
+// would put the parameters in local memory.
 struct ScanJob {
     const int32_t* in[2];
     long long* out[2];
@@ -34,7 +35,7 @@ struct ScanJob {
 // sums[y * gridDim.x + b] = the sum of tile b of array y
 __global__ void __launch_bounds__(kScanThreads) k_scan_sums(ScanJob job, long long n, long long* __restrict__ sums) {
     __shared__ long long sh[kScanThreads / 32];
-    const int32_t* in = job.in[blockIdx.y];
+    const int32_t* in = blockIdx.y ? job.in[1] : job.in[0];
     const long long base = (long long)blockIdx.x * kScanTile;
     long long s = 0;
 #pragma unroll
@@ -52,8 +53,8 @@ template <bool FLAT>
 __global__ void __launch_bounds__(kScanThreads) k_scan_write(ScanJob job, long long n, const long long* __restrict__ pre) {
     __shared__ long long sh[kScanThreads / 32];
     __shared__ long long warp_sum[kScanThreads / 32];
-    const int32_t* in = job.in[blockIdx.y];
-    long long* out = job.out[blockIdx.y];
+    const int32_t* in = blockIdx.y ? job.in[1] : job.in[0];
+    long long* out = blockIdx.y ? job.out[1] : job.out[0];
     const long long* p = pre + (long long)blockIdx.y * gridDim.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     long long before = 0;
@@ -167,6 +168,18 @@ cudaError_t scan_counts2(const int32_t* in0, const int32_t* in1, long long n, lo
     if (scratch_bytes < scan_scratch_bytes(n)) return cudaErrorInvalidValue;
     const ScanJob job = {{in0, in1}, {out0, out1}};
     return scan_job(job, 2, n, reinterpret_cast<long long*>(scratch), s);
+}
+
+cudaError_t scan_local_bytes(size_t* bytes) {
+    const void* kernels[3] = {(const void*)k_scan_sums, (const void*)k_scan_write<true>, (const void*)k_scan_write<false>};
+    *bytes = 0;
+    for (const void* k : kernels) {
+        cudaFuncAttributes a;
+        const cudaError_t e = cudaFuncGetAttributes(&a, k);
+        if (e != cudaSuccess) return e;
+        *bytes = std::max(*bytes, a.localSizeBytes);
+    }
+    return cudaSuccess;
 }
 
 __global__ void k_compact(const int32_t* __restrict__ flag, long long n, const long long* __restrict__ off,
