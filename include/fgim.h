@@ -104,12 +104,12 @@ typedef struct {
     int32_t rev_cap;         /* cap of each reverse list in Visit; 0 = k */
     int32_t ensure_reachable;/* 1 = run the reachability fix after Alg. 5 */
     int32_t reach_beam;      /* pool of the searches of the reachability fix; 0 = 64 */
-    int32_t join_filter;     /* fgim_precision of Update's candidate distances: 0 = BF16 tensor-core tile
-                                (tcgen05), 1 = FP32 SIMT tile, 2 = FP8 E4M3 tensor-core tile with one
-                                scale per vector. Every form re-ranks its survivors with the exact FP32
-                                distance, so the lists are the same; only speed differs. Passes whose
-                                shapes a tensor-core tile does not cover (BF16: dim % 16 != 0; FP8:
-                                dim % 32 != 0; both: |C_n| > 128, |C| > 256) use the FP32 tile. */
+    int32_t join_filter;     /* fgim_precision of Update's candidate distances: 0 = 16-bit tensor-core tile
+                                (tcgen05), 1 = FP32 SIMT tile, 2 = FP8 E4M3 tensor-core tile where it is
+                                fine enough for the lists, else the 16-bit one. Every form re-ranks its
+                                survivors with the exact FP32 distance, so the lists are the same; only
+                                speed differs. Rows are padded with zeros to whole MMA steps (any dim).
+                                Passes with |C_n| > 128 or |C| > 256 use the FP32 tile. */
     int32_t byte_rows;       /* 0 = auto: when every coordinate is an integer in [0, 255] and dim <= 128,
                                 dim % 16 == 0, the searches, the join's re-rank and the prune read one
                                 byte per coordinate and form the distances in exact integer arithmetic
@@ -134,9 +134,16 @@ typedef enum { FGIM_PRUNE_ALPHA_RNG = 0, FGIM_PRUNE_MRNG = 1, FGIM_PRUNE_TAU_MNG
 /* Precision of Update's candidate distances (fgim_params.join_filter). The reduced-precision forms
  * are filters: a pair is re-ranked with the exact FP32 distance unless a rigorous bound (Cauchy-
  * Schwarz on the rows' conversion errors plus the FP32 accumulation error of the tile) shows it
- * cannot enter the list, so the kept ids equal the FP32 form's. FP8: s = amax|x| / 448 per vector,
- * q = saturating round-to-nearest E4M3 of x / s, the tile forms sum q_a q_b, scaled by s_a s_b. */
+ * cannot enter the list, so the kept ids equal the FP32 form's. 16-bit: BF16 rows where every coordinate
+ * is a BF16 value (byte rows, BF16 storage, or found so), else FP16 of the row times a power of two that
+ * brings its largest coordinate near 2^14. FP8: s = amax|x| / 448 per vector, q = saturating
+ * round-to-nearest E4M3 of x / s, the tile forms sum q_a q_b, scaled by s_a s_b; when the first pass finds
+ * that for more than half of the lists the error bound of two such rows exceeds 1/8 of the distance of the
+ * list's last entry, E4M3 would decide next to nothing and the call's passes take the 16-bit tile.
+ * fgim_last_join_operand tells which copy a call used. */
 typedef enum { FGIM_PREC_BF16 = 0, FGIM_PREC_FP32 = 1, FGIM_PREC_FP8E4M3 = 2 } fgim_precision;
+/* The vectors' copy that Update's tensor-core tile read (NONE: no pass, or join_filter FP32). */
+typedef enum { FGIM_OPERAND_NONE = 0, FGIM_OPERAND_BF16 = 1, FGIM_OPERAND_FP16 = 2, FGIM_OPERAND_E4M3 = 3 } fgim_operand;
 
 /* k-NNG buffers, caller-owned device memory: [n, k] each. */
 typedef struct {
@@ -349,6 +356,10 @@ fgim_status fgim_build_pg(const void* vectors, int64_t n, int32_t dim, int32_t d
 /* Counters of the last merge/search call made by this host thread. */
 void fgim_last_stats(fgim_stats* out);
 
+/* The copy of the vectors that Update's tensor-core tile read in the last call on this host thread
+ * (join_class of the stats tells how many vertices took a tensor-core tile at all). */
+fgim_operand fgim_last_join_operand(void);
+
 /*
  * Scratch memory: every call takes its scratch from a stream-ordered pool the library keeps
  * per device, and the pool keeps what it has mapped for later calls (a merge of 1M vectors
@@ -372,11 +383,15 @@ void fgim_trim_memory(void);
  *                       (and at most 128 candidates) one warp per vertex on byte rows, the
  *                       rest in the tensor-core tile (same results; 0 = never, a large value =
  *                       every eligible vertex); -1 = the default cut-off (10).
+ *   "fp8_force"         1: join_filter FP8 takes the E4M3 tile even where its bound is too coarse
+ *                       for the lists (same results); 0 = default.
+ *   "pool_high_bytes"   any value: the scratch pool's high-water mark starts over.
  *   "fail_alloc_after"  >= 0: the scratch allocation of a call that comes after this many
  *                       successful ones fails as if the device were out of memory (the call
  *                       returns FGIM_ENOMEM); -1 = off (default).
  * fgim_test_get("pool_used_bytes"): bytes of the current device's scratch pool handed out
- * and not yet handed back (0 whenever no call is running); fgim_test_get("scratch_allocs"):
+ * and not yet handed back (0 whenever no call is running); "pool_high_bytes": the most handed out
+ * at once since the mark was set back; fgim_test_get("scratch_allocs"):
  * scratch allocations made by the last call on this host thread; "rev_select_local_bytes" and
  * "scan_local_bytes": local memory per thread of the reverse-list selection and of the prefix
  * sums on the current device; -1 for an unknown name.

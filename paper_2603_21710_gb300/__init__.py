@@ -16,17 +16,19 @@ from typing import List, Optional, Sequence
 import torch
 
 from . import _lib
-from ._lib import FgimError, KNNG, Graph, Params, Shard, check, last_stats, load  # noqa: F401
+from ._lib import (FgimError, KNNG, Graph, Params, Shard, check, last_join_operand, last_stats,  # noqa: F401
+                   load)
 
 __all__ = ["MergeInput", "merge", "merge_batch", "merge_host", "hnsw_levels", "hnsw_layer", "build_layers",
            "search_hnsw", "build_pg", "cross_query", "refine_pass", "indegree_repair", "prune",
-           "reverse_insert", "reach_fix", "search", "last_stats", "load", "launch_count", "FgimError",
+           "reverse_insert", "reach_fix", "search", "last_stats", "last_join_operand", "load", "launch_count", "FgimError",
            "FLAG_NEW", "FLAG_REPLACED", "profiling"]
 
 FLAG_NEW = 1
 FLAG_REPLACED = 2
-# Update's candidate-distance precision: BF16 tensor-core tile, FP32 SIMT tile or FP8 E4M3
-# tensor-core tile with per-vector scales (same results: survivors are re-ranked exactly)
+# Update's candidate-distance precision: 16-bit tensor-core tile (BF16 rows where exact, else scaled FP16), FP32 SIMT tile,
+# or FP8 E4M3 tensor-core tile with per-vector scales, which gives way to the 16-bit one where it is too coarse for the
+# lists (last_join_operand); same results: survivors are re-ranked exactly
 JOIN_FILTERS = {"tc": 0, "bf16": 0, "fp32": 1, "simt": 1, "fp8": 2, "e4m3": 2, 0: 0, 1: 1, 2: 2}
 # row storage: "auto" reads one byte per coordinate when the data allow it (integers in
 # [0, 255], d <= 128, d % 16 == 0; distances are then exact integers, equal to the FP32

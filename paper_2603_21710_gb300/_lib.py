@@ -107,6 +107,7 @@ EXPORTS = {
                                            ctypes.c_void_p, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32,
                                            ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]),
     "fgim_last_stats": (None, [ctypes.c_void_p]),
+    "fgim_last_join_operand": (ctypes.c_int, []),
     "fgim_graph_alloc": (ctypes.c_int, [ctypes.c_int64, ctypes.c_int32, ctypes.c_void_p]),
     "fgim_graph_free": (None, [ctypes.c_void_p]),
     "fgim_autotune": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p, ctypes.c_char_p,
@@ -160,6 +161,15 @@ def last_stats() -> dict:
     s = Stats()
     load().fgim_last_stats(ctypes.byref(s))
     return s.as_dict()
+
+
+JOIN_OPERANDS = ("none", "bf16", "fp16", "e4m3")
+
+
+def last_join_operand() -> str:
+    """The copy of the vectors that Update's tensor-core tile read in this thread's last call: "bf16", "fp16",
+    "e4m3", or "none" (no refinement pass, or join_filter "fp32")."""
+    return JOIN_OPERANDS[load().fgim_last_join_operand()]
 
 
 def test_set(knob: str, value: int) -> None:

@@ -35,6 +35,7 @@ struct PendingEvent {
 static thread_local std::vector<PendingEvent> t_pending;
 static thread_local fgim_stats t_stats;
 static thread_local std::string t_last_error;
+static thread_local int t_join_operand = FGIM_OPERAND_NONE;   // of the current call's Update tile
 
 LaunchScope::LaunchScope(const char* n, cudaStream_t s) : name(n), stream(s), e0(nullptr), e1(nullptr), timed(false) {
     g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -110,6 +111,7 @@ static std::atomic<int> g_test_hop_budget{0};
 static std::atomic<long long> g_test_fail_after{-1};
 static std::atomic<int> g_test_batch_union{1};
 static std::atomic<int> g_test_sparse_nn{-1};   // >= 0: the cut-off of the warp-per-vertex Update form
+static std::atomic<int> g_test_fp8_force{0};    // 1: join_filter FP8 takes the E4M3 tile however coarse it is
 static thread_local long long t_allocs = 0;   // scratch allocations of the current call
 
 static cudaMemPool_t lib_pool() {
@@ -163,6 +165,12 @@ class Scratch {
         return static_cast<T*>(p);
     }
     bool ok() const { return ok_; }
+    void give_back(void* p) {   // before the call ends; work already on the stream may still use it
+        auto it = std::find(ptrs_.begin(), ptrs_.end(), p);
+        if (it == ptrs_.end()) return;
+        ptrs_.erase(it);
+        cudaFreeAsync(p, s_);
+    }
     void release() {
         for (void* p : ptrs_) cudaFreeAsync(p, s_);
         ptrs_.clear();
@@ -604,11 +612,13 @@ static void join_operand(Ctx& c, const Problem& P, const fgim_knng* g, RefineBuf
         int* coarse = c.alloc<int>(1);
         ck(launch_prep_fp8(P.X, N, P.d, b.dp, Xq, b.tcm, c.s));
         ck(launch_fp8_coarse(*g, b.tcm, P.inv, P.metric, coarse, c.s));
-        if (2LL * c.read_i32(coarse) <= N) {
+        if (2LL * c.read_i32(coarse) <= N || g_test_fp8_force.load(std::memory_order_relaxed) != 0) {
             b.Xb = Xq;   // one byte per coordinate, addressed like 16-bit pairs
             b.fp8 = true;
+            t_join_operand = FGIM_OPERAND_E4M3;
             return;
         }
+        c.sc.give_back(Xq);   // no larger than the 16-bit copy, which takes its place
     }
     b.dp = (P.d + 15) / 16 * 16;
     b.Xb = c.alloc<uint16_t>(N * b.dp);
@@ -617,10 +627,12 @@ static void join_operand(Ctx& c, const Problem& P, const fgim_knng* g, RefineBuf
         ck(launch_prep_f16(P.X, N, P.d, b.dp, b.Xb, b.tcm, not_bf16, c.s));
         if (c.read_i32(not_bf16) != 0) {
             b.f16 = true;
+            t_join_operand = FGIM_OPERAND_FP16;
             return;
         }
     }
     ck(launch_prep_bf16(P.X, N, P.d, b.dp, b.Xb, b.tcm, c.s));
+    t_join_operand = FGIM_OPERAND_BF16;
 }
 
 static void refine_pass(Ctx& c, const Problem& P, const fgim_params* p, fgim_knng* g, fgim_stats* st,
@@ -790,6 +802,7 @@ static fgim_status guarded(F&& f) {
 static void begin_call() {
     std::memset(&t_stats, 0, sizeof(t_stats));
     t_last_error.clear();
+    t_join_operand = FGIM_OPERAND_NONE;
     t_allocs = 0;
 }
 
@@ -1705,6 +1718,22 @@ int32_t fgim_test_set(const char* knob, int64_t value) {
         g_test_sparse_nn.store(value >= 0 ? (int)std::min<int64_t>(value, 1 << 20) : -1);
         return 1;
     }
+    if (k == "fp8_force") {
+        g_test_fp8_force.store(value != 0 ? 1 : 0);
+        return 1;
+    }
+    if (k == "pool_high_bytes") {   // the high-water mark starts over
+        int dev = 0;
+        uint64_t zero = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        std::lock_guard<std::mutex> lk(g_pool_mu);
+        auto it = g_pools.find(dev);
+        if (it != g_pools.end()) cudaMemPoolSetAttribute(it->second, cudaMemPoolAttrUsedMemHigh, &zero);
+        return 1;
+    }
     if (k == "fail_alloc_after") {
         g_test_fail_after.store(value >= 0 ? (long long)value : -1);
         return 1;
@@ -1715,7 +1744,7 @@ int32_t fgim_test_set(const char* knob, int64_t value) {
 int64_t fgim_test_get(const char* what) {
     if (!what) return -1;
     if (std::string(what) == "scratch_allocs") return (int64_t)t_allocs;   // of the last call on this thread
-    if (std::string(what) == "pool_used_bytes") {
+    if (std::string(what) == "pool_used_bytes" || std::string(what) == "pool_high_bytes") {
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) {
             cudaGetLastError();
@@ -1725,7 +1754,8 @@ int64_t fgim_test_get(const char* what) {
         auto it = g_pools.find(dev);
         if (it == g_pools.end()) return 0;
         uint64_t used = 0;
-        if (cudaMemPoolGetAttribute(it->second, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+        const cudaMemPoolAttr attr = what[5] == 'u' ? cudaMemPoolAttrUsedMemCurrent : cudaMemPoolAttrUsedMemHigh;
+        if (cudaMemPoolGetAttribute(it->second, attr, &used) != cudaSuccess) {
             cudaGetLastError();
             return -1;
         }
@@ -1750,6 +1780,8 @@ void fgim_trim_memory(void) {
 void fgim_last_stats(fgim_stats* out) {
     if (out) *out = t_stats;
 }
+
+fgim_operand fgim_last_join_operand(void) { return static_cast<fgim_operand>(t_join_operand); }
 
 const char* fgim_strerror(fgim_status s) {
     switch (s) {
