@@ -9,7 +9,9 @@ host before timing.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
 
-Prints one JSON line. Under torchrun (N > 1) every rank merges its own replica of the
+Prints one JSON line on stdout: the headline figures and one short entry per other workload, a few KB (what
+collects such lines may keep no more). The whole record, with every kernel's time, step and roofline, goes to
+stderr as one line {"record": ...} before it. Under torchrun (N > 1) every rank merges its own replica of the
 workload (weak scaling, no collective on the data path); value = all ranks' points /
 the slowest rank's time.
 """
@@ -105,6 +107,37 @@ def max_over_ranks(x: float, ws: int, device=None) -> float:
     t = torch.tensor([float(x)], dtype=torch.float64, device=device)
     dist.all_reduce(t, op=dist.ReduceOp.MAX)
     return float(t.item())
+
+
+# ---------------------------------------------------------------------------- the printed line
+CONFIG_KEYS = ("value", "unit", "ms_per_step", "join_operand", "recall@10", "recall@10_gpu", "rows_identical_to_oracle",
+               "error")
+
+
+def _short(v):
+    """Floats to seven significant digits, texts to 200 characters (the record has them whole)."""
+    if isinstance(v, dict):
+        return {k: _short(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [_short(x) for x in v]
+    if isinstance(v, float):
+        return float(f"{v:.7g}")
+    return v[:200] if isinstance(v, str) else v
+
+
+def headline(rec):
+    """The part of a record that is printed as the result line: what the metric is judged by."""
+    line = {k: v for k, v in rec.items() if k not in ("kernels", "roofline_by_kernel", "merge_stats", "step_ms", "plain_fp32",
+                                                       "masked", "hnsw", "input_pg_build", "stage_a_work_model", "configs")}
+    if rec.get("e2e"):
+        line["e2e"] = {k: v for k, v in rec["e2e"].items() if not isinstance(v, (list, tuple))}
+    for k in ("plain_fp32", "masked", "hnsw", "input_pg_build"):
+        if rec.get(k):
+            line[k] = {q: rec[k][q] for q in ("value", "ms_per_step", "same_graph", "build_ms", "recall@10", "gpu_ms", "equal")
+                       if q in rec[k]}
+    if "configs" in rec:
+        line["configs"] = {name: {k: c[k] for k in CONFIG_KEYS if k in c} for name, c in rec["configs"].items()}
+    return _short(line)
 
 
 # ---------------------------------------------------------------------------- inputs
@@ -852,7 +885,8 @@ def run_fgim(args):
             except Exception as ex:   # a sub-record that fails is reported, not fatal to the headline line
                 line["configs"][name] = {"error": f"{type(ex).__name__}: {ex}"}
                 torch.cuda.synchronize()
-    print(json.dumps(line), flush=True)
+    print(json.dumps({"record": line}), file=sys.stderr, flush=True)
+    print(json.dumps(headline(line)), flush=True)
 
 
 def measure_batched(fg, dev, peaks, n_merges, lo, hi, steps, warmup):
