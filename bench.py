@@ -49,7 +49,7 @@ def parse():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--join-filter", default="tc", choices=["tc", "fp32"],
-                    help="Update's pair filter: BF16 tensor-core tile (default) or FP32 SIMT tile")
+                    help="Update's pair filter: 16-bit tensor-core tile (default) or FP32 SIMT tile")
     ap.add_argument("--no-plain", action="store_true", help="skip timing the plain FP32 form alongside")
     ap.add_argument("--no-masked", action="store_true",
                     help="skip timing the merge with invalid vertices (a quarter of them) alongside")
@@ -63,7 +63,7 @@ def parse():
     ap.add_argument("--batched-hi", type=int, default=200_000)
     ap.add_argument("--configs", default="small,precision,fp8,batched",
                     help="other workloads timed after the headline one, each in its own sub-record: "
-                         "'precision' (1M d=96 IP, BF16 filter against plain FP32), 'fp8' (1M d=960, 8 uneven "
+                         "'precision' (1M d=96 IP, 16-bit filter against plain FP32), 'fp8' (1M d=960, 8 uneven "
                          "shards), 'batched' (64 merges, ~4M points, d=768 BF16 cosine, one call), 'small' (20k, "
                          "d=32, with the single-thread oracle); '' or 'none' = none")
     ap.add_argument("--no-autotune", action="store_true",
@@ -535,7 +535,7 @@ def timed_merges(fg, inp, kw, steps, warmup, profile=False):
             if n:
                 kernels[name] = {"launches": n, "ms": ms}
     return {"step_ms": [a.elapsed_time(b) for a, b in ev], "kernels": kernels, "out": out,
-            "launches": fg.launch_count() - launches0}
+            "launches": fg.launch_count() - launches0, "operand": fg.last_join_operand()}
 
 
 def oracle_sample_check(fg, recipe, n, kw, metric_name, dev, filter_, nq=1000, host_graphs=False):
@@ -597,7 +597,7 @@ def measure_small(fg, dev, peaks):
     return {"workload": "small: N=20,000 (2 x 10,000), d=32, 50-cluster Gaussian mixture, squared L2, input PGs "
                         "M=16 ef=64, k=16, R=32, alpha=1.2, I_max=3",
             "value": w.N / (ms_c * 1e-3), "unit": UNIT, "ms_per_step": ms_c, "steps": 5, "warmup": 3,
-            "form": "BF16 tensor-core join filter", "l2_policy": "L2-resident (2.6 MB of vectors): a parity workload",
+            "form": "16-bit tensor-core join filter", "join_operand": ch["operand"], "l2_policy": "L2-resident (2.6 MB of vectors): a parity workload",
             "plain_fp32": {"value": w.N / (ms_p * 1e-3), "unit": UNIT, "ms_per_step": ms_p,
                            "same_graph": bool(torch.equal(pl["out"]["ids"], ch["out"]["ids"]))},
             "oracle": {"seconds_1_thread": times[1], "seconds_all_threads": times[0], "cores": os.cpu_count() or 1,
@@ -608,7 +608,7 @@ def measure_small(fg, dev, peaks):
 
 
 def measure_config(fg, name, dev, peaks, steps=2, warmup=1, nq_eval=1000):
-    """One sub-record: the chosen form (BF16 tensor-core join filter) and the plain FP32 form
+    """One sub-record: the chosen form (tensor-core join filter) and the plain FP32 form
     (FP32 rows, FP32 SIMT join filter) of one workload at full size, the roofline of the chosen
     form's dominant kernel and the merged graph's search recall@10 at beam 64."""
     import torch
@@ -636,6 +636,7 @@ def measure_config(fg, name, dev, peaks, steps=2, warmup=1, nq_eval=1000):
         ot = timed_merges(fg, inp, dict(kw, join_filter=jf), 1, 0)
         ms_o = float(np.mean(ot["step_ms"]))
         others[jf] = {"value": w.N / (ms_o * 1e-3), "unit": UNIT, "ms_per_step": ms_o, "steps": 1,
+                      "join_operand": ot["operand"],
                       "same_graph": bool(torch.equal(ot["out"]["ids"], ch["out"]["ids"]))}
         del ot
     ms_c, ms_p = float(np.mean(ch["step_ms"])), float(np.mean(pl["step_ms"]))
@@ -654,9 +655,10 @@ def measure_config(fg, name, dev, peaks, steps=2, warmup=1, nq_eval=1000):
                 for k_ in ("k_cross_query", "k_join", "k_prune") if k_ in rk}
     rec = {"workload": c["workload"], "N": w.N, "d": w.d, "shards": w.shard_sizes, "value": w.N / (ms_c * 1e-3),
            "unit": UNIT, "ms_per_step": ms_c, "steps": steps, "warmup": warmup, "step_ms": ch["step_ms"],
-           "form": {"tc": "BF16", "fp8": "FP8 E4M3 (per-vector scales)"}[c["filter"]] +
+           "form": {"tc": "16-bit", "fp8": "FP8 E4M3 (16-bit where too coarse)"}[c["filter"]] +
                    " tensor-core join filter with exact FP32 re-rank, FP32 rows elsewhere",
-           "other_forms": {{"tc": "bf16"}.get(k_, k_): v for k_, v in others.items()},
+           "join_operand": ch["operand"],   # the copy that Update's tile read
+           "other_forms": {{"tc": "16-bit"}.get(k_, k_): v for k_, v in others.items()},
            "plain_fp32": {"value": w.N / (ms_p * 1e-3), "unit": UNIT, "ms_per_step": ms_p, "steps": 1,
                           "form": "FP32 rows, FP32 SIMT join filter",
                           "same_graph": bool(torch.equal(pl["out"]["ids"], ch["out"]["ids"]))},
