@@ -208,9 +208,10 @@ static inline void need(bool ok, fgim_status st, const char* what) {
 }
 
 // counters on the device: [0] ndc, [1] hops, [2] pairs, [3] repaired, [4] attached, [5] candidates joined,
-// [6] zero-indegree vertices of the last repair, [8] the beam searches' item counter
+// [6] zero-indegree vertices of the last repair, [kItemCounter] the beam searches' item counter
 struct Ctx {
     static constexpr int kCtxWords = 18;
+    static_assert(kItemCounter < 16, "the status words follow the 16 counters");
     cudaStream_t s;
     Scratch sc;
     int* status = nullptr;

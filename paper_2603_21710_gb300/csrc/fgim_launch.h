@@ -8,6 +8,9 @@
 
 namespace fgim {
 
+// a call's counters[kItemCounter]: the items a beam-search launch has handed out to its warps (zeroed by the launch)
+constexpr int kItemCounter = 8;
+
 // ---- k_search.cu
 // X: FP32 rows; X8: the same rows as bytes when every coordinate is an integer in [0, 255]
 // (searches then read X8, with identical results), else nullptr

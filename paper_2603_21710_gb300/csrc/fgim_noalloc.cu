@@ -28,7 +28,12 @@ namespace fgim {
 // largest base set and query batch whose cosine norms fit the array
 constexpr long long kNoAllocMaxBase = 1LL << 20;
 constexpr long long kNoAllocMaxQueries = 1LL << 16;
-constexpr size_t kNoAllocHeader = 256;   // status word (int) and two 64-bit counters, padded
+// status words (int[4]) at 0, the search's 64-bit counters at kNoAllocCounters: evaluations, expansions and, the last of
+// them, the item counter that warps take their queries from (counters[kItemCounter])
+constexpr size_t kNoAllocCounters = 64;
+constexpr size_t kNoAllocHeader = 256;
+static_assert(kNoAllocCounters + (kItemCounter + 1) * sizeof(unsigned long long) <= kNoAllocHeader,
+              "the header holds every counter a search writes");
 constexpr size_t kNoAllocBytes = kNoAllocHeader + (size_t)(kNoAllocMaxBase + kNoAllocMaxQueries) * sizeof(float);
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
@@ -86,7 +91,7 @@ fgim_status fgim_search_noalloc(const void* base, int64_t n, int32_t dim, int32_
     }
     cudaStream_t s = (cudaStream_t)stream;
     int* status = reinterpret_cast<int*>(scratch);
-    unsigned long long* counters = reinterpret_cast<unsigned long long*>(scratch + 64);
+    unsigned long long* counters = reinterpret_cast<unsigned long long*>(scratch + kNoAllocCounters);
     float* inv = reinterpret_cast<float*>(scratch + kNoAllocHeader);
     float* qinv = inv + kNoAllocMaxBase;
     cudaError_t e = cudaMemsetAsync(scratch, 0, kNoAllocHeader, s);   // the status and counters start at zero

@@ -586,7 +586,7 @@ __host__ __device__ inline WarpLayout warp_layout(int d, int L, int htbits, int 
 static inline int beam_warps(int d) { return d <= 128 ? 4 : 1; }
 
 // Grid of a beam-search kernel over nq items of rows of d coordinates, and the counter its warps take
-// their items from: *next (counters[8], zeroed here) hands out the items after the first of every warp;
+// their items from: *next (counters[kItemCounter], zeroed here) hands out the items after the first of every warp;
 // nullptr: one item per warp (few items, wide rows).
 template <typename K>
 cudaError_t beam_grid(K kernel, int d, int wpb, size_t smem, long long nq, unsigned long long* counters, unsigned* blocks,
@@ -602,7 +602,7 @@ cudaError_t beam_grid(K kernel, int d, int wpb, size_t smem, long long nq, unsig
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, wpb * 32, smem)) != cudaSuccess) return e;
     if (per_sm < 1 || need <= (long long)per_sm * sms) return e;
     *blocks = (unsigned)(per_sm * sms);
-    *next = counters + 8;
+    *next = counters + kItemCounter;
     return cudaMemsetAsync(*next, 0, sizeof(**next), s);
 }
 
