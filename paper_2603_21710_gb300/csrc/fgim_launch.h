@@ -100,7 +100,6 @@ cudaError_t launch_valid_flags(const uint8_t* mask, long long n, int32_t* flag, 
 cudaError_t launch_phi(const int32_t* flag, const long long* off, long long n, int32_t* phi, cudaStream_t s);
 // out[r] = X[src[r]] for r < nv (rows of d floats)
 cudaError_t launch_gather_rows(const float* X, const int32_t* src, long long nv, int d, float* out, cudaStream_t s);
-cudaError_t launch_fill_i32(int32_t* p, long long n, int32_t v, cudaStream_t s);
 // indices i (ascending) with flag[i] != 0, written to out; count to *count (device)
 cudaError_t compact_flags(const int32_t* flag, long long n, int32_t* out, long long* offsets_scratch,
                           void* scan_scratch, size_t scan_bytes, cudaStream_t s);

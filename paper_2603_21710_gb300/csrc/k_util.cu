@@ -197,18 +197,6 @@ cudaError_t compact_flags(const int32_t* flag, long long n, int32_t* out, long l
     return cudaGetLastError();
 }
 
-__global__ void k_fill_i32(int32_t* p, long long n, int32_t v) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = v;
-}
-
-cudaError_t launch_fill_i32(int32_t* p, long long n, int32_t v, cudaStream_t s) {
-    if (n <= 0) return cudaSuccess;
-    LaunchScope ls("k_fill_i32", s);
-    k_fill_i32<<<(unsigned)cdiv(n, 256), 256, 0, s>>>(p, n, v);
-    return cudaGetLastError();
-}
-
 // float4 chunk c of an FP32 row, or of a BF16 row (decoded exactly)
 __device__ __forceinline__ float4 norm_chunk(const float* row, int c) { return reinterpret_cast<const float4*>(row)[c]; }
 __device__ __forceinline__ float4 norm_chunk(const uint16_t* row, int c) {
