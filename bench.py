@@ -373,7 +373,7 @@ def row_bytes(w) -> int:
 TRAFFIC_SOURCES = {
     "k_cross_query": ["k_cross.cu", "k_cross.cuh", "k_beam.cuh"],
     "k_join": ["k_refine.cu", "tc_sm100.cuh"],   # the Update launches: k_join_tc and k_join_sparse
-    "k_prune": ["k_prune.cu"],
+    "k_prune": ["k_select.cu", "k_beam.cuh"],
 }
 
 
