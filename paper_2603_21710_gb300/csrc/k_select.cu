@@ -67,8 +67,7 @@ __host__ __device__ inline SelectLayout select_layout(int k, int R, int d, int n
 template <int NW>
 __device__ __forceinline__ int load_list(const int32_t* __restrict__ ids, const float* __restrict__ dist, int k, long long N,
                                          int vw, int lane, int32_t* cid, float* dl, int* status) {
-    int nv = 0;
-    bool more = true;
+    int nv = k;
     for (int s0 = 0; s0 < k; s0 += 32) {
         const int s = s0 + lane;
         int32_t id = s < k ? ids[s] : -1;
@@ -81,8 +80,7 @@ __device__ __forceinline__ int load_list(const int32_t* __restrict__ ids, const 
             dl[s] = dist[s];
         }
         const unsigned none = __ballot_sync(kFull, id < 0);
-        if (more) nv += none ? __ffs(none) - 1 : 32;
-        more = more && none == 0u;
+        if (none) nv = min(nv, s0 + __ffs(none) - 1);
     }
     return nv;
 }
