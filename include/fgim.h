@@ -59,7 +59,8 @@ typedef enum { FGIM_L2SQ = 0, FGIM_IP = 1, FGIM_COSINE = 2 } fgim_metric;
 
 /* Storage of the input vectors. BF16 vectors (bfloat16, round-to-nearest-even encodings of
  * the values the caller means) are decoded once per call into an FP32 working copy on the
- * device; every distance is that of the decoded values. */
+ * device, except by the searches of rows wider than 128 coordinates, which read them as they
+ * are; every distance is that of the decoded values. */
 typedef enum { FGIM_F32 = 0, FGIM_BF16 = 1 } fgim_dtype;
 
 /* Size limits of the library. */
@@ -268,7 +269,8 @@ fgim_status fgim_reach_fix(const fgim_shard* shards, int32_t h, const fgim_param
 /*
  * Alg. 1 over a merged graph for nq queries: pool `beam` (<= FGIM_MAX_L), returns the
  * first `topk` (<= beam) results. base: [n, dim] vectors in global-id order; base and
- * queries are both in `dtype` (BF16 ones are decoded into FP32 scratch first).
+ * queries are both in `dtype`. A BF16 base of up to 128 coordinates, or not 8-byte aligned, is
+ * decoded into FP32 scratch first; a wider one is read as stored.
  */
 fgim_status fgim_search(const void* base, int64_t n, int32_t dim, int32_t dtype, int32_t metric,
                         const int32_t* graph_ids, int32_t R, int32_t entry, const void* queries, int32_t nq,

@@ -34,7 +34,11 @@ constexpr long long kTeamWide = 304;         // two blocks per SM
 // Queries up to which a block each is faster than a warp each. Wide rows (100k, d = 768 BF16, cosine): 100
 // queries 0.74 -> 0.33 ms, 300: 0.69 -> 0.38, 1,000: 0.73 and 0.69 (and the FP32 d = 960 form slower). Rows of up to
 // 128 coordinates: never (one query 0.122 and 0.132 ms, 1,000: 0.26 and 0.31): there the leader's own steps
-// are the chain. With HNSW layers the single launch counts: 1,001 queries over six layers 0.34 -> 0.25 ms.
+// are the chain. With HNSW layers the single launch counts (a warp each, a launch per layer, against a block each; pool
+// 64, layers' pool 8): 1,000 queries of 100k d = 96 0.345 -> 0.254 ms, 60k d = 768 BF16 0.735 -> 0.615, 60k d = 960
+// 1.183 -> 1.117, 100k d = 132 0.589 -> 0.506; 1,216 queries 0.336 -> 0.255, 0.742 -> 0.642, 1.186 -> 1.230, 0.631 ->
+// 0.628. With pool 128 (layers' pool 32) wide rows cross earlier: 1,000 queries 1.005 -> 1.119 (d = 768), 0.793 -> 0.922
+// (d = 132), 2.078 -> 1.702 (d = 960), d = 96 0.503 -> 0.453; one line serves all.
 constexpr long long kTeamQueries = 608;
 constexpr long long kTeamLayered = 1216;
 struct TeamLayer {
@@ -72,7 +76,7 @@ cudaError_t coop_grid(K kernel, int threads, long long want, int* blocks) {
 
 // Rounds that commit a prefix of a window (indegree repair, reachability fix): blocks of 16 warps, so that a
 // full window has a warp per item in at most 128 blocks (a grid-wide barrier costs less the fewer blocks
-// arrive: the 1M merge's reachability rounds 13.5 ms with 512 blocks of 4 warps, 8.3 ms so, 8.9 ms with 64 blocks
+// arrive: the 1M merge's reachability rounds 11.4 ms with 512 blocks of 4 warps, 7.4 ms so, 7.9 ms with 64 blocks
 // of 32); the next round looks at four times the items the last one committed, within [256, most] (what
 // lies past the first conflict is planned for nothing). The window changes no result.
 constexpr int kRoundThreads = 512;
@@ -141,8 +145,8 @@ struct RefineBuffers {
     // scan scratch
     void* scan_tmp;
     size_t scan_bytes;
-    // largest candidate set and C_n of a pass and the three launch lists' sizes and largest
-    // sets (device, 8 ints), a pinned host slot to read them, and the launch lists (3 x cap)
+    // largest candidate set and C_n of a pass and the four launch lists' sizes and largest
+    // sets (device, 10 ints), a pinned host slot to read them, and the launch lists (4 x cap)
     int32_t* max_nc;
     int32_t* host_i32;
     long long class_count[5];   // out of refine_join: vertices per form (TC <= 64, <= 128, > 128; FP32 tile;
@@ -150,7 +154,7 @@ struct RefineBuffers {
     uint64_t* wk;               // worst key of every list (filled by refine_join for the Update launches)
     int sparse_nn;              // vertices with |C_n| <= sparse_nn (and |C| <= 128) join one warp each
                                 // (byte rows; 0: never)
-    bool fp8;                   // Xb holds E4M3 rows with per-vector scales (tcm.w) instead of BF16 rows
+    bool fp8;                   // Xb holds E4M3 rows with per-vector scales (tcm.w) instead of 16-bit ones
     int32_t* blist;
     long long blist_cap;
     // tensor-core filter inputs: BF16, FP16 (f16) or E4M3 (fp8) copy of the vectors, rows of dp >= dim

@@ -180,13 +180,15 @@ __device__ __forceinline__ T take_row_totals(const T (&v)[4], int r0, T mine, in
 // FP32 rows up to 128 coordinates: eight lanes per row, four rows per warp load, eight loads in
 // flight. Lane p adds the partials of chunks p, p + 16 and p + 8, p + 24 (the butterfly's offsets 16
 // and 8) by itself and the eight lanes' sums go through its last three levels four rows at a time. (One
-// row per warp load with the 32 x 32 partials re-added through 4 KB of shared memory, the earlier form,
-// took a third more instructions per row and halved the warps that fit on an SM.)
+// row per warp load, its 32 x 32 partials re-added through 4 KB of shared memory, takes a third more
+// instructions per row and halves the warps that fit on an SM.)
 // Wider rows: eight rows at a time, one lane per chunk, two chunks of every row (16 loads) in
 // flight; the eight rows' partials go through the butterfly together. The kernels are compiled for fewer
 // resident warps here (16 per SM in the cross query, 12 in k_search): the gather is bound by L2 and DRAM
 // latency, and loads in flight count for more than warps. Measured (d = 768 BF16, 120k): cross query
-// 13.9 ms with 8 loads and 20 warps, 12.5 ms so; k_search 1.51 and 0.89 ms.
+// 13.9 ms with 8 loads and 20 warps, 12.5 ms so; k_search 1.51 and 0.89 ms. On FP32 rows the eight rows' chunks
+// and sums are more than the registers hold: 48 to 112 bytes spill in the cross query (128 registers), up to 36 in
+// k_search (168).
 // Byte rows (d <= 128, d % 16 == 0): every partial sum of the canonical FP32 value is then an
 // integer below 128 * 255^2 < 2^24, so it is exact and the canonical value is the exact
 // integer result. Lanes take 16 bytes each (32 / lanes-per-row rows per warp load) and form

@@ -772,7 +772,8 @@ cudaError_t launch_fp8_coarse(const fgim_knng& g, const float4* tcm, const float
 // pairs instead of eight (80 registers) six CTAs fit on an SM instead of four: each is a chain of a few
 // memory round trips, and four kept the SM's schedulers 48 % busy. Join of 300k d = 96: 12.4 -> 10.0 ms,
 // 120k d = 768 BF16 12.4 -> 9.9, 50k d = 100 4.0 -> 3.3, 20k d = 32 0.78 -> 0.62. (Byte rows keep eight warps of
-// 64 registers per CTA, which fill an SM at four; nearly all of their sets are larger anyway.)
+// 64 registers per CTA, which fill an SM at four; nearly all of their sets are larger anyway.) The re-rank of FP32 rows
+// holds both rows' chunks of all its pairs: 260 to 280 bytes spill at 128 registers, 72 to 128 at 80.
 constexpr int kTCSmall = 64;
 __host__ __device__ __forceinline__ int tc_row(int i, int qs) { return ((i & 3) << qs) + (i >> 2); }
 __host__ __device__ __forceinline__ int tc_cand(int lane_row) { return 4 * (lane_row & 31) + (lane_row >> 5); }

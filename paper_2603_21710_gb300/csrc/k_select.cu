@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(128, sizeof(RT) == 1 ? 8 : SMALLD ? 5 : 4) k_p
 // lane. In the second 32 candidates, when more than 16 neighbours are kept already (few candidates are
 // occluded, and few are still needed), a lane holds a kept neighbour's row instead and the
 // candidates come one after another. Bound by the 32 dot products per lane and step and the shared
-// memory reads (8 of one address each; with both rows of a pair in shared memory, as before, 40
+// memory reads (8 of one address each; with both rows of a pair in shared memory it would be 40
 // bank cycles per step).
 constexpr int kBytesK = 64;
 constexpr int kManyKept = 16;

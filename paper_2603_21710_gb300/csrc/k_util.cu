@@ -1,5 +1,5 @@
 // Small building blocks: exclusive scans (two launches: the tiles' sums, then every block adds up the sums
-// before its own; five launches before, most of a small merge's launches), compaction by flags, fills, inverse norms.
+// before its own; the launches of its scans weigh in a small merge), compaction by flags, inverse norms.
 #include <algorithm>
 
 #include "fgim_launch.h"
