@@ -181,7 +181,7 @@ cudaError_t launch_bfs_parents(const int32_t* graph, int R, long long N, const i
 
 // min-label propagation over the undirected edges between unreached vertices, all passes in one
 // cooperative launch over the list of the unreached vertices, so that the host reads nothing between passes (14
-// launches of a 1M merge become 5, 1.9 -> 1.2 ms; a batch of 64 merges takes as long as with a launch per pass, 18.5 ms).
+// launches of a 1M merge become 5, 1.9 -> 1.2 ms; a batch of 64 merges takes as long as with a launch per pass, 9 ms).
 // st[0]: their number, st[1 + it % 3]: pass it changed a label.
 __global__ void __launch_bounds__(512) k_cc(const int32_t* __restrict__ graph, int R, long long N,
                                             const int32_t* __restrict__ visited, int32_t* label, int32_t* list,
