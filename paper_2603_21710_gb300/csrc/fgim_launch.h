@@ -59,6 +59,25 @@ cudaError_t launch_search_team(const void* X, bool bf16, const float* inv_norm, 
 // X8[i] = X[i] as a byte; *flag |= 1 unless every X[i] is an integer in [0, 255] (n_elems % 4 == 0)
 cudaError_t launch_narrow_u8(const float* X, long long n_elems, uint8_t* X8, int* flag, cudaStream_t s);
 
+// Lets launches of `kernel` ask for `smem` bytes of dynamic shared memory. The limit belongs to the kernel, not to the
+// launch, so a call must not set it to its own size: a call of another thread may stand between its setting and its launch,
+// and a smaller limit would make that launch fail. Every call that needs more than the default (48 KB) sets the
+// same value, the most a block can have; the others leave the limit alone.
+template <typename K>
+cudaError_t allow_smem(K kernel, size_t smem) {
+    constexpr size_t kByDefault = 47 * 1024;   // beside up to 1 KB of static shared memory
+    if (smem <= kByDefault) return cudaSuccess;
+    int dev = 0, most = 0;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess) return e;
+    most -= (int)a.sharedSizeBytes;
+    if (smem > (size_t)most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // the grid of a cooperative launch: `want` blocks, at most as many as are resident at once (the grid-wide
 // barriers wait for all of them)
 template <typename K>

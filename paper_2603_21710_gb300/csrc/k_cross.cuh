@@ -129,8 +129,7 @@ cudaError_t launch_cross_query_t(const ShardTable& t, const float* X, const uint
     if (e != cudaSuccess) return e;
 #define FGIM_LAUNCH_CQ2(MT, SD, RT, MS, PH)                                                                          \
     do {                                                                                                           \
-        e = cudaFuncSetAttribute(k_cross_query<MT, SD, RT, MS, PH>, cudaFuncAttributeMaxDynamicSharedMemorySize,       \
-                                 (int)smem);                                                                       \
+        e = allow_smem(k_cross_query<MT, SD, RT, MS, PH>, smem); \
         if (e != cudaSuccess) break;                                                                               \
         unsigned blocks = 0;                                                                                       \
         unsigned long long* next = nullptr;                                                                        \

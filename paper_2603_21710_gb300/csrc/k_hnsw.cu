@@ -115,7 +115,7 @@ cudaError_t launch_layer_knn(const float* Xl, const uint8_t* X8l, const float* i
     cudaError_t e = cudaSuccess;
 #define FGIM_LAUNCH_LK(MT, SD, RT)                                                                               \
     do {                                                                                                         \
-        e = cudaFuncSetAttribute(k_layer_knn<MT, SD, RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+        e = allow_smem(k_layer_knn<MT, SD, RT>, smem); \
         if (e != cudaSuccess) break;                                                                             \
         LaunchScope ls("k_layer_knn", s);                                                                        \
         k_layer_knn<MT, SD, RT><<<blocks, wpb * 32, smem, s>>>(Xl, reinterpret_cast<const RT*>(rows), inv, n, d, kk, \

@@ -340,7 +340,7 @@ cudaError_t launch_pg_edges(const int32_t* rows, long long b, int M, const int32
     }
     const int wpb = 4, W = M + (int)b;
     const size_t smem = (size_t)wpb * W * 8;
-    if ((e = cudaFuncSetAttribute(k_pg_rev_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    if ((e = allow_smem(k_pg_rev_merge, smem)) != cudaSuccess)
         return e;
     LaunchScope ls("k_pg_rev_merge", s);
     k_pg_rev_merge<<<(unsigned)cdivp(edges, wpb), wpb * 32, smem, s>>>(targets, off, cin, fill, rev, M, W, nbr, nd, cnt,

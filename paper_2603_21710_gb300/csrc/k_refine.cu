@@ -1883,8 +1883,7 @@ cudaError_t refine_join(const ShardTable& t, const float* X, const float* inv_no
             const int32_t* list = b.blist + (long long)q * b.blist_cap;
 #define FGIM_LAUNCH_TC4(MT, BY, LG, F8, SM)                                                                         \
     do {                                                                                                          \
-        e = cudaFuncSetAttribute(k_join_tc<MT, BY, LG, F8, SM>, cudaFuncAttributeMaxDynamicSharedMemorySize,          \
-                                 (int)smem);                                                                      \
+        e = allow_smem(k_join_tc<MT, BY, LG, F8, SM>, smem); \
         if (e != cudaSuccess) break;                                                                              \
         LaunchScope ls("k_join", s);                                                                              \
         k_join_tc<MT, BY, LG, F8, SM><<<(unsigned)count, (BY) ? 256 : kTCThreads, smem, s>>>(                           \
@@ -1930,7 +1929,7 @@ cudaError_t refine_join(const ShardTable& t, const float* X, const float* inv_no
             const unsigned grid = (unsigned)cdivll(count, kSparseWarps);
 #define FGIM_LAUNCH_SP(MT)                                                                                        \
     do {                                                                                                          \
-        e = cudaFuncSetAttribute(k_join_sparse<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);      \
+        e = allow_smem(k_join_sparse<MT>, smem); \
         if (e != cudaSuccess) break;                                                                              \
         LaunchScope ls("k_join_sparse", s);                                                                       \
         k_join_sparse<MT><<<grid, kSparseWarps * 32, smem, s>>>(                                                  \
@@ -1954,7 +1953,7 @@ cudaError_t refine_join(const ShardTable& t, const float* X, const float* inv_no
     const size_t smem = SL.bytes;
 #define FGIM_LAUNCH_JS(MT, ST)                                                                                    \
     do {                                                                                                          \
-        e = cudaFuncSetAttribute(k_join_staged<MT, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+        e = allow_smem(k_join_staged<MT, ST>, smem); \
         if (e != cudaSuccess) break;                                                                              \
         LaunchScope ls("k_join", s);                                                                              \
         k_join_staged<MT, ST><<<(unsigned)nv, kJThreads, smem, s>>>(t, X, inv_norm, g.k, g.ids, g.dist, b.cand,    \

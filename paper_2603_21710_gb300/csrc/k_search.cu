@@ -66,7 +66,7 @@ cudaError_t launch_search(const float* X, const uint8_t* X8, const float* inv_no
     cudaError_t e = cudaSuccess;
 #define FGIM_LAUNCH_S(MT, SD, RT, MS)                                                                                  \
     do {                                                                                                           \
-        e = cudaFuncSetAttribute(k_search<MT, SD, RT, MS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);   \
+        e = allow_smem(k_search<MT, SD, RT, MS>, smem); \
         if (e != cudaSuccess) break;                                                                               \
         unsigned blocks = 0;                                                                                       \
         unsigned long long* next = nullptr;                                                                        \

@@ -367,7 +367,7 @@ cudaError_t launch_prune(const float* X, const uint8_t* X8, const uint16_t* Xh, 
         const size_t smem = (size_t)prune_bytes_per_warp(k, R, d) * 4;
 #define FGIM_LAUNCH_PB(MT)                                                                                        \
     do {                                                                                                          \
-        e = cudaFuncSetAttribute(k_prune_bytes<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);      \
+        e = allow_smem(k_prune_bytes<MT>, smem); \
         if (e != cudaSuccess) break;                                                                              \
         LaunchScope ls("k_prune", s);                                                                             \
         k_prune_bytes<MT><<<(unsigned)((nrows + 3) / 4), 128, smem, s>>>(X8, inv_norm, N, nrows, d, k, g.ids, g.dist, \
@@ -386,8 +386,7 @@ cudaError_t launch_prune(const float* X, const uint8_t* X8, const uint16_t* Xh, 
     const unsigned blocks = (unsigned)(split ? nrows : (nrows + 3) / 4);
 #define FGIM_LAUNCH_P2(MT, SD, RT, W, ST, ROWS)                                                                   \
     do {                                                                                                          \
-        e = cudaFuncSetAttribute(k_prune<MT, SD, RT, W, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,         \
-                                 (int)smem);                                                                      \
+        e = allow_smem(k_prune<MT, SD, RT, W, ST>, smem); \
         if (e != cudaSuccess) break;                                                                              \
         LaunchScope ls("k_prune", s);                                                                             \
         k_prune<MT, SD, RT, W, ST><<<blocks, 128, smem, s>>>(ROWS, inv_norm, N, nrows, d, k, g.ids, g.dist, T, R, \

@@ -347,8 +347,7 @@ cudaError_t launch_search_team(const void* X, bool bf16, const float* inv_norm, 
     cudaError_t e = cudaSuccess;
 #define FGIM_LAUNCH_T(MT, SD, RT, MS)                                                                              \
     do {                                                                                                           \
-        e = cudaFuncSetAttribute(k_search_team<MT, SD, RT, MS>, cudaFuncAttributeMaxDynamicSharedMemorySize,       \
-                                 (int)smem);                                                                       \
+        e = allow_smem(k_search_team<MT, SD, RT, MS>, smem); \
         if (e != cudaSuccess) break;                                                                               \
         LaunchScope ls("k_search", s);                                                                             \
         k_search_team<MT, SD, RT, MS><<<(unsigned)nq, threads, smem, s>>>(                                    \
